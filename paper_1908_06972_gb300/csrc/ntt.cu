@@ -14,8 +14,8 @@
 // each thread keeps 16 points in registers and applies up to 4 stages per round
 // (Harvey butterflies with an estimated Shoup quotient: forward values in [0, 8q), uncorrected
 // for primes below 2^57 in the N = 2^16 kernels; inverse values in [0, 4q)), and
-// rounds exchange through shared memory.  N <= 2^14: one pass, one CTA per limb.
-// N = 2^15, 2^16: two passes (8 + 7 or 8 + 8 stages).
+// rounds exchange through shared memory.  N = 2^12..2^16: two passes (columns of 2^(logn-8) points,
+// then rows of 256).  N <= 2^11: one pass, one CTA per limb.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -146,33 +146,35 @@ __device__ __forceinline__ int pass_limb(int flags) {
 // two phases in the opposite order.  Lane = sub-transform, so every shared and remote
 // access is a stride-33 (odd) walk: conflict-free.  One HBM read and one write per limb.
 //
-// One round = four stages on 16 registers: register e holds element (e << W0) | wpart of
-// the current 256-point sub-transform; DIMHI = 0 for column stages (s = 7 - p), 8 for row
-// stages (s = 15 - p, r = the row being transformed).
-// LM (the row round W0 = 0 of stages 12..15, thread = row r, lane w): the twiddles come from
-// the lane-major copy of that round's twiddles, lm = its entries for (prime, row r, lane w):
-// slot (2^k - 1 + j) of stage 12 + k at lm[16 (2^k - 1 + j)], loaded under the L2 policy pol.
-// RT (the row round W0 = 4 of stages 8..11, thread = row r): the row's 15 twiddles of those
-// stages were copied to shared memory, stage 8 + k entry j at rt[2^k - 1 + j].
-template <bool INV, int W0, int DIMHI, bool LAZY = false, bool UNSCALED = false, bool LM = false, bool RT = false>
-__device__ __forceinline__ void ntt16_round(u64 (&x)[16], int wpart, int r, const ulonglong2* __restrict__ tw,
-                                            u64 q, u64 q2, ulonglong2 NI, ulonglong2 NI1,
-                                            const ulonglong2* __restrict__ lm = nullptr,
-                                            const ulonglong2* rt = nullptr, u64 pol = 0) {
-    static_assert(!LM || (W0 == 0 && DIMHI == 8), "lane-major twiddles serve the row round of stages 12..15");
-    static_assert(!RT || (W0 == 4 && DIMHI == 8), "staged row twiddles serve the row round of stages 8..11");
+// One round = up to four stages on 16 registers: register e holds element (e << W0) | wpart of
+// the current sub-transform of a pass; bit p of an element is paired by stage TOP - p (columns of
+// 2^SA points: TOP = SA - 1; rows of 256 points after them: TOP = SA + 7, r = the row).  NB: the
+// lowest NB of the register bits are paired (4 but for the second round of short columns).
+// LM (the row round W0 = 0, thread = row r, lane w): the twiddles of the last four stages come
+// from their lane-major copy, lm = its entries for (prime, row r, lane w): slot (2^k - 1 + j) of
+// the k-th of these stages at lm[16 (2^k - 1 + j)], loaded under the L2 policy pol.
+// RT (the row round W0 = 4, thread = row r): the row's 15 twiddles of its first four stages
+// were copied to shared memory, the k-th stage's entry j at rt[2^k - 1 + j].
+template <bool INV, int W0, int TOP, int NB = 4, bool LAZY = false, bool UNSCALED = false, bool LM = false,
+          bool RT = false>
+__device__ __forceinline__ void ntt_round(u64 (&x)[16], int wpart, int r, const ulonglong2* __restrict__ tw, u64 q,
+                                          u64 q2, ulonglong2 NI, ulonglong2 NI1,
+                                          const ulonglong2* __restrict__ lm = nullptr,
+                                          const ulonglong2* rt = nullptr, u64 pol = 0) {
+    static_assert(!LM || W0 == 0, "lane-major twiddles serve the row round of the last four stages");
+    static_assert(!RT || W0 == 4, "staged row twiddles serve the first row round");
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const int lb = INV ? k : 3 - k;
+    for (int k = 0; k < NB; k++) {
+        const int lb = INV ? k : NB - 1 - k;
         const int p = W0 + lb;
-        const int s = DIMHI + 7 - p;
+        const int s = TOP - p;
 #pragma unroll
         for (int e = 0; e < 16; e++) {
             if (e & (1 << lb)) continue;
             const int elem = (e << W0) | wpart;
             const int idx = (1 << s) + (r << (7 - p)) + (elem >> (p + 1));
-            const ulonglong2 W = LM   ? ldg_pol(&lm[16 * ((1 << (s - 12)) - 1 + (e >> (p + 1)))], pol)
-                                 : RT ? rt[(1 << (s - 8)) - 1 + (elem >> (p + 1))]
+            const ulonglong2 W = LM   ? ldg_pol(&lm[16 * ((1 << (3 - p)) - 1 + (e >> (p + 1)))], pol)
+                                 : RT ? rt[(1 << (7 - p)) - 1 + (elem >> (p + 1))]
                                       : __ldg(&tw[idx]);
             if (!INV) {
                 ct_bfly<LAZY>(x[e], x[e | (1 << lb)], W, q, q2);
@@ -218,13 +220,13 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
         const int col = 32 * c + lane;
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << 4) | w) * 256 + col];
-        ntt16_round<false, 4, 0>(x, w, 0, tw, q, q2, NI, NI1);
+        ntt_round<false, 4, 7>(x, w, 0, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((e << 4) | w) * ST + lane] = x[e];
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + lane];
-        ntt16_round<false, 0, 0>(x, w << 4, 0, tw, q, q2, NI, NI1);
+        ntt_round<false, 0, 7>(x, w << 4, 0, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + lane] = x[e];
         cluster.sync();
@@ -237,13 +239,13 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
             x[e] = rem[r * ST + (cx & 31)];
         }
         cluster.sync();
-        ntt16_round<false, 4, 8>(x, w, r, tw, q, q2, NI, NI1);
+        ntt_round<false, 4, 15>(x, w, r, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((e << 4) | w) * ST + lane] = x[e];
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + lane];
-        ntt16_round<false, 0, 8>(x, w << 4, r, tw, q, q2, NI, NI1);
+        ntt_round<false, 0, 15>(x, w << 4, r, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + lane] = canon8(x[e], q, q2);
         __syncthreads();
@@ -265,13 +267,13 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + lane];
-        ntt16_round<true, 0, 8>(x, w << 4, r, tw, q, q2, NI, NI1);
+        ntt_round<true, 0, 15>(x, w << 4, r, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + lane] = x[e];
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = sm[((e << 4) | w) * ST + lane];
-        ntt16_round<true, 4, 8>(x, w, r, tw, q, q2, NI, NI1);
+        ntt_round<true, 4, 15>(x, w, r, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((e << 4) | w) * ST + lane] = x[e];
         cluster.sync();
@@ -284,40 +286,57 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
             x[e] = rem[col * ST + (row & 31)];
         }
         cluster.sync();
-        ntt16_round<true, 0, 0>(x, w << 4, 0, tw, q, q2, NI, NI1);
+        ntt_round<true, 0, 7>(x, w << 4, 0, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + lane] = x[e];
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = sm[((e << 4) | w) * ST + lane];
-        ntt16_round<true, 4, 0>(x, w, 0, tw, q, q2, NI, NI1);
+        ntt_round<true, 4, 7>(x, w, 0, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++) dst[(size_t)((e << 4) | w) * 256 + col] = canon4(x[e], q, q2);
     }
 }
 
-// ---- N = 2^16 in two passes of 8 stages, global memory touched from registers ----------------
-// Pass A (stages 0..7): 256-point column transforms at stride T = 2^LOGT; a CTA takes 16
-// adjacent columns, lane bits 0..3 = column, so every global access of a warp reads or
-// writes two 128-byte runs.  Pass B (stages 8..15): 16 contiguous 256-point rows per CTA,
-// lane bits 0..3 = point.  Each pass does 2 rounds of 4 stages with one shared-memory
-// exchange (odd strides 17 / 273: conflict-free); pass B stages its final store (forward)
-// or first load (inverse) through shared memory to keep the global side coalesced.
+// ---- N = 2^12..2^16 in two passes, global memory touched from registers ----------------------
+// The limb is viewed as 2^SA rows of 256 words (SA = logn - 8, 4..8).  Pass A (stages 0..SA-1):
+// the 256 columns of 2^SA points at stride 256; a CTA takes C adjacent columns, lanes on adjacent
+// columns, so every global access of a warp reads or writes whole 128-byte runs.  Pass B (stages
+// SA..logn-1): contiguous rows of 256 points, 16 lanes on adjacent points of a row, R rows per CTA.
+// Each pass keeps 16 points per thread in registers and does rounds of up to four stages with
+// one shared-memory exchange between them (rows: odd strides 17 / 273, conflict-free; columns: a
+// warp's lanes are adjacent columns).  Pass B stages its final store (forward) or first load
+// (inverse) through shared memory to keep the global side coalesced.
+// Bound: the integer multiply pipe for launches of many limbs, the latency of one thread's 16 points
+// for launches of a few.  Against the generic kernels below (one CTA per limb to N = 2^14, staged
+// passes at 2^15; GB300): one HMUL + rescale at N = 2^13, level 3: 188 -> 100 us (its three inverse
+// launches took 58 us each on 1 to 3 SMs); 31 HMULs + rescales at N = 2^15, levels 12..18: 6.15 -> 3.70 ms.
+// Why these shapes: at N = 2^16 and 2^15 CTAs of 256 threads (16 columns, 32 columns; 16 rows); the
+// smaller rings meet launches of a few limbs, so their CTAs are small (64 or 128 threads) to
+// spread a limb over the SMs.
 constexpr int kRowStride = 273;  // 256 + 16 padding + 1
 constexpr u64 kLazyBound = 1ull << 57;  // forward butterflies skip the correction below this prime
+__host__ __device__ constexpr int cols_per_cta(int SA) { return SA == 8 ? 16 : 32; }
+__host__ __device__ constexpr int rows_per_cta(int SA) { return SA >= 7 ? 16 : SA == 6 ? 8 : 4; }
+__host__ __device__ constexpr int col_threads(int SA) { return cols_per_cta(SA) << (SA - 4); }
+__host__ __device__ constexpr int row_threads(int SA) { return rows_per_cta(SA) * 16; }
 
+// MT: resident threads per SM the registers are bounded for (768: 80 registers, 1024: 64).
 // UNSCALED (inverse): the last stage is a plain Gentleman-Sande butterfly (no N^-1) and the
 // output stays in [0, 4q): N times the inverse transform, for a consumer that scales anyway.
-template <bool INV, int LOGT, int MINB, bool UNSCALED = false>
-__global__ void __launch_bounds__(256, MINB) k_ntt8_strided(DevTables t, PolySet in, PolySet out, int flags) {
-    __shared__ u64 sm[256 * 17];
+template <bool INV, int SA, int MT, bool UNSCALED = false>
+__global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
+    k_ntt_cols(DevTables t, PolySet in, PolySet out, int flags) {
+    constexpr int C = cols_per_cta(SA), LO = SA - 4;     // LO: bits of the second round
+    constexpr int ST = C == 16 ? 17 : C;
+    __shared__ u64 sm[SA > 4 ? (1 << SA) * ST : 1];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
-    const int logn = t.logn;
+    const int logn = SA + 8;
     const int pi = prime_of(Ro, limb);
-    const int cc = threadIdx.x & 15, w = threadIdx.x >> 4;
-    const int col = blockIdx.x * 16 + cc;
+    const int cc = threadIdx.x % C, w = threadIdx.x / C;
+    const int col = blockIdx.x * C + cc;
     const u64* src = in.p[poly].ptr + ((size_t)limb << logn) + col;
     u64* dst = Ro.ptr + ((size_t)limb << logn) + col;
     const u64 q = __ldg(&t.primes[pi].q);
@@ -329,31 +348,35 @@ __global__ void __launch_bounds__(256, MINB) k_ntt8_strided(DevTables t, PolySet
     if (!INV) {
         const bool lazy = q < kLazyBound;  // uniform over the CTA (one limb)
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << 4) | w) << LOGT];
-        if (lazy) ntt16_round<false, 4, 0, true>(x, w, 0, tw, q, q2, NI, NI1);
-        else ntt16_round<false, 4, 0>(x, w, 0, tw, q, q2, NI, NI1);
+        for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << LO) | w) << 8];
+        if (lazy) ntt_round<false, LO, SA - 1, 4, true>(x, w, 0, tw, q, q2, NI, NI1);
+        else ntt_round<false, LO, SA - 1>(x, w, 0, tw, q, q2, NI, NI1);
+        if constexpr (SA > 4) {
 #pragma unroll
-        for (int e = 0; e < 16; e++) sm[((e << 4) | w) * 17 + cc] = x[e];
-        __syncthreads();
+            for (int e = 0; e < 16; e++) sm[((e << LO) | w) * ST + cc] = x[e];
+            __syncthreads();
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * 17 + cc];
-        if (lazy) ntt16_round<false, 0, 0, true>(x, w << 4, 0, tw, q, q2, NI, NI1);
-        else ntt16_round<false, 0, 0>(x, w << 4, 0, tw, q, q2, NI, NI1);
+            for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + cc];
+            if (lazy) ntt_round<false, 0, SA - 1, LO, true>(x, w << 4, 0, tw, q, q2, NI, NI1);
+            else ntt_round<false, 0, SA - 1, LO>(x, w << 4, 0, tw, q, q2, NI, NI1);
+        }
 #pragma unroll
-        for (int e = 0; e < 16; e++) dst[(size_t)((w << 4) | e) << LOGT] = x[e];
+        for (int e = 0; e < 16; e++) dst[(size_t)((w << 4) | e) << 8] = x[e];
     } else {
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = src[(size_t)((w << 4) | e) << LOGT];
-        ntt16_round<true, 0, 0>(x, w << 4, 0, tw, q, q2, NI, NI1);
+        for (int e = 0; e < 16; e++) x[e] = src[(size_t)((w << 4) | e) << 8];
+        if constexpr (SA > 4) {
+            ntt_round<true, 0, SA - 1, LO>(x, w << 4, 0, tw, q, q2, NI, NI1);
 #pragma unroll
-        for (int e = 0; e < 16; e++) sm[((w << 4) | e) * 17 + cc] = x[e];
-        __syncthreads();
+            for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + cc] = x[e];
+            __syncthreads();
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = sm[((e << 4) | w) * 17 + cc];
-        ntt16_round<true, 4, 0, false, UNSCALED>(x, w, 0, tw, q, q2, NI, NI1);
+            for (int e = 0; e < 16; e++) x[e] = sm[((e << LO) | w) * ST + cc];
+        }
+        ntt_round<true, LO, SA - 1, 4, false, UNSCALED>(x, w, 0, tw, q, q2, NI, NI1);
 #pragma unroll
         for (int e = 0; e < 16; e++)
-            dst[(size_t)((e << 4) | w) << LOGT] = (flags & kPassFinal) && !UNSCALED ? canon4(x[e], q, q2) : x[e];
+            dst[(size_t)((e << LO) | w) << 8] = (flags & kPassFinal) && !UNSCALED ? canon4(x[e], q, q2) : x[e];
     }
 }
 
@@ -369,60 +392,62 @@ __device__ __forceinline__ u64 reduce_below66(u64 x, u64 q, u32 r, u32 sh) {
     return v >= q ? v - q : v;
 }
 
-// ---- lane-major copy of the twiddles of stages 12..15 ---------------------------------------
-// In the round of stages 12..15 of a row pass, thread (row u, lane w) uses the 15 twiddles
-// 2^(12+k) + u 2^(4+k) + w 2^k + j (k < 4, j < 2^k): row- and lane-specific, each read once.
+// ---- lane-major copy of the twiddles of the last four stages ----------------------------------
+// In the second round of a row pass, thread (row u, lane w) uses the 15 twiddles
+// 2^(SA+4+k) + u 2^(4+k) + w 2^k + j (k < 4, j < 2^k): row- and lane-specific, each read once.
 // Read from the natural table, one warp load touches 32 cache lines for 16 bytes each.  The
 // lane-major copy holds, per prime and row, [15 slots][16 lanes] (slot 2^k - 1 + j), so the 16
 // lanes of a row read 256 contiguous bytes per load.
 constexpr int kRowTwSlots = 15;
-// The 16 rows' twiddles of stages 8..11 (row u: entry 2^(8+k) + u 2^k + j, k < 4, j < 2^k) into
-// rt[16][15]: one 16-byte load and store for 240 of the 256 threads, made visible by the caller's
-// next barrier.
+// The R rows' twiddles of the first four row stages (row u: entry 2^(SA+k) + u 2^k + j, k < 4,
+// j < 2^k) into rt[R][15]: one 16-byte load and store for 15 of every 16 threads, made visible by
+// the caller's next barrier.
+template <int SA>
 __device__ __forceinline__ void stage_row_round1(const ulonglong2* __restrict__ tw, int u0, ulonglong2* rt, u64 pol) {
     const int t = threadIdx.x;
-    if (t < 16 * 15) {
+    if (t < rows_per_cta(SA) * 15) {
         const int cc = t / 15, e = t % 15;
         const int k = e >= 7 ? 3 : e >= 3 ? 2 : e >= 1 ? 1 : 0;
         const int j = e + 1 - (1 << k);
-        rt[t] = ldg_pol(&tw[(1 << (8 + k)) + ((u0 + cc) << k) + j], pol);
+        rt[t] = ldg_pol(&tw[(1 << (SA + k)) + ((u0 + cc) << k) + j], pol);
     }
 }
+template <int SA>
 __device__ __forceinline__ const ulonglong2* lm_base(const ulonglong2* rows, int pi, int u, int w) {
-    return rows + ((size_t)pi * 256 + u) * (kRowTwSlots * 16) + w;
+    return rows + (((size_t)pi << SA) + u) * (kRowTwSlots * 16) + w;
 }
 
-// Forward stages 8..15 of the 16 rows of this CTA (limb `limb` of prime pi, rows read from
+// Forward stages SA..SA+7 of the rows of this CTA (limb `limb` of prime pi, rows read from
 // src): canonical results are left in sm, row c2 point m at c2 * kRowStride + m + (m >> 4),
 // after a barrier.
-template <bool LM = false>
-__device__ __forceinline__ void contig_fwd_rows(const DevTables& t, const u64* __restrict__ src, int pi, u64* sm) {
-    const int logn = t.logn;
+template <int SA>
+__device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restrict__ src, int pi, u64* sm) {
+    constexpr int R = rows_per_cta(SA), TOP = SA + 7;
     const int w = threadIdx.x & 15, cc = threadIdx.x >> 4;
-    const int u = blockIdx.x * 16 + cc;
+    const int u = blockIdx.x * R + cc;
     const u64 q = __ldg(&t.primes[pi].q);
     const u64 q2 = 2 * q;
-    const ulonglong2* tw = t.fwd + ((size_t)pi << logn);
+    const ulonglong2* tw = t.fwd + ((size_t)pi << (SA + 8));
     const ulonglong2 NI = make_ulonglong2(0, 0);
-    const ulonglong2* lm = LM ? lm_base(t.fwd_rows, pi, u, w) : nullptr;
+    const ulonglong2* lm = lm_base<SA>(t.fwd_rows, pi, u, w);
     const u64 pol = tw_policy(t.ntt_order & 2);
-    __shared__ ulonglong2 rt[16 * 15];  // LM: twiddles of stages 8..11 of the 16 rows
+    __shared__ ulonglong2 rt[R * 15];  // twiddles of the first four row stages
     u64* my = sm + cc * kRowStride;
     u64 x[16];
     const bool lazy = q < kLazyBound;  // uniform over the CTA (one limb)
-    if (LM) stage_row_round1(tw, blockIdx.x * 16, rt, pol);
+    stage_row_round1<SA>(tw, blockIdx.x * R, rt, pol);
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = src[((size_t)u << 8) | (e << 4) | w];
-    if (LM) __syncthreads();
-    if (lazy) ntt16_round<false, 4, 8, true, false, false, LM>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
-    else ntt16_round<false, 4, 8, false, false, false, LM>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
+    __syncthreads();
+    if (lazy) ntt_round<false, 4, TOP, 4, true, false, false, true>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
+    else ntt_round<false, 4, TOP, 4, false, false, false, true>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
 #pragma unroll
     for (int e = 0; e < 16; e++) my[e * 17 + w] = x[e];  // point e*16 + w
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[w * 17 + e];  // point w*16 + e
     if (lazy) {
-        ntt16_round<false, 0, 8, true, false, LM>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
+        ntt_round<false, 0, TOP, 4, true, false, true>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
         const u32 ps = __ldg(&t.primes[pi].s);
         if (ps >= 24) {
             const u32 r = (u32)(__ldg(&t.primes[pi].mu) >> 32);
@@ -437,75 +462,77 @@ __device__ __forceinline__ void contig_fwd_rows(const DevTables& t, const u64* _
             }
         }
     } else {
-        ntt16_round<false, 0, 8, false, false, LM>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
+        ntt_round<false, 0, TOP, 4, false, false, true>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
 #pragma unroll
         for (int e = 0; e < 16; e++) my[w * 17 + e] = canon8(x[e], q, q2);
     }
     __syncthreads();
 }
 
-template <bool INV, int MINB, bool LM = false>
-__global__ void __launch_bounds__(256, MINB) k_ntt8_contig(DevTables t, PolySet in, PolySet out, int flags) {
-    __shared__ u64 sm[16 * kRowStride];
+template <bool INV, int SA, int MT>
+__global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
+    k_ntt_rows(DevTables t, PolySet in, PolySet out, int flags) {
+    constexpr int R = rows_per_cta(SA), TOP = SA + 7, logn = SA + 8;
+    __shared__ u64 sm[R * kRowStride];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
-    const int logn = t.logn;
     const int pi = prime_of(Ro, limb);
     const u64* src = in.p[poly].ptr + ((size_t)limb << logn);
     u64* dst = Ro.ptr + ((size_t)limb << logn);
     if (!INV) {
-        contig_fwd_rows<LM>(t, src, pi, sm);
+        fwd_rows<SA>(t, src, pi, sm);
 #pragma unroll
         for (int k = 0; k < 16; k++) {
-            const int f = threadIdx.x + 256 * k;
+            const int f = threadIdx.x + R * 16 * k;
             const int c2 = f >> 8, m = f & 255;
-            dst[((size_t)(blockIdx.x * 16 + c2) << 8) | m] = sm[c2 * kRowStride + m + (m >> 4)];
+            dst[((size_t)(blockIdx.x * R + c2) << 8) | m] = sm[c2 * kRowStride + m + (m >> 4)];
         }
         return;
     }
     const int w = threadIdx.x & 15, cc = threadIdx.x >> 4;
-    const int u = blockIdx.x * 16 + cc;
+    const int u = blockIdx.x * R + cc;
     const u64 q = __ldg(&t.primes[pi].q);
     const u64 q2 = 2 * q;
     const ulonglong2* tw = t.inv + ((size_t)pi << logn);
     const ulonglong2 NI = __ldg(&t.ninv[pi]);
     const ulonglong2 NI1 = __ldg(&t.inv1ninv[pi]);
-    const ulonglong2* lm = LM ? lm_base(t.inv_rows, pi, u, w) : nullptr;
+    const ulonglong2* lm = lm_base<SA>(t.inv_rows, pi, u, w);
     const u64 pol = tw_policy(t.ntt_order & 2);
     u64* my = sm + cc * kRowStride;
     u64 x[16];
 #pragma unroll
     for (int k = 0; k < 16; k++) {
-        const int f = threadIdx.x + 256 * k;
+        const int f = threadIdx.x + R * 16 * k;
         const int c2 = f >> 8, m = f & 255;
-        sm[c2 * kRowStride + m + (m >> 4)] = src[((size_t)(blockIdx.x * 16 + c2) << 8) | m];
+        sm[c2 * kRowStride + m + (m >> 4)] = src[((size_t)(blockIdx.x * R + c2) << 8) | m];
     }
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[w * 17 + e];  // point w*16 + e
-    ntt16_round<true, 0, 8, false, false, LM>(x, w << 4, u, tw, q, q2, NI, NI1, lm, nullptr, pol);
+    ntt_round<true, 0, TOP, 4, false, false, true>(x, w << 4, u, tw, q, q2, NI, NI1, lm, nullptr, pol);
 #pragma unroll
     for (int e = 0; e < 16; e++) my[w * 17 + e] = x[e];
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[e * 17 + w];  // point e*16 + w
-    ntt16_round<true, 4, 8>(x, w, u, tw, q, q2, NI, NI1);
+    ntt_round<true, 4, TOP>(x, w, u, tw, q, q2, NI, NI1);
 #pragma unroll
     for (int e = 0; e < 16; e++)
         dst[((size_t)u << 8) | (e << 4) | w] = (flags & kPassFinal) ? canon4(x[e], q, q2) : x[e];
 }
 
-// Forward stages 8..15 fused with the ModDown epilogue: for the canonical transform value v,
+// Forward row stages fused with the ModDown epilogue: for the canonical transform value v,
 // out = (x + c - v) s mod q (+ acc when the polynomial has one), with per-limb constants
-// {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of stages 0..7.
-template <int MINB, bool LM = false>
-__global__ void __launch_bounds__(256, MINB) k_ntt8_contig_epi(DevTables t, PolySet in, NttEpi e, int flags) {
-    __shared__ u64 sm[16 * kRowStride];
+// {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of the column pass.
+template <int SA, int MT>
+__global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
+    k_ntt_rows_epi(DevTables t, PolySet in, NttEpi e, int flags) {
+    constexpr int R = rows_per_cta(SA), NT = R * 16, logn = SA + 8;
+    __shared__ u64 sm[R * kRowStride];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ri = in.p[poly];
     if (limb >= Ri.nlimbs) return;
-    const int logn = t.logn;
     const int pi = prime_of(Ri, limb);
     const size_t base = (size_t)limb << logn;
     const u64* __restrict__ xs = e.x.p[poly].ptr + base;
@@ -513,33 +540,34 @@ __global__ void __launch_bounds__(256, MINB) k_ntt8_contig_epi(DevTables t, Poly
     u64* __restrict__ os = e.out.p[poly].ptr + base;
     if (flags & kPassPrefetch) {
         // ask L2 for this CTA's tile of the epilogue operands (one 128-byte line per thread and
-        // operand: 16 rows x 256 words) so that their DRAM reads overlap the transform
+        // operand: R rows x 256 words) so that their DRAM reads overlap the transform
         const int f = threadIdx.x * 16;
-        const size_t j = ((size_t)(blockIdx.x * 16 + (f >> 8)) << 8) | (f & 255);
+        const size_t j = ((size_t)(blockIdx.x * R + (f >> 8)) << 8) | (f & 255);
         asm volatile("prefetch.global.L2 [%0];" ::"l"(xs + j));
         if (as) asm volatile("prefetch.global.L2 [%0];" ::"l"(as + base + j));
     }
-    contig_fwd_rows<LM>(t, Ri.ptr + base, pi, sm);
+    fwd_rows<SA>(t, Ri.ptr + base, pi, sm);
     const u64 q = __ldg(&t.primes[pi].q);
     const u64 c = __ldg(&e.consts[3 * limb]), s = __ldg(&e.consts[3 * limb + 1]), sp = __ldg(&e.consts[3 * limb + 2]);
-    // each thread: two adjacent points (16-byte loads and stores) of rows r0, r0 + 2, ..., r0 + 14;
-    // the operands of four rows are loaded before any is used, so that more bytes are in flight
-    // (the transform's registers are free by now).  An even point m and m + 1 share their
-    // 16-point group, so their transform values are adjacent in shared memory.
-    const int m = 2 * (threadIdx.x & 127), r0 = threadIdx.x >> 7;
+    // each thread: two adjacent points (16-byte loads and stores) of eight rows or row parts; the
+    // operands of four are loaded before any is used, so that more bytes are in flight (the
+    // transform's registers are free by now).  An even point m and m + 1 share their 16-point
+    // group, so their transform values are adjacent in shared memory.
 #pragma unroll
     for (int h = 0; h < 2; h++) {
         ulonglong2 xv[4], av[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-            const size_t j = ((size_t)(blockIdx.x * 16 + r0 + 2 * (4 * h + i)) << 8) | m;
+            const int f = 2 * (threadIdx.x + NT * (4 * h + i));
+            const size_t j = ((size_t)(blockIdx.x * R) << 8) + f;
             xv[i] = *reinterpret_cast<const ulonglong2*>(xs + j);
             if (as) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
         }
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-            const int c2 = r0 + 2 * (4 * h + i);
-            const size_t j = ((size_t)(blockIdx.x * 16 + c2) << 8) | m;
+            const int f = 2 * (threadIdx.x + NT * (4 * h + i));
+            const int c2 = f >> 8, m = f & 255;
+            const size_t j = ((size_t)(blockIdx.x * R) << 8) + f;
             const u64* v = sm + c2 * kRowStride + m + (m >> 4);
             ulonglong2 r;
             r.x = mul_shoup(submod(addmod(xv[i].x, c, q), v[0], q), s, sp, q);
@@ -553,102 +581,89 @@ __global__ void __launch_bounds__(256, MINB) k_ntt8_contig_epi(DevTables t, Poly
     }
 }
 
-template <int MINB>
+// Shared-memory carveout of the kernels bounded for 1024 threads per SM (four CTAs of 35 KB): one
+// that fits them, the rest L1.
+template <int SA, int MT>
 static void prepare_twopass(void) {
-    if (MINB == 4 && first_on_device((const void*)&k_ntt8_contig_epi<MINB, true>)) {
-        // four CTAs of 35 KB shared memory: a carveout that fits them, the rest L1
+    if (MT == 1024 && first_on_device((const void*)&k_ntt_rows_epi<SA, MT>)) {
         const int co = 64;
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_strided<false, 8, MINB>, cudaFuncAttributePreferredSharedMemoryCarveout, co));
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_strided<true, 8, MINB>, cudaFuncAttributePreferredSharedMemoryCarveout, co));
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_strided<true, 8, MINB, true>,
-                                      cudaFuncAttributePreferredSharedMemoryCarveout, co));
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_contig<false, MINB, true>, cudaFuncAttributePreferredSharedMemoryCarveout, co));
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_contig<true, MINB, true>, cudaFuncAttributePreferredSharedMemoryCarveout, co));
-        PFT_CUDA(cudaFuncSetAttribute(k_ntt8_contig_epi<MINB, true>, cudaFuncAttributePreferredSharedMemoryCarveout, co));
+        auto set = [&](auto k) { PFT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, co)); };
+        set(k_ntt_cols<false, SA, MT>);
+        set(k_ntt_cols<true, SA, MT>);
+        set(k_ntt_cols<true, SA, MT, true>);
+        set(k_ntt_rows<false, SA, MT>);
+        set(k_ntt_rows<true, SA, MT>);
+        set(k_ntt_rows_epi<SA, MT>);
     }
-}
-
-template <bool INV, int MINB, bool LM>
-static void launch_contig(const DevTables& t, const PolySet& in, const PolySet& out, int flags, cudaStream_t st) {
-    dim3 grid(16, (unsigned)out.max_limbs, (unsigned)out.count);
-    k_ntt8_contig<INV, MINB, LM><<<grid, 256, 0, st>>>(t, in, out, flags);
 }
 // flags of the second pass of a transform over the same data
 static int second_pass(const DevTables& t, int flags) { return flags | ((t.ntt_order & 1) ? kPassReverse : 0); }
 
-template <int MINB, bool LM>
-static void launch_ntt16_twopass_v(const DevTables& t, const PolySet& in, const PolySet& out, bool inverse,
-                                   cudaStream_t st) {
-    prepare_twopass<MINB>();
-    dim3 grid(16, (unsigned)out.max_limbs, (unsigned)out.count);  // 256 sub-transforms / 16 per CTA
-    const double work = set_limbs(out) * (double)(t.n / 2) * 8;
-    if (!inverse) {
-        {
-            PFT_PROF("ntt.fwd.strided", st, work);
-            k_ntt8_strided<false, 8, MINB><<<grid, 256, 0, st>>>(t, in, out, 0);
-        }
+template <int SA, int MT>
+struct TwoPass {
+    static dim3 col_grid(const PolySet& s) {
+        return dim3(256 / cols_per_cta(SA), (unsigned)s.max_limbs, (unsigned)s.count);
+    }
+    static dim3 row_grid(const PolySet& s) {
+        return dim3((1 << SA) / rows_per_cta(SA), (unsigned)s.max_limbs, (unsigned)s.count);
+    }
+    static double work(const DevTables& t, const PolySet& s, int stages) {
+        return set_limbs(s) * (double)(t.n / 2) * stages;
+    }
+    static void cols_fwd(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
+        prepare_twopass<SA, MT>();
+        PFT_PROF("ntt.fwd.strided", st, work(t, out, SA));
+        k_ntt_cols<false, SA, MT><<<col_grid(out), col_threads(SA), 0, st>>>(t, in, out, 0);
         PFT_LAUNCH_CHECK("ntt pass A");
-        {
-            PFT_PROF("ntt.fwd.contig", st, work);
-            launch_contig<false, MINB, LM>(t, out, out, second_pass(t, kPassFinal), st);
-        }
+    }
+    static void forward(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
+        cols_fwd(t, in, out, st);
+        PFT_PROF("ntt.fwd.contig", st, work(t, out, 8));
+        k_ntt_rows<false, SA, MT><<<row_grid(out), row_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("ntt pass B");
-    } else {
+    }
+    static void forward_epi(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
+        cols_fwd(t, io, io, st);
+        // named apart from the plain transform launches: it also moves the epilogue's operands
+        PFT_PROF("epi.ntt_moddown", st, work(t, io, 8));
+        k_ntt_rows_epi<SA, MT><<<row_grid(io), row_threads(SA), 0, st>>>(
+            t, io, e, second_pass(t, (t.ntt_order & 4) ? kPassPrefetch : 0));
+        PFT_LAUNCH_CHECK("ntt pass B + ModDown epilogue");
+    }
+    static void inverse(const DevTables& t, const PolySet& in, const PolySet& out, bool unscaled, cudaStream_t st) {
+        prepare_twopass<SA, MT>();
         {
-            PFT_PROF("ntt.inv.contig", st, work);
-            launch_contig<true, MINB, LM>(t, in, out, 0, st);
+            PFT_PROF("ntt.inv.contig", st, work(t, out, 8));
+            k_ntt_rows<true, SA, MT><<<row_grid(out), row_threads(SA), 0, st>>>(t, in, out, 0);
         }
         PFT_LAUNCH_CHECK("intt pass B");
-        {
-            PFT_PROF("ntt.inv.strided", st, work);
-            k_ntt8_strided<true, 8, MINB><<<grid, 256, 0, st>>>(t, out, out, second_pass(t, kPassFinal));
-        }
+        PFT_PROF("ntt.inv.strided", st, work(t, out, SA));
+        if (unscaled)
+            k_ntt_cols<true, SA, MT, true>
+                <<<col_grid(out), col_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
+        else
+            k_ntt_cols<true, SA, MT><<<col_grid(out), col_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("intt pass A");
     }
-}
-
-// variant 0: 3 CTAs per SM; 1: 4 CTAs per SM (both with the lane-major row twiddles)
-static void launch_ntt16_twopass(const DevTables& t, const PolySet& in, const PolySet& out, bool inverse, int v16,
-                                 cudaStream_t st) {
-    if (v16 == 1) launch_ntt16_twopass_v<4, true>(t, in, out, inverse, st);
-    else launch_ntt16_twopass_v<3, true>(t, in, out, inverse, st);
-}
-
-template <int MINB, bool LM>
-static void launch_ntt16_inverse_unscaled_v(const DevTables& t, const PolySet& in, const PolySet& out,
-                                            cudaStream_t st) {
-    prepare_twopass<MINB>();
-    dim3 grid(16, (unsigned)out.max_limbs, (unsigned)out.count);
-    const double work = set_limbs(out) * (double)(t.n / 2) * 8;
-    {
-        PFT_PROF("ntt.inv.contig", st, work);
-        launch_contig<true, MINB, LM>(t, in, out, 0, st);
+};
+// f(TwoPass<..>) for the ring's shape; v: 0 = bounded for 768 resident threads per SM (3 CTAs of 256),
+// 1 = for 1024 (4 CTAs; N = 2^16 and 2^15)
+template <class F>
+static void with_twopass(const DevTables& t, int v, F f) {
+    switch (t.logn) {
+        case 12: f(TwoPass<4, 768>()); break;
+        case 13: f(TwoPass<5, 768>()); break;
+        case 14: f(TwoPass<6, 768>()); break;
+        case 15:
+            if (v == 1) f(TwoPass<7, 1024>());
+            else f(TwoPass<7, 768>());
+            break;
+        case 16:
+            if (v == 1) f(TwoPass<8, 1024>());
+            else f(TwoPass<8, 768>());
+            break;
+        default: fail(PFT_ERR_ARG, "internal: no two-pass transform for this ring degree");
     }
-    PFT_LAUNCH_CHECK("intt pass B");
-    {
-        PFT_PROF("ntt.inv.strided", st, work);
-        k_ntt8_strided<true, 8, MINB, true><<<grid, 256, 0, st>>>(t, out, out, second_pass(t, kPassFinal));
-    }
-    PFT_LAUNCH_CHECK("intt pass A (unscaled)");
-}
-
-template <int MINB, bool LM>
-static void launch_ntt16_epi_v(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
-    prepare_twopass<MINB>();
-    dim3 grid(16, (unsigned)io.max_limbs, (unsigned)io.count);
-    const double work = set_limbs(io) * (double)(t.n / 2) * 8;
-    {
-        PFT_PROF("ntt.fwd.strided", st, work);
-        k_ntt8_strided<false, 8, MINB><<<grid, 256, 0, st>>>(t, io, io, 0);
-    }
-    PFT_LAUNCH_CHECK("ntt pass A");
-    {
-        // named apart from the plain transform launches: it also moves the epilogue's operands
-        PFT_PROF("epi.ntt_moddown", st, work);
-        k_ntt8_contig_epi<MINB, LM><<<grid, 256, 0, st>>>(t, io, e,
-                                                           second_pass(t, (t.ntt_order & 4) ? kPassPrefetch : 0));
-    }
-    PFT_LAUNCH_CHECK("ntt pass B + ModDown epilogue");
 }
 
 template <bool INV, int MINB>
@@ -668,11 +683,11 @@ static void launch_ntt16_cluster(const DevTables& t, const PolySet& in, const Po
     launch_ntt16_cluster_v<INV, 2>(t, in, out, st);
 }
 
-// N = 2^16 variant: the context's choice (pft_autotune), unless PFT_NTT16 names one
-// (twopass, twopass4, cluster, generic).
-// the N = 2^16 kernel family of a launch of `limbs` limbs: the environment's choice, else the
-// autotuned plan of the launch's size bucket, else the context's fixed variant
-static int ntt16_variant(const DevTables& t, double limbs = -1) {
+// The kernel family of a launch of `limbs` limbs (N >= 2^12): 0 / 1 two-pass register rounds, 2 cluster
+// (N = 2^16 only), 3 generic.  N = 2^16: the environment's choice (PFT_NTT16 = twopass, twopass4,
+// cluster, generic) first; N >= 2^15: the autotuned plan of the launch's size bucket; then the
+// context's fixed variant.
+static int ntt_family(const DevTables& t, double limbs) {
     static int env = -2;
     if (env == -2) {
         const char* e = getenv("PFT_NTT16");
@@ -683,12 +698,11 @@ static int ntt16_variant(const DevTables& t, double limbs = -1) {
                  : strcmp(e, "generic") == 0  ? 3
                                               : -1;
     }
-    if (env >= 0) return env;
-    if (limbs >= 0) {
-        const int k = t.plan[ntt_bucket(limbs)].kind;
-        if (k >= 0) return k;
-    }
-    return t.ntt_variant;
+    if (t.logn < 12) return 3;
+    int k = t.ntt_variant;
+    if (t.logn == 16 && env >= 0) k = env;
+    else if (t.logn >= 15 && t.plan[ntt_bucket(limbs)].kind >= 0) k = t.plan[ntt_bucket(limbs)].kind;
+    return k == 2 && t.logn != 16 ? 0 : k;
 }
 
 template <int S, int C, bool INV>
@@ -896,6 +910,8 @@ int ntt_candidates(int logn, DevTables::Plan* out, const char** names, int cap) 
         {"staged 9+6", {3, 2, {9, 6, 0}, {8, 64, 0}}},
         {"staged 6+9", {3, 2, {6, 9, 0}, {64, 8, 0}}},
         {"staged 5+5+5 (three passes)", {3, 3, {5, 5, 5}, {128, 128, 128}}},
+        {"two-pass 7+8 (register rounds), 3 CTAs/SM", {0, 0, {0, 0, 0}, {0, 0, 0}}},
+        {"two-pass 7+8 (register rounds), 4 CTAs/SM", {1, 0, {0, 0, 0}, {0, 0, 0}}},
     };
     const Cand* c = logn == 16 ? c16 : logn == 15 ? c15 : nullptr;
     const int n = logn == 16 ? (int)(sizeof(c16) / sizeof(c16[0])) : logn == 15 ? (int)(sizeof(c15) / sizeof(c15[0])) : 0;
@@ -926,40 +942,22 @@ static void run_single(const DevTables& t, const PolySet& in, const PolySet& out
 
 static void run(const DevTables& t, const PolySet& in, const PolySet& out, bool inverse, cudaStream_t st) {
     if (out.count == 0) return;
-    if (t.logn <= 14) {
-        if (inverse) run_single<true>(t, in, out, st);
-        else run_single<false>(t, in, out, st);
-        return;
-    }
-    const DevTables::Plan& pl = t.plan[ntt_bucket(set_limbs(out))];
-    const int v16 = t.logn == 16 ? ntt16_variant(t, set_limbs(out)) : (pl.kind == 3 ? 3 : -1);
-    if (v16 == 3 && pl.kind == 3) {  // a generic plan chosen for this launch size
-        run_generic(t, pl, in, out, inverse, st);
-        return;
-    }
-    if (v16 == 0 || v16 == 1) {
-        launch_ntt16_twopass(t, in, out, inverse, v16, st);
-    } else if (v16 == 2) {
+    const int fam = ntt_family(t, set_limbs(out));
+    if (fam <= 1) {
+        with_twopass(t, fam, [&](auto tp) {
+            if (inverse) tp.inverse(t, in, out, false, st);
+            else tp.forward(t, in, out, st);
+        });
+    } else if (fam == 2) {
         if (!inverse) launch_ntt16_cluster<false>(t, in, out, st);
         else launch_ntt16_cluster<true>(t, in, out, st);
-    } else if (t.logn == 16) {
-        if (!inverse) {
-            launch_pass<8, 16, false>(t, in, out, 0, 0, st);   // stages 0..7, stride 256
-            launch_pass<8, 16, false>(t, out, out, 8, 1, st);  // stages 8..15, contiguous
-        } else {
-            launch_pass<8, 16, true>(t, in, out, 8, 0, st);
-            launch_pass<8, 16, true>(t, out, out, 0, 1, st);
-        }
-    } else if (t.logn == 15) {
-        if (!inverse) {
-            launch_pass<8, 16, false>(t, in, out, 0, 0, st);
-            launch_pass<7, 16, false>(t, out, out, 8, 1, st);
-        } else {
-            launch_pass<7, 16, true>(t, in, out, 8, 0, st);
-            launch_pass<8, 16, true>(t, out, out, 0, 1, st);
-        }
-    } else {
-        fail(PFT_ERR_ARG, "unsupported ring degree");
+    } else if (t.logn <= 14) {
+        if (inverse) run_single<true>(t, in, out, st);
+        else run_single<false>(t, in, out, st);
+    } else {  // generic passes: the autotuned plan's, or 8 + 8 / 8 + 7 stages
+        const DevTables::Plan& pl = t.plan[ntt_bucket(set_limbs(out))];
+        static const DevTables::Plan p16 = {3, 2, {8, 8, 0}, {16, 16, 0}}, p15 = {3, 2, {8, 7, 0}, {16, 16, 0}};
+        run_generic(t, pl.kind == 3 ? pl : t.logn == 16 ? p16 : p15, in, out, inverse, st);
     }
 }
 
@@ -1081,21 +1079,17 @@ void mul_rates(cudaStream_t st, double* lo, double* hi, double* wide) {
 
 bool ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
     if (out.count == 0) return true;
-    if (t.logn != 16) return false;
-    const int v16 = ntt16_variant(t, set_limbs(out));
-    if (v16 != 0 && v16 != 1) return false;
-    if (v16 == 1) launch_ntt16_inverse_unscaled_v<4, true>(t, in, out, st);
-    else launch_ntt16_inverse_unscaled_v<3, true>(t, in, out, st);
+    const int fam = ntt_family(t, set_limbs(out));
+    if (fam > 1) return false;
+    with_twopass(t, fam, [&](auto tp) { tp.inverse(t, in, out, true, st); });
     return true;
 }
 
 bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
     if (io.count == 0) return true;
-    if (t.logn != 16) return false;
-    const int v16 = ntt16_variant(t, set_limbs(io));
-    if (v16 != 0 && v16 != 1) return false;
-    if (v16 == 1) launch_ntt16_epi_v<4, true>(t, io, e, st);
-    else launch_ntt16_epi_v<3, true>(t, io, e, st);
+    const int fam = ntt_family(t, set_limbs(io));
+    if (fam > 1) return false;
+    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, io, e, st); });
     return true;
 }
 void ntt_inverse(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {

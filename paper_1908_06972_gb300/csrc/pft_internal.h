@@ -61,9 +61,9 @@ struct DevTables {
     ulonglong2* inv;       // [P][N] (psi^-brv(i), shoup)
     ulonglong2* ninv;      // [P] (N^-1, shoup)
     ulonglong2* inv1ninv;  // [P] (psi^-brv(1) N^-1, shoup)
-    // N = 2^16 only (else null): the twiddles of stages 12..15 of fwd / inv in lane-major order,
-    // [P][256 rows u][15 slots][16 lanes w]: slot 2^k - 1 + j, lane w holds entry
-    // 2^(12+k) + u 2^(4+k) + w 2^k + j of the natural table
+    // N >= 2^12 (else null): the twiddles of the last four stages of fwd / inv in lane-major order,
+    // [P][2^SA rows u][15 slots][16 lanes w], SA = logn - 8: slot 2^k - 1 + j, lane w holds entry
+    // 2^(SA+4+k) + u 2^(4+k) + w 2^k + j of the natural table
     ulonglong2* fwd_rows;
     ulonglong2* inv_rows;
     int bconv_tc;          // basis conversion of four source primes on the tensor cores (1, opt-in:
@@ -75,8 +75,8 @@ struct DevTables {
     // pass asks L2 for its epilogue operands at the start of each CTA: faster while the epilogue
     // read one 8-byte word per row, slower since it reads 16 bytes four rows ahead).  Default 3.
     int ntt_order;
-    int ntt_variant;       // N = 2^16 transform: 0 two-pass (3 CTAs/SM), 1 two-pass (4 CTAs/SM),
-                           // 2 one-launch cluster, 3 generic staged passes
+    int ntt_variant;       // transform of N >= 2^12: 0 two-pass (3 CTAs/SM), 1 two-pass (4 CTAs/SM),
+                           // 2 one-launch cluster (N = 2^16), 3 generic staged passes
     // Transform plan per launch size (bucket of the launch's total limbs: <= 64, <= 512,
     // larger), chosen by the autotuner; kind < 0: the fixed variant above.
     struct Plan {
