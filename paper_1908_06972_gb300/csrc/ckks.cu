@@ -417,9 +417,11 @@ KeyRef keyref(pft_ctx* c, u32 key_id) {
 
 // conv <- NTT(conv), then out = (x + c - conv) s (+ acc; entries of acc with a null pointer, or
 // an empty acc: none), with per-limb constants {c, s, s'}: one fused pass where the transform
-// variant has it, else the transform and the elementwise epilogue.
+// variant has it, else the transform and the elementwise epilogue.  gs (only where
+// ntt_always_fused): entry i's accumulator is read through X -> X^gs[i] if gs[i] > 1.
 static void ntt_fwd_sub_scale(pft_ctx* c, const std::vector<PolyRef>& conv, const std::vector<PolyRef>& x,
-                              const std::vector<PolyRef>& acc, const std::vector<PolyRef>& out, const u64* consts) {
+                              const std::vector<PolyRef>& acc, const std::vector<PolyRef>& out, const u64* consts,
+                              const std::vector<u32>* gs = nullptr) {
     std::vector<PolyRef> a = acc;
     if (a.empty())
         for (const PolyRef& r : x) a.push_back(ref(nullptr, r.nlimbs));
@@ -430,9 +432,11 @@ static void ntt_fwd_sub_scale(pft_ctx* c, const std::vector<PolyRef>& conv, cons
         e.acc = mkset(a, lo, hi);
         e.out = mkset(out, lo, hi);
         e.consts = consts;
+        for (size_t i = lo; i < hi; i++) e.g[i - lo] = gs ? (*gs)[i] : 0;
         if (fused) fused = ntt_forward_epilogue(c->tabs, mkset(conv, lo, hi), e, c->stream);
     });
     if (fused) return;
+    NEED(!gs, PFT_ERR_ARG, "internal: permuted accumulators without the fused pass");
     ntt_fwd(c, conv, conv);
     std::vector<PolyRef> xw, yw, aw, ow, xn, yn, on;
     for (size_t i = 0; i < conv.size(); i++) {
@@ -449,6 +453,48 @@ static void ntt_fwd_sub_scale(pft_ctx* c, const std::vector<PolyRef>& conv, cons
     }
     if (!ow.empty()) subscale(c, xw, &yw, &aw, ow, consts);
     if (!on.empty()) subscale(c, xn, &yn, nullptr, on, consts);
+}
+
+// ModUp of digit j of an input at level l: coefficient form at `coef` to the rows of `ext` outside
+// the digit
+static BconvJob modup_job(pft_ctx* c, int l, int j, const u64* coef, u64* ext, bool unscaled) {
+    const size_t tab = (size_t)(l - 1) * c->beta_max + j;
+    BconvJob J;
+    J.ns = std::min(l, (j + 1) * c->alpha) - j * c->alpha;
+    J.src_p0 = J.skip_lo = j * c->alpha;
+    J.skip_hi = J.skip_lo + J.ns;
+    J.src = coef + (size_t)J.skip_lo * c->n;
+    J.dst = ext;
+    J.table = (unscaled ? c->modup_tab_u : c->modup_tab)[tab];
+    J.tc = c->modup_tc[tab];
+    J.nrows = l + c->k;
+    J.split = l;
+    J.base2 = c->L;
+    J.pad = 0;
+    return J;
+}
+// ModDown of special rows (coefficient form) to q_0..q_{l-1}
+static BconvJob moddown_job(pft_ctx* c, int l, const u64* special, u64* conv, bool unscaled) {
+    BconvJob J;
+    J.src = special;
+    J.dst = conv;
+    J.table = (unscaled ? c->moddown_tab_u : c->moddown_tab)[l - 1];
+    J.tc = c->moddown_tc[l - 1];
+    J.ns = c->k;
+    J.src_p0 = c->L;
+    J.nrows = l;
+    J.skip_lo = 0;
+    J.skip_hi = 0;
+    J.split = l;
+    J.base2 = c->L;
+    J.pad = 0;
+    return J;
+}
+// the converted rows of digit j at level l (those outside the digit)
+static void modup_rows(pft_ctx* c, int l, int j, u64* ext, std::vector<PolyRef>& rows) {
+    const int lo = j * c->alpha, hi = std::min(l, lo + c->alpha);
+    if (lo > 0) rows.push_back(ref(ext, lo, 0));
+    rows.push_back(ref(ext + (size_t)hi * c->n, l + c->k - hi, hi, l - hi, c->L));
 }
 
 void keyswitch_batch(pft_ctx* c, u32 key_id, const std::vector<KsIO>& io) {
@@ -491,24 +537,8 @@ void keyswitch_batch(pft_ctx* c, u32 key_id, const std::vector<KsIO>& io) {
     {
         std::vector<BconvJob> jobs;
         for (size_t b = 0; b < B; b++) {
-            const int l = io[b].l, E = l + k, beta = (l + alpha - 1) / alpha;
-            for (int j = 0; j < beta; j++) {
-                const int lo = j * alpha, hi = std::min(l, lo + alpha);
-                BconvJob J;
-                J.src = dc(b) + (size_t)lo * limb;
-                J.dst = ext(b, j);
-                J.table = (unscaled ? c->modup_tab_u : c->modup_tab)[(size_t)(l - 1) * c->beta_max + j];
-                J.tc = c->modup_tc[(size_t)(l - 1) * c->beta_max + j];
-                J.ns = hi - lo;
-                J.src_p0 = lo;
-                J.nrows = E;
-                J.skip_lo = lo;
-                J.skip_hi = hi;
-                J.split = l;
-                J.base2 = L;
-                J.pad = 0;
-                jobs.push_back(J);
-            }
+            const int l = io[b].l, beta = (l + alpha - 1) / alpha;
+            for (int j = 0; j < beta; j++) jobs.push_back(modup_job(c, l, j, dc(b), ext(b, j), unscaled));
         }
         bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
         // the digit's own rows are d itself: the inner product reads them there
@@ -517,12 +547,8 @@ void keyswitch_batch(pft_ctx* c, u32 key_id, const std::vector<KsIO>& io) {
     {
         std::vector<PolyRef> rows;
         for (size_t b = 0; b < B; b++) {
-            const int l = io[b].l, E = l + k, beta = (l + alpha - 1) / alpha;
-            for (int j = 0; j < beta; j++) {
-                const int lo = j * alpha, hi = std::min(l, lo + alpha);
-                if (lo > 0) rows.push_back(ref(ext(b, j), lo, 0));
-                rows.push_back(ref(ext(b, j) + (size_t)hi * limb, E - hi, hi, l - hi, L));
-            }
+            const int l = io[b].l, beta = (l + alpha - 1) / alpha;
+            for (int j = 0; j < beta; j++) modup_rows(c, l, j, ext(b, j), rows);
         }
         ntt_fwd(c, rows, rows);
     }
@@ -534,36 +560,19 @@ void keyswitch_batch(pft_ctx* c, u32 key_id, const std::vector<KsIO>& io) {
             d[b].u = uu(b, 0);
             d[b].d = io[b].d;
             d[b].l = io[b].l;
-            d[b].pad = 0;
         }
         ks_inner_multi(c->tabs, d.data(), (int)B, key, L, k, alpha, c->stream);
     }
     // 5. ModDown: coefficient form of the special rows, conversion to q_0..q_{l-1}, evaluation form
     {
         std::vector<PolyRef> sp;
-        std::vector<BconvJob> jobs;
-        for (size_t b = 0; b < B; b++) {
-            const int l = io[b].l;
-            for (int pol = 0; pol < 2; pol++) {
-                sp.push_back(ref(uu(b, pol) + (size_t)l * limb, k, 0, 0, L));
-                BconvJob J;
-                J.src = uu(b, pol) + (size_t)l * limb;
-                J.dst = cv(b, pol);
-                J.table = nullptr;  // chosen below, with the form of the transform
-                J.tc = c->moddown_tc[l - 1];
-                J.ns = k;
-                J.src_p0 = L;
-                J.nrows = l;
-                J.skip_lo = 0;
-                J.skip_hi = 0;
-                J.split = l;
-                J.base2 = L;
-                J.pad = 0;
-                jobs.push_back(J);
-            }
-        }
+        for (size_t b = 0; b < B; b++)
+            for (int pol = 0; pol < 2; pol++) sp.push_back(ref(uu(b, pol) + (size_t)io[b].l * limb, k, 0, 0, L));
         const bool unscaled5 = ntt_inv_unscaled(c, sp, sp);
-        for (BconvJob& J : jobs) J.table = (unscaled5 ? c->moddown_tab_u : c->moddown_tab)[J.nrows - 1];
+        std::vector<BconvJob> jobs;
+        for (size_t b = 0; b < B; b++)
+            for (int pol = 0; pol < 2; pol++)
+                jobs.push_back(moddown_job(c, io[b].l, uu(b, pol) + (size_t)io[b].l * limb, cv(b, pol), unscaled5));
         bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
     }
     // 6. out = acc + (u_Q - conv) P^-1, fused with the last forward pass of conv where the
@@ -767,21 +776,189 @@ static void op_rotate_batch(pft_ctx* c, const pft_ct* const* a, int B, int32_t s
     keyswitch_batch(c, g, io);
 }
 
-// Rotations of one ciphertext by several steps sharing one ModUp of c1 (hoisting): the
-// extended digits (evaluation form) are permuted by each step's automorphism, then go through
+// Rotations of ciphertexts (any levels) by several steps, the ModUp of each c1 shared by its
+// rotations (hoisting): the extended digits (evaluation form) go through each step's automorphism,
 // the inner product with that step's key and ModDown; out_i = (aut(c0) + u0', u1').
-void op_rotate_hoisted(pft_ctx* c, const pft_ct* a, const int32_t* steps, int n, pft_ct* const* outs) {
-    check_ct(c, a);
+// outs[i * n + s] = in[i] rotated by steps[s].
+//
+// One form for all keys and rings: the automorphism is applied where the digits and c0 are read
+// (k_ks_inner_bulk, k_ntt_rows_epi), every stage is one launch over a tile of inputs and steps.
+// Tiles: inputs whose extended digits fit kHoistExtBytes; steps such that the products of the tile
+// fit kHoistTileBytes (launches of some hundred limbs already fill the GPU; one input and step are
+// 10 MiB at level 3 and 64 MiB at level 30), halved while the allocator refuses.
+constexpr size_t kHoistExtBytes = (size_t)2 << 30, kHoistTileBytes = (size_t)512 << 20;
+
+static void hoisted_tile(pft_ctx* c, const pft_ct* const* in, int B, const std::vector<u32>& gs,
+                         const std::vector<std::vector<pft_ct*>>& outs) {
+    const int k = c->k, L = c->L, alpha = c->alpha, n = (int)gs.size();
+    const size_t limb = (size_t)c->n;
+    std::vector<size_t> oDc(B), oExt(B), oU(B), oCv(B);
+    size_t tDc = 0, tExt = 0, tU = 0, tCv = 0;
+    for (int b = 0; b < B; b++) {
+        const int l = in[b]->level, E = l + k, beta = (l + alpha - 1) / alpha;
+        oDc[b] = tDc;
+        oExt[b] = tExt;
+        oU[b] = tU;
+        oCv[b] = tCv;
+        tDc += l;
+        tExt += (size_t)beta * E;
+        tU += 2 * (size_t)E;
+        tCv += 2 * (size_t)l;
+    }
+    Scratch Ext(c, tExt * limb * 8);
+    auto ext = [&](int b, int j) { return Ext.u() + (oExt[b] + (size_t)j * (in[b]->level + k)) * limb; };
+    std::vector<KsDesc> desc(B);
+    {
+        // ModUp of every c1, once
+        Scratch Dc(c, tDc * limb * 8);
+        std::vector<PolyRef> src, dst, rows;
+        for (int b = 0; b < B; b++) {
+            src.push_back(cpoly(in[b]->data, in[b]->level, c->n, 1));
+            dst.push_back(ref(Dc.u() + oDc[b] * limb, in[b]->level));
+        }
+        const bool unscaled = ntt_inv_unscaled(c, src, dst);  // N^-1 then in the conversion tables
+        std::vector<BconvJob> jobs;
+        for (int b = 0; b < B; b++) {
+            const int l = in[b]->level, beta = (l + alpha - 1) / alpha;
+            for (int j = 0; j < beta; j++) {
+                jobs.push_back(modup_job(c, l, j, dst[b].ptr, ext(b, j), unscaled));
+                modup_rows(c, l, j, ext(b, j), rows);
+            }
+        }
+        bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
+        ntt_fwd(c, rows, rows);
+    }
+    int tile = (int)std::max<size_t>(1, std::min<size_t>(n, kHoistTileBytes / ((tU + tCv) * limb * 8)));
+    std::unique_ptr<Scratch> U, Cv;
+    for (;;) {
+        try {
+            U.reset(new Scratch(c, tile * tU * limb * 8));
+            Cv.reset(new Scratch(c, tile * tCv * limb * 8));
+            break;
+        } catch (const Error& e) {
+            U.reset();
+            if (e.code != PFT_ERR_OOM || tile == 1) throw;
+            tile = (tile + 1) / 2;
+        }
+    }
+    for (int b = 0; b < B; b++) {
+        desc[b].ext = ext(b, 0);
+        desc[b].u = U->u() + oU[b] * limb;
+        desc[b].d = in[b]->data + (size_t)in[b]->level * limb;
+        desc[b].l = in[b]->level;
+    }
+    for (int s0 = 0; s0 < n; s0 += tile) {
+        const int ns = std::min(tile, n - s0);
+        std::vector<KeyRef> keys;
+        for (int s = 0; s < ns; s++) keys.push_back(keyref(c, gs[s0 + s]));
+        ks_inner_hoisted(c->tabs, desc.data(), B, keys.data(), &gs[s0], ns, tU * limb, L, k, alpha, c->stream);
+        std::vector<PolyRef> sp, cvr, x, acc, o;
+        std::vector<u32> g;
+        for (int s = 0; s < ns; s++)
+            for (int b = 0; b < B; b++) {
+                const int l = in[b]->level;
+                pft_ct* ob = outs[b][s0 + s];
+                for (int pol = 0; pol < 2; pol++) {
+                    u64* up = U->u() + (s * tU + oU[b] + (size_t)pol * (l + k)) * limb;
+                    sp.push_back(ref(up + (size_t)l * limb, k, 0, 0, L));
+                    cvr.push_back(ref(Cv->u() + (s * tCv + oCv[b] + (size_t)pol * l) * limb, l));
+                    x.push_back(ref(up, l));
+                    acc.push_back(ref(pol ? nullptr : in[b]->data, l));
+                    o.push_back(cpoly(ob->data, l, c->n, pol));
+                    g.push_back(gs[s0 + s]);
+                }
+            }
+        const bool unscaled = ntt_inv_unscaled(c, sp, sp);
+        std::vector<BconvJob> jobs;
+        for (size_t i = 0; i < sp.size(); i++)
+            jobs.push_back(moddown_job(c, cvr[i].nlimbs, sp[i].ptr, cvr[i].ptr, unscaled));
+        bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
+        ntt_fwd_sub_scale(c, cvr, x, acc, o, c->moddown_consts, &g);
+    }
+}
+
+static void rotate_hoisted_one(pft_ctx* c, const pft_ct* a, const std::vector<u32>& gs,
+                               const std::vector<pft_ct*>& outs);
+
+void op_rotate_hoisted(pft_ctx* c, const pft_ct* const* in, int B, const int32_t* steps, int n, pft_ct* const* outs) {
     NEED(n >= 0 && (n == 0 || (steps && outs)), PFT_ERR_ARG, "bad arguments");
+    int lmax = 0;
+    for (int b = 0; b < B; b++) {
+        check_ct(c, in[b]);
+        lmax = std::max(lmax, in[b]->level);
+        for (int s = 0; s < n; s++)
+            NEED(outs[(size_t)b * n + s] && outs[(size_t)b * n + s] != in[b], PFT_ERR_ARG,
+                 "outputs must be distinct from the input");
+    }
+    std::vector<u32> gs;
+    std::vector<int> at;
+    bool streamed = ntt_always_fused(c->tabs);
+    for (int s = 0; s < n; s++) {
+        const u32 g = galois_of(c->n, steps[s]);
+        NEED(g == 1 || c->keys.count(g), PFT_ERR_NO_KEY, "no rotation key for step " + std::to_string(steps[s]));
+        if (g == 1) continue;
+        gs.push_back(g);
+        at.push_back(s);
+        streamed = streamed && ks_inner_bulk_ok(c->tabs, keyref(c, g), lmax, c->alpha);
+    }
+    // a handle that appears for several steps of one input ends with the last step's rotation: only
+    // that one is computed (the steps of a tile run in one launch)
+    if (std::set<pft_ct*>(outs, outs + (size_t)B * n).size() != (size_t)B * n) {
+        NEED(B == 1, PFT_ERR_ARG, "internal: an output appears twice");
+        std::vector<int32_t> st;
+        std::vector<pft_ct*> o;
+        for (int s = 0; s < n; s++)
+            if (std::find(outs + s + 1, outs + n, outs[s]) == outs + n) {
+                st.push_back(steps[s]);
+                o.push_back(outs[s]);
+            }
+        op_rotate_hoisted(c, in, 1, st.data(), (int)st.size(), o.data());
+        return;
+    }
+    const size_t limb = (size_t)c->n;
+    std::vector<std::vector<pft_ct*>> act(B);
+    for (int b = 0; b < B; b++) {
+        const int l = in[b]->level;
+        for (int s = 0, i = 0; s < n; s++) {
+            pft_ct* o = outs[(size_t)b * n + s];
+            ensure_ct(c, o, l);
+            o->scale = in[b]->scale;
+            if (i < (int)at.size() && at[i] == s) {
+                act[b].push_back(o);
+                i++;
+            } else {  // identity rotation
+                PFT_CUDA(cudaMemcpyAsync(o->data, in[b]->data, 2 * l * limb * 8, cudaMemcpyDeviceToDevice, c->stream));
+            }
+        }
+    }
+    if (gs.empty()) return;
+    if (!streamed) {  // compressed keys, more than 16 digits, rings or plans without the fused pass
+        for (int b = 0; b < B; b++) rotate_hoisted_one(c, in[b], gs, act[b]);
+        return;
+    }
+    int b0 = 0;
+    while (b0 < B) {
+        int b1 = b0;
+        size_t bytes = 0;
+        while (b1 < B) {
+            const int l = in[b1]->level;
+            const size_t w = ((size_t)(l + c->alpha - 1) / c->alpha * (l + c->k) + l) * limb * 8;
+            if (b1 > b0 && bytes + w > kHoistExtBytes) break;
+            bytes += w;
+            b1++;
+        }
+        hoisted_tile(c, in + b0, b1 - b0, gs,
+                     std::vector<std::vector<pft_ct*>>(act.begin() + b0, act.begin() + b1));
+        b0 = b1;
+    }
+}
+
+// The same for one ciphertext, step by step, with permuted copies of the extended digits and of c0:
+// where the streamed form above does not apply.
+static void rotate_hoisted_one(pft_ctx* c, const pft_ct* a, const std::vector<u32>& gs,
+                               const std::vector<pft_ct*>& outs) {
     const int l = a->level, k = c->k, L = c->L, alpha = c->alpha, E = l + k, beta = (l + alpha - 1) / alpha;
     const size_t limb = (size_t)c->n;
-    std::vector<u32> gs(n);
-    for (int i = 0; i < n; i++) {
-        NEED(outs[i] && outs[i] != a, PFT_ERR_ARG, "outputs must be distinct from the input");
-        gs[i] = galois_of(c->n, steps[i]);
-        NEED(gs[i] == 1 || c->keys.count(gs[i]), PFT_ERR_NO_KEY, "no rotation key for step " + std::to_string(steps[i]));
-    }
-    if (n == 0) return;
     Scratch Dc(c, l * limb * 8), Ext(c, (size_t)beta * E * limb * 8), ExtG(c, (size_t)beta * E * limb * 8),
         U(c, 2 * (size_t)E * limb * 8), Cv(c, 2 * (size_t)l * limb * 8), A0(c, l * limb * 8);
     u64* c1 = a->data + (size_t)l * limb;
@@ -794,38 +971,17 @@ void op_rotate_hoisted(pft_ctx* c, const pft_ct* a, const int32_t* steps, int n,
         std::vector<PolyRef> cin, cout, rows;
         for (int j = 0; j < beta; j++) {
             const int lo = j * alpha, hi = std::min(l, lo + alpha);
-            BconvJob J;
-            J.src = Dc.u() + (size_t)lo * limb;
-            J.dst = ext(Ext.u(), j);
-            J.table = (unscaled ? c->modup_tab_u : c->modup_tab)[(size_t)(l - 1) * c->beta_max + j];
-            J.tc = c->modup_tc[(size_t)(l - 1) * c->beta_max + j];
-            J.ns = hi - lo;
-            J.src_p0 = lo;
-            J.nrows = E;
-            J.skip_lo = lo;
-            J.skip_hi = hi;
-            J.split = l;
-            J.base2 = L;
-            J.pad = 0;
-            jobs.push_back(J);
+            jobs.push_back(modup_job(c, l, j, Dc.u(), ext(Ext.u(), j), unscaled));
+            modup_rows(c, l, j, ext(Ext.u(), j), rows);
             cin.push_back(ref(c1 + (size_t)lo * limb, hi - lo, lo));
             cout.push_back(ref(ext(Ext.u(), j) + (size_t)lo * limb, hi - lo, lo));
-            if (lo > 0) rows.push_back(ref(ext(Ext.u(), j), lo, 0));
-            rows.push_back(ref(ext(Ext.u(), j) + (size_t)hi * limb, E - hi, hi, l - hi, L));
         }
         bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
         ew(c, EwOp::Copy, cin, {}, cout);
         ntt_fwd(c, rows, rows);
     }
-    for (int i = 0; i < n; i++) {
+    for (size_t i = 0; i < gs.size(); i++) {
         pft_ct* o = outs[i];
-        const double sc = a->scale;
-        ensure_ct(c, o, l);
-        o->scale = sc;
-        if (gs[i] == 1) {
-            PFT_CUDA(cudaMemcpyAsync(o->data, a->data, 2 * l * limb * 8, cudaMemcpyDeviceToDevice, c->stream));
-            continue;
-        }
         // automorphism of the extended digits and of c0
         std::vector<PolyRef> ein, eout;
         for (int j = 0; j < beta; j++) {
@@ -841,28 +997,14 @@ void op_rotate_hoisted(pft_ctx* c, const pft_ct* a, const int32_t* steps, int n,
         ks_inner_multi(c->tabs, &d, 1, keyref(c, gs[i]), L, k, alpha, c->stream);
         // ModDown
         std::vector<PolyRef> sp, cvr;
-        std::vector<BconvJob> jobs;
         for (int pol = 0; pol < 2; pol++) {
-            u64* up = U.u() + (size_t)pol * E * limb;
-            sp.push_back(ref(up + (size_t)l * limb, k, 0, 0, L));
+            sp.push_back(ref(U.u() + ((size_t)pol * E + l) * limb, k, 0, 0, L));
             cvr.push_back(ref(Cv.u() + (size_t)pol * l * limb, l));
-            BconvJob J;
-            J.src = up + (size_t)l * limb;
-            J.dst = Cv.u() + (size_t)pol * l * limb;
-            J.table = nullptr;  // chosen with the form of the transform
-            J.tc = c->moddown_tc[l - 1];
-            J.ns = k;
-            J.src_p0 = L;
-            J.nrows = l;
-            J.skip_lo = 0;
-            J.skip_hi = 0;
-            J.split = l;
-            J.base2 = L;
-            J.pad = 0;
-            jobs.push_back(J);
         }
         const bool unscaled_sp = ntt_inv_unscaled(c, sp, sp);
-        for (BconvJob& J : jobs) J.table = (unscaled_sp ? c->moddown_tab_u : c->moddown_tab)[l - 1];
+        std::vector<BconvJob> jobs;
+        for (int pol = 0; pol < 2; pol++)
+            jobs.push_back(moddown_job(c, l, sp[pol].ptr, cvr[pol].ptr, unscaled_sp));
         bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
         const std::vector<PolyRef> xs{ref(U.u(), l), ref(U.u() + (size_t)E * limb, l)};
         const std::vector<PolyRef> as{ref(A0.u(), l), ref(nullptr, l)};
@@ -1238,58 +1380,70 @@ static void ft_finish_columns(pft_ctx* c, const pft_ft_model* M, const std::vect
     op_rescale_batch(c, S.data(), (int)S.size(), S.data());
 }
 
-// BEGIN, diagonal packing: Q = sum_k rot(v, k) D_k, documents in chunks that bound the memory
-// of the rotated copies.
+// BEGIN, diagonal packing: Q = sum_i sum_k rot(v_i, k) D_{i,k} (chunk i of the vocabulary): the n - 1
+// hoisted rotations of every chunk of every document in one batched call, then one dot product
+// of chunks n terms per document.  Documents (any levels, ordered by level) go in groups that bound
+// the memory of the rotated copies.
 static void ft_begin_diag(pft_ctx* c, const pft_ft_model* M, const std::vector<FtDoc*>& docs) {
     const int cols = M->n, nch = M->chunks;
     const size_t limb = c->n;
     std::vector<int32_t> hsteps;
     for (int k = 1; k < cols; k++) hsteps.push_back(k);
     for (FtDoc* d : docs) ft_init_work(c, d, 1, d->v[0]->scale * M->H[0]->scale);
-    // per document: the n - 1 hoisted rotations of each vocabulary chunk, then one dot product
-    // Q = sum_i sum_k rot(v_i, k) D_{i,k} over all of them (K = chunks n terms)
     const size_t rot_per_doc = (size_t)nch * (cols - 1);
-    for (auto& kv : docs_by_level(docs)) {
-        const int l = kv.first;
-        const std::vector<FtDoc*>& G = kv.second;
-        const size_t per_doc = rot_per_doc * 2 * l * limb * 8;
-        const size_t chunk = std::max<size_t>(1, std::min<size_t>(G.size(), ((size_t)16 << 30) / per_doc));
-        for (size_t b0 = 0; b0 < G.size(); b0 += chunk) {
-            const size_t b1 = std::min(G.size(), b0 + chunk);
-            std::vector<pft_ct> R((b1 - b0) * rot_per_doc);
-            struct CleanR {
-                pft_ctx* c;
-                std::vector<pft_ct>* T;
-                ~CleanR() {
-                    for (auto& x : *T) dfree(c, x.data);
-                }
-            } cleanR{c, &R};
-            for (auto& x : R) x.ctx = c;
-            auto rot = [&](size_t b, int i, int k) -> pft_ct& {  // rot(v_i, k) of document b, k >= 1
-                return R[(b - b0) * rot_per_doc + (size_t)i * (cols - 1) + k - 1];
-            };
-            for (size_t b = b0; b < b1; b++)
-                for (int i = 0; i < nch; i++) {
-                    std::vector<pft_ct*> outs;
-                    for (int k = 1; k < cols; k++) outs.push_back(&rot(b, i, k));
-                    op_rotate_hoisted(c, G[b]->v[i], hsteps.data(), cols - 1, outs.data());
-                }
+    std::vector<FtDoc*> order(docs);
+    std::stable_sort(order.begin(), order.end(), [](const FtDoc* x, const FtDoc* y) { return x->l < y->l; });
+    size_t b0 = 0;
+    while (b0 < order.size()) {
+        size_t b1 = b0, bytes = 0;
+        while (b1 < order.size()) {
+            const size_t w = rot_per_doc * 2 * order[b1]->l * limb * 8;
+            if (b1 > b0 && bytes + w > ((size_t)16 << 30)) break;
+            bytes += w;
+            b1++;
+        }
+        std::vector<pft_ct> R((b1 - b0) * rot_per_doc);
+        struct CleanR {
+            pft_ctx* c;
+            std::vector<pft_ct>* T;
+            ~CleanR() {
+                for (auto& x : *T) dfree(c, x.data);
+            }
+        } cleanR{c, &R};
+        std::vector<const pft_ct*> in;
+        std::vector<pft_ct*> outs;
+        for (size_t b = b0; b < b1; b++)
+            for (int i = 0; i < nch; i++) in.push_back(order[b]->v[i]);
+        for (auto& x : R) {  // [document][chunk][k - 1]
+            x.ctx = c;
+            outs.push_back(&x);
+        }
+        op_rotate_hoisted(c, in.data(), (int)in.size(), hsteps.data(), cols - 1, outs.data());
+        const std::vector<FtDoc*> group(order.begin() + b0, order.begin() + b1);
+        size_t at = 0;
+        for (auto& kv : docs_by_level(group)) {  // ascending levels: the order of `group`
+            const int l = kv.first;
             std::vector<const u64*> A, Bv;
             std::vector<u64*> O;
             for (int i = 0; i < nch; i++)
                 for (int k = 0; k < cols; k++) Bv.push_back(M->H[(size_t)i * cols + k]->data);
-            for (size_t b = b0; b < b1; b++)
+            for (FtDoc* d : kv.second) {
+                const pft_ct* rot = &R[at * rot_per_doc];
+                at++;
                 for (int pol = 0; pol < 2; pol++) {
                     for (int i = 0; i < nch; i++) {
-                        A.push_back(G[b]->v[i]->data + (size_t)pol * l * limb);
-                        for (int k = 1; k < cols; k++) A.push_back(rot(b, i, k).data + (size_t)pol * l * limb);
+                        A.push_back(d->v[i]->data + (size_t)pol * l * limb);
+                        for (int k = 1; k < cols; k++)
+                            A.push_back(rot[(size_t)i * (cols - 1) + k - 1].data + (size_t)pol * l * limb);
                     }
-                    O.push_back(G[b]->W[0].data + (size_t)pol * l * limb);
+                    O.push_back(d->W[0].data + (size_t)pol * l * limb);
                 }
+            }
             Scratch dA(c, A.size() * 8), dB(c, Bv.size() * 8), dO(c, O.size() * 8);
-            ew_dot(c->tabs, upload(c, dA, A), upload(c, dB, Bv), upload(c, dO, O), (int)O.size(), nch * cols, true,
-                   l, c->stream);
+            ew_dot(c->tabs, upload(c, dA, A), upload(c, dB, Bv), upload(c, dO, O), (int)O.size(), nch * cols, true, l,
+                   c->stream);
         }
+        b0 = b1;
     }
 }
 
@@ -2086,7 +2240,7 @@ int pft_dot_plain_batch(pft_ctx* c, const pft_ct* const* cts, const pft_pt* cons
 }
 
 int pft_rotate_hoisted(pft_ctx* c, const pft_ct* a, const int32_t* steps, int n, pft_ct* const* outs) {
-    return guard(c, [&] { op_rotate_hoisted(c, a, steps, n, outs); });
+    return guard(c, [&] { op_rotate_hoisted(c, &a, 1, steps, n, outs); });
 }
 int pft_add_batch(pft_ctx* c, const pft_ct* const* a, const pft_ct* const* b, int B, pft_ct* const* out) {
     return guard(c, [&] {

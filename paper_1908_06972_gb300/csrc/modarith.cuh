@@ -137,4 +137,16 @@ __device__ __forceinline__ DPrime load_prime(const DPrime* tab, int i) {
     return p;
 }
 
+// Galois automorphism X -> X^g in the evaluation layout, as a source index.
+// Entry i holds a(psi^(2 brv(i) + 1)); a(X^g) there equals a(psi^((2 brv(i) + 1) g)),
+// i.e. entry brv(((2 brv(i) + 1) g mod 2N - 1) / 2) of the input.
+__device__ __forceinline__ u32 automorph_src(u32 i, int logn, u64 g) {
+    const u32 mask2n = (2u << logn) - 1;
+    const u32 bi = __brev(i) >> (32 - logn);
+    const u32 e = (u32)(((u64)(2 * bi + 1) * g) & mask2n);
+    return __brev((e - 1) >> 1) >> (32 - logn);
+}
+// The top bits of a source index depend only on the top bits of its destination, so every aligned
+// block of 2^b destinations reads one aligned block of 2^b sources.
+
 }  // namespace pft

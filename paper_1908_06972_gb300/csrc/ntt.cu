@@ -537,6 +537,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     const size_t base = (size_t)limb << logn;
     const u64* __restrict__ xs = e.x.p[poly].ptr + base;
     const u64* __restrict__ as = e.acc.p[poly].ptr;  // null: no accumulator for this polynomial
+    const u32 g = e.g[poly];                         // above 1: the accumulator is read through X -> X^g
     u64* __restrict__ os = e.out.p[poly].ptr + base;
     if (flags & kPassPrefetch) {
         // ask L2 for this CTA's tile of the epilogue operands (one 128-byte line per thread and
@@ -561,7 +562,10 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
             const int f = 2 * (threadIdx.x + NT * (4 * h + i));
             const size_t j = ((size_t)(blockIdx.x * R) << 8) + f;
             xv[i] = *reinterpret_cast<const ulonglong2*>(xs + j);
-            if (as) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
+            if (as && g <= 1) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
+            if (as && g > 1)  // a row of 256 points reads one row of 256 sources: L1 holds it
+                av[i] = make_ulonglong2(as[base + automorph_src((u32)j, logn, g)],
+                                        as[base + automorph_src((u32)j + 1, logn, g)]);
         }
 #pragma unroll
         for (int i = 0; i < 4; i++) {
@@ -1085,6 +1089,11 @@ bool ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& 
     return true;
 }
 
+bool ntt_always_fused(const DevTables& t) {
+    for (double limbs : {1.0, 100.0, 1000.0})
+        if (ntt_family(t, limbs) > 1) return false;
+    return true;
+}
 bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
     if (io.count == 0) return true;
     const int fam = ntt_family(t, set_limbs(io));

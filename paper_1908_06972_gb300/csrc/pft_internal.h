@@ -134,13 +134,17 @@ inline double set_limbs(const PolySet& s) {
 void ntt_forward(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
 // The ModDown epilogue applied by the last forward pass: out = (x + c - NTT(io)) s (+ acc; a null
 // acc pointer: none), per-limb constants {c, s, s'} at consts[3 limb].
+// acc may be read through X -> X^g per polynomial (g[i] > 1; then out must not overlap acc).
 struct NttEpi {
     PolySet x, acc, out;
     const u64* consts;
+    u32 g[kMaxSet];
 };
 // Forward transform of io (in place) fused with the epilogue; false (nothing launched) where
 // the ring or the transform variant has no fused kernel.
 bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st);
+// Whether launches of every size have that fused kernel.
+bool ntt_always_fused(const DevTables& t);
 // N times the inverse transform (no N^-1 at the last stage, values in [0, 4q)) for consumers
 // that scale their input anyway; false (nothing launched) where the ring or the transform
 // variant has no such kernel.
@@ -201,7 +205,7 @@ struct KsDesc {
     const u64* d;  // the input in evaluation form: rows of digit j are read here (ext's copies
                    // of them are not written); null: ext holds them
     int l;
-    int pad;
+    int beta;  // digits at level l (set by the launcher)
 };
 constexpr int kMaxKs = 128;  // inputs per launch (by-value parameters)
 // A switching key as the inner product reads it: [beta][2 (b, a)][L+k][N] in evaluation form,
@@ -220,6 +224,14 @@ struct KeyRef {
 };
 void ks_inner_multi(const DevTables& t, const KsDesc* descs_host, int B, const KeyRef& key, int L, int k, int alpha,
                     cudaStream_t st);
+// Whether the streamed kernel serves inputs up to level lmax with this key (whole blocks of 256
+// coefficients, an uncompressed key, at most 16 digits).
+bool ks_inner_bulk_ok(const DevTables& t, const KeyRef& key, int lmax, int alpha);
+// The inner products of the same inputs, read through X -> X^gs[z], with key z of nk keys (all
+// ks_inner_bulk_ok): input b's result for key z goes to u + z * zstride (words).
+constexpr int kMaxKsKeys = 64;  // keys per launch (by-value parameters)
+void ks_inner_hoisted(const DevTables& t, const KsDesc* descs_host, int B, const KeyRef* keys, const u32* gs, int nk,
+                      size_t zstride, int L, int k, int alpha, cudaStream_t st);
 // Whether a kernel's bounded wait has expired since the last reset (reads a device flag).
 int wait_timeout_flag(bool reset, cudaStream_t st);
 // Persistent job queue: elementwise jobs over ciphertexts of any rings and levels in one launch.

@@ -256,15 +256,6 @@ void sub_scale(const DevTables& t, const PolySet& x, const PolySet* y, const Pol
 }
 
 // ---- Galois automorphism X -> X^g in the evaluation layout ---------------------------------
-// Entry i holds a(psi^(2 brv(i) + 1)); a(X^g) there equals a(psi^((2 brv(i) + 1) g)),
-// i.e. entry brv(((2 brv(i) + 1) g mod 2N - 1) / 2) of the input.
-__device__ __forceinline__ u32 automorph_src(u32 i, int logn, u64 g) {
-    const u32 mask2n = (2u << logn) - 1;
-    const u32 bi = __brev(i) >> (32 - logn);
-    const u32 e = (u32)(((u64)(2 * bi + 1) * g) & mask2n);
-    return __brev((e - 1) >> 1) >> (32 - logn);
-}
-
 // Multiplication by an odd g modulo 2N fixes the low bits of an exponent given its low bits,
 // so in the bit-reversed layout the top bits of a source index depend only on the top bits of
 // its destination: every block of kAutBlock consecutive outputs reads one block of
@@ -738,12 +729,14 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
     }
 }
 
-// ---- the same with bulk copies (cp.async.bulk + mbarrier) ---------------------------------
-// CTA = one key row x 256 coefficients, 128 threads with two coefficients each and the key
-// slice in registers.  The digit rows of the inputs that use the row stream through a ring
-// of kKsStages shared-memory stages (one input's digits, 2 KiB each) filled by one thread
-// with 1-D bulk copies whose bytes an mbarrier per stage counts: the CTA computes input u
-// while the copies of the next inputs are in flight.  Every wait is bounded; on expiry the
+// ---- the same with bulk copies (cp.async.bulk + mbarrier), up to 16 digits, several keys ----------
+// CTA = one key row x 256 coefficients of one key, with the key slice in registers: two
+// coefficients per thread (128 threads) up to 8 digits, one (256 threads) up to 16.  The digit
+// rows of the inputs that use the row stream through a ring of kKsStages shared-memory stages
+// (2 KiB per digit row; a stage holds the rows of several inputs where they have few digits, so
+// that the two CTA barriers per stage and the copies in flight cover enough bytes) filled by one
+// thread with 1-D bulk copies whose bytes an mbarrier per stage counts: the CTA computes one
+// stage while the copies of the next are in flight.  Every wait is bounded; on expiry the
 // kernel records the failure in g_wait_timeout, then drains its own copies in flight: one
 // thread waits for every stage that still expects bytes, with a bound 16 times the first
 // (kDrainPolls), before the CTA returns.  A copy of 2 KiB per digit row lands in microseconds;
@@ -752,7 +745,19 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // PFT_ERR_TIMEOUT from pft_device_status).  (Per-warp waits with an "empty" mbarrier per stage
 // in place of the two CTA barriers per input measured slower: 201 against 196 us for 4
 // ciphertexts at level 30; so did one coefficient per thread in CTAs of 256 threads, 64
-// registers and twice the resident warps: 221 us.)
+// registers and twice the resident warps, for 8 digits: 221 us.)
+// Bound: HBM and the multiply pipe together from 3 digits on (187 us for 4 ciphertexts at level 30,
+// 5.3 TB/s), the latency of a stage below.  64 inputs of one digit (level 3): 265 us with one input
+// per stage, 194 us with four.  9 digits at N = 2^15 (31 inputs, levels 12..18) ran in the generic kernel
+// before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms.
+// The key slice is loaded before the ring is started: after it (copies in flight first) measured
+// slower for few inputs, 95 against 87 us for one at level 30.
+// PERM (hoisted rotations): grid z = several keys over the same inputs, key z with Galois element
+// g[z]; the digit rows are read through X -> X^g.  A chunk of 256 destinations reads one aligned
+// block of 256 sources, so the copies stay whole blocks and only the reads from shared memory are
+// permuted: no permuted copy of the extended digits is made (it was beta (l + k) limbs written and
+// read per rotation).  With the batching of op_rotate_hoisted over inputs and steps, 32 rotation-light
+// inferences at level 3: 132 -> 48 ms; 4 at N = 2^15, levels 12..18: 80 -> 22 ms.
 constexpr int kKsStages = 3;
 constexpr int kKsChunk = 256;                // coefficients per CTA (2 KiB per digit row)
 constexpr long long kWaitPolls = 1ll << 22;  // polls of a bounded wait (seconds at most)
@@ -806,10 +811,19 @@ __device__ __forceinline__ u64 ks_value(const Acc3K& s, const DPrime& P) {
     return mont_reduce(a.hi, a.lo, P.q, P.mneg);
 }
 
-template <int BMAX>
-__global__ void __launch_bounds__(128) k_ks_inner_bulk(DevTables t, KsBatch bt, int B, KeyRef kr, int L, int k,
-                                                       int alpha, int stage_digits) {
-    extern __shared__ __align__(128) u64 ring[];  // [kKsStages][stage_digits][kKsChunk]
+__host__ __device__ constexpr int ks_cpt(int bmax) { return bmax <= 8 ? 2 : 1; }  // coefficients per thread
+struct KsKeys {
+    const u64* mont[kMaxKsKeys];
+    u32 g[kMaxKsKeys];
+};
+
+template <int BMAX, bool PERM>
+__global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
+    k_ks_inner_bulk(DevTables t, KsBatch bt, int B, KsKeys keys, size_t zstride, int L, int k, int alpha,
+                    int stage_digits, int per_stage_arg) {
+    constexpr int CPT = ks_cpt(BMAX);
+    const int per_stage = BMAX > 2 ? 1 : per_stage_arg;  // digits above 2: one input per stage
+    extern __shared__ __align__(128) u64 ring[];  // [kKsStages][per_stage][stage_digits][kKsChunk]
     __shared__ __align__(8) u64 bars[kKsStages];
     // special rows first: every input uses them, so their CTAs are the longest and should not
     // form the last wave
@@ -819,16 +833,38 @@ __global__ void __launch_bounds__(128) k_ks_inner_bulk(DevTables t, KsBatch bt, 
     const int need = bt.need[row];
     if (need == 0) return;  // uniform over the CTA
     const size_t chunk0 = (size_t)blockIdx.x * kKsChunk;
-    const int xl = 2 * threadIdx.x;
+    const int xl = CPT * threadIdx.x;
     const size_t xo = chunk0 + xl;
     const DPrime P = load_prime(t.primes, row);
-    const u64* key = kr.mont;  // split Montgomery form: k0 | k1 << 32 with k 2^64 mod p = k1 2^30 + k0
-    ulonglong2 kb[BMAX], ka[BMAX];
+    const u64* key = keys.mont[blockIdx.z];  // split Montgomery form: k0 | k1 << 32 with k 2^64 mod p = k1 2^30 + k0
+    const size_t uz = PERM ? (size_t)blockIdx.z * zstride : 0;
+    size_t src0 = chunk0;
+    int xs[CPT];  // this thread's coefficients in a staged row
+#pragma unroll
+    for (int c = 0; c < CPT; c++) xs[c] = xl + c;
+    if (PERM) {
+        const u32 g = keys.g[blockIdx.z];
+        src0 = automorph_src((u32)chunk0, logn, g) & ~(u32)(kKsChunk - 1);
+#pragma unroll
+        for (int c = 0; c < CPT; c++) xs[c] = automorph_src((u32)xo + c, logn, g) & (kKsChunk - 1);
+    }
+    u64 kb[BMAX][CPT], ka[BMAX][CPT];
 #pragma unroll
     for (int j = 0; j < BMAX; j++) {
         if (j < need) {
-            kb[j] = __ldg(reinterpret_cast<const ulonglong2*>(key + ((((size_t)j * 2 + 0) * rows_total + row) << logn) + xo));
-            ka[j] = __ldg(reinterpret_cast<const ulonglong2*>(key + ((((size_t)j * 2 + 1) * rows_total + row) << logn) + xo));
+            const u64* pb = key + ((((size_t)j * 2 + 0) * rows_total + row) << logn) + xo;
+            const u64* pa = key + ((((size_t)j * 2 + 1) * rows_total + row) << logn) + xo;
+            if constexpr (CPT == 2) {
+                const ulonglong2 vb = __ldg(reinterpret_cast<const ulonglong2*>(pb));
+                const ulonglong2 va = __ldg(reinterpret_cast<const ulonglong2*>(pa));
+                kb[j][0] = vb.x;
+                kb[j][1] = vb.y;
+                ka[j][0] = va.x;
+                ka[j][1] = va.y;
+            } else {
+                kb[j][0] = __ldg(pb);
+                ka[j][0] = __ldg(pa);
+            }
         }
     }
     auto used = [&](int b) { return !(row < L && row >= bt.d[b].l); };
@@ -836,76 +872,130 @@ __global__ void __launch_bounds__(128) k_ks_inner_bulk(DevTables t, KsBatch bt, 
         while (b < B && !used(b)) b++;
         return b;
     };
-    // thread 0 fills stage s with the digit rows of input b
-    auto issue = [&](int b, int s) {
+    auto rows_of = [&](int b, int s, int i) {  // thread 0: the copies of input b's digit rows, i-th of stage s
         const KsDesc& D = bt.d[b];
-        const int l = D.l, E = l + k, beta = (l + alpha - 1) / alpha;
-        const int m = row < L ? row : l + row - L;
-        mbar_expect_tx(&bars[s], (u32)(beta * kKsChunk * 8));
-        for (int j = 0; j < beta; j++)
-            bulk_g2s(ring + ((size_t)s * stage_digits + j) * kKsChunk, ks_row(D, j, E, m, alpha, logn) + chunk0,
-                     (u32)(kKsChunk * 8), &bars[s]);
+        const int E = D.l + k, m = row < L ? row : D.l + row - L;
+        for (int j = 0; j < D.beta; j++)
+            bulk_g2s(ring + (((size_t)s * per_stage + i) * stage_digits + j) * kKsChunk,
+                     ks_row(D, j, E, m, alpha, logn) + src0, (u32)(kKsChunk * 8), &bars[s]);
+    };
+    // thread 0 fills stage s with the digit rows of up to per_stage used inputs from b on
+    auto issue = [&](int b, int s) {
+        if (per_stage == 1) {
+            mbar_expect_tx(&bars[s], (u32)(bt.d[b].beta * kKsChunk * 8));
+            rows_of(b, s, 0);
+            return;
+        }
+        u32 rows = 0;
+        for (int i = 0, bb = b; i < per_stage && bb < B; i++, bb = next(bb + 1)) rows += (u32)bt.d[bb].beta;
+        mbar_expect_tx(&bars[s], rows * (kKsChunk * 8));
+        for (int i = 0; i < per_stage && b < B; i++, b = next(b + 1)) rows_of(b, s, i);
+    };
+    auto skip = [&](int b) {  // the first used input after a stage that starts at b
+        for (int i = 0; i < per_stage && b < B; i++) b = next(b + 1);
+        return b;
     };
     if (threadIdx.x == 0) {
         for (int s2 = 0; s2 < kKsStages; s2++) mbar_init(&bars[s2], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    // prologue: the first kKsStages used inputs
-    int ib = next(0);
-    if (threadIdx.x == 0) {
-        int bb = ib;
-        for (int s2 = 0; s2 < kKsStages && bb < B; s2++, bb = next(bb + 1)) issue(bb, s2);
-    }
-    for (int s2 = 0; s2 < kKsStages && ib < B; s2++) ib = next(ib + 1);  // ib: next input to issue
-    int u = 0;
-    for (int b = next(0); b < B; b = next(b + 1), u++) {
-        const int s = u % kKsStages;
-        const u32 parity = (u32)((u / kKsStages) & 1);
+    int ib = next(0), issued = 0;  // the next input to issue, stages issued so far
+    for (; issued < kKsStages && ib < B; issued++, ib = skip(ib))
+        if (threadIdx.x == 0) issue(ib, issued);
+    int u = 0, s = 0;
+    u32 parity = 0;
+    for (int b = next(0); b < B; u++) {
         const bool ok = __syncthreads_and(mbar_wait(&bars[s], parity));
         if (!ok) {
             // record, then wait (bounded) for the copies still in flight on the other stages
             if (threadIdx.x == 0) {
                 atomicExch(&g_wait_timeout, 1);
                 mbar_wait(&bars[s], parity, kDrainPolls);
-                int uu = u + 1;
-                for (int bb = next(b + 1); bb < ib; bb = next(bb + 1), uu++)
+                for (int uu = u + 1; uu < issued; uu++)
                     mbar_wait(&bars[uu % kKsStages], (u32)((uu / kKsStages) & 1), kDrainPolls);
             }
             return;
         }
-        const KsDesc& D = bt.d[b];
-        const int l = D.l, E = l + k, beta = (l + alpha - 1) / alpha;
-        const int m = row < L ? row : l + row - L;
-        const u64* st = ring + (size_t)s * stage_digits * kKsChunk + xl;
-        // sums of at most 8 products of residues below 2^60 in 30-bit-split Karatsuba partial
-        // sums (three widening multiply-adds per product), then one Montgomery reduction: the key
-        // words carry the factor 2^64 (sum < 8 p^2 < p 2^63)
-        Acc3K s0x = {0, 0, 0}, s0y = {0, 0, 0}, s1x = {0, 0, 0}, s1y = {0, 0, 0};
+        for (int i = 0; i < per_stage && b < B; i++, b = next(b + 1)) {
+            const KsDesc& D = bt.d[b];
+            const int l = D.l, E = l + k, beta = D.beta;
+            const int m = row < L ? row : l + row - L;
+            const u64* st = ring + ((size_t)s * per_stage + i) * stage_digits * kKsChunk;
+            // sums of at most 8 products of residues below 2^60 in 30-bit-split Karatsuba partial
+            // sums (three widening multiply-adds per product), then one Montgomery reduction: the
+            // key words carry the factor 2^64 (sum < 8 p^2 < p 2^63)
+            u64 r0[CPT], r1[CPT];
 #pragma unroll
-        for (int j = 0; j < BMAX; j++) {
-            if (j < beta) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(st + (size_t)j * kKsChunk);
-                ks_mac(s0x, s1x, v.x, kb[j].x, ka[j].x);
-                ks_mac(s0y, s1y, v.y, kb[j].y, ka[j].y);
+            for (int h = 0; h < BMAX; h += 8) {
+                if (h > 0 && beta <= h) break;
+                Acc3K s0[CPT], s1[CPT];
+#pragma unroll
+                for (int c = 0; c < CPT; c++) s0[c] = s1[c] = {0, 0, 0};
+#pragma unroll
+                for (int j = h; j < (BMAX < h + 8 ? BMAX : h + 8); j++) {
+                    if (j < beta) {
+                        u64 v[CPT];
+                        if constexpr (CPT == 2 && !PERM) {
+                            const ulonglong2 vv =
+                                *reinterpret_cast<const ulonglong2*>(st + (size_t)j * kKsChunk + xl);
+                            v[0] = vv.x;
+                            v[1] = vv.y;
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < CPT; c++) v[c] = st[(size_t)j * kKsChunk + xs[c]];
+                        }
+#pragma unroll
+                        for (int c = 0; c < CPT; c++) ks_mac(s0[c], s1[c], v[c], kb[j][c], ka[j][c]);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < CPT; c++) {
+                    const u64 v0 = ks_value(s0[c], P), v1 = ks_value(s1[c], P);
+                    r0[c] = h ? addmod(r0[c], v0, P.q) : v0;
+                    r1[c] = h ? addmod(r1[c], v1, P.q) : v1;
+                }
+            }
+            u64* o0 = D.u + uz + ((size_t)m << logn) + xo;
+            u64* o1 = D.u + uz + (((size_t)E + m) << logn) + xo;
+            if constexpr (CPT == 2) {
+                *reinterpret_cast<ulonglong2*>(o0) = make_ulonglong2(r0[0], r0[1]);
+                *reinterpret_cast<ulonglong2*>(o1) = make_ulonglong2(r1[0], r1[1]);
+            } else {
+                *o0 = r0[0];
+                *o1 = r1[0];
             }
         }
-        ulonglong2 r0, r1;
-        r0.x = ks_value(s0x, P);
-        r0.y = ks_value(s0y, P);
-        r1.x = ks_value(s1x, P);
-        r1.y = ks_value(s1y, P);
-        *reinterpret_cast<ulonglong2*>(D.u + ((size_t)m << logn) + xo) = r0;
-        *reinterpret_cast<ulonglong2*>(D.u + (((size_t)E + m) << logn) + xo) = r1;
         __syncthreads();  // every thread has read stage s
         if (ib < B) {
             if (threadIdx.x == 0) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 issue(ib, s);
             }
-            ib = next(ib + 1);
+            issued++;
+            ib = skip(ib);
+        }
+        if (++s == kKsStages) {
+            s = 0;
+            parity ^= 1;
         }
     }
+}
+
+template <int BMAX, bool PERM>
+static void launch_ks_bulk(const DevTables& t, const KsBatch& bt, int B, const KsKeys& keys, int nk, size_t zstride,
+                           int L, int k, int alpha, int lmax, int digits, cudaStream_t st) {
+    // inputs per stage: 8 KiB of digit rows (24 KiB per CTA), but no fewer than kKsStages stages over
+    // the batch
+    const int per = std::max(1, std::min(digits <= 2 ? 4 / digits : 1, (B + kKsStages - 1) / kKsStages));
+    const size_t smem = (size_t)kKsStages * per * digits * kKsChunk * 8;
+    if (first_on_device((const void*)&k_ks_inner_bulk<BMAX, PERM>))
+        PFT_CUDA(cudaFuncSetAttribute(k_ks_inner_bulk<BMAX, PERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((size_t)kKsStages * std::max(8, BMAX) * kKsChunk * 8)));
+    // rows no input reaches (above the highest level) get no CTA
+    const dim3 grid((unsigned)(t.n / kKsChunk), (unsigned)(lmax + k), (unsigned)nk);
+    k_ks_inner_bulk<BMAX, PERM>
+        <<<grid, kKsChunk / ks_cpt(BMAX), smem, st>>>(t, bt, B, keys, zstride, L, k, alpha, digits, per);
 }
 
 // Self-test of the bounded wait: an mbarrier that expects bytes no copy delivers (no copy is
@@ -1083,48 +1173,89 @@ __global__ void k_ks_inner_multi_generic(DevTables t, KsBatch bt, int B, KeyRef 
     }
 }
 
+bool ks_inner_bulk_ok(const DevTables& t, const KeyRef& key, int lmax, int alpha) {
+    return (lmax + alpha - 1) / alpha <= 16 && !key.compressed && key.mont && t.n % kKsChunk == 0;
+}
+
+// need[] of the batch's rows, the bytes one key's pass moves and the highest level
+static KsBatch ks_batch(const DevTables& t, const KsDesc* descs, int cnt, int L, int k, int alpha, double* bytes,
+                        int* lmax) {
+    KsBatch bt;
+    *bytes = 0;
+    *lmax = 0;
+    for (int r = 0; r < kMaxPrimes; r++) bt.need[r] = 0;
+    for (int i = 0; i < cnt; i++) {
+        bt.d[i] = descs[i];
+        const int l = descs[i].l, E = l + k, beta = (l + alpha - 1) / alpha;
+        bt.d[i].beta = beta;
+        *bytes += (double)(beta + 2) * E * t.n * 8.0;
+        *lmax = max(*lmax, l);
+        for (int r = 0; r < L + k; r++)
+            if ((r >= L || r < l) && bt.need[r] < beta) bt.need[r] = (uint8_t)beta;
+    }
+    return bt;
+}
+
+template <bool PERM>
+static void ks_bulk(const DevTables& t, const KsBatch& bt, int B, const KsKeys& keys, int nk, size_t zstride, int L,
+                    int k, int alpha, int lmax, cudaStream_t st) {
+    const int digits = (lmax + alpha - 1) / alpha;
+    auto go = [&](auto f) { f(t, bt, B, keys, nk, zstride, L, k, alpha, lmax, digits, st); };
+    if (digits <= 1) go(launch_ks_bulk<1, PERM>);
+    else if (digits <= 2) go(launch_ks_bulk<2, PERM>);
+    else if (digits <= 4) go(launch_ks_bulk<4, PERM>);
+    else if (digits <= 8) go(launch_ks_bulk<8, PERM>);
+    else go(launch_ks_bulk<16, PERM>);
+}
+
 void ks_inner_multi(const DevTables& t, const KsDesc* descs, int B, const KeyRef& key, int L, int k, int alpha,
                     cudaStream_t st) {
-    const int beta_max = (L + alpha - 1) / alpha;
     for (int a = 0; a < B; a += kMaxKs) {
         const int cnt = B - a < kMaxKs ? B - a : kMaxKs;
-        KsBatch bt;
-        double bytes = 0;
-        int lmax = 0;
-        for (int r = 0; r < kMaxPrimes; r++) bt.need[r] = 0;
-        for (int i = 0; i < cnt; i++) {
-            bt.d[i] = descs[a + i];
-            const int l = descs[a + i].l, E = l + k, beta = (l + alpha - 1) / alpha;
-            bytes += (double)(beta + 2) * E * t.n * 8.0;
-            lmax = max(lmax, l);
-            for (int r = 0; r < L + k; r++)
-                if ((r >= L || r < l) && bt.need[r] < beta) bt.need[r] = (uint8_t)beta;
-        }
-        bytes += (key.compressed ? 1.0 : 2.0) * ((lmax + alpha - 1) / alpha) * (lmax + k) * t.n * 8.0;  // key rows read
+        double bytes;
+        int lmax;
+        const KsBatch bt = ks_batch(t, descs + a, cnt, L, k, alpha, &bytes, &lmax);
+        const int beta = (lmax + alpha - 1) / alpha;
+        bytes += (key.compressed ? 1.0 : 2.0) * beta * (lmax + k) * t.n * 8.0;  // key rows read
         dim3 grid2((unsigned)((t.n / 2 + 127) / 128), (unsigned)(L + k));
         dim3 grid1((unsigned)((t.n + 127) / 128), (unsigned)(L + k));
         PFT_PROF("ks_inner", st, bytes);
-        if (beta_max <= 8 && !key.compressed && key.mont && t.n % kKsChunk == 0) {
-            const int sd = beta_max <= 4 ? 4 : 8;
-            dim3 gb((unsigned)(t.n / kKsChunk), (unsigned)(L + k));
-            const size_t smem = (size_t)kKsStages * sd * kKsChunk * 8;
-            // the 8-digit ring needs 48 KiB of dynamic shared memory
-            if (first_on_device((const void*)&k_ks_inner_bulk<8>)) {
-                PFT_CUDA(cudaFuncSetAttribute(k_ks_inner_bulk<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)((size_t)kKsStages * 8 * kKsChunk * 8)));
-                PFT_CUDA(cudaFuncSetAttribute(k_ks_inner_bulk<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)((size_t)kKsStages * 8 * kKsChunk * 8)));
-            }
-            if (sd == 4) k_ks_inner_bulk<4><<<gb, 128, smem, st>>>(t, bt, cnt, key, L, k, alpha, sd);
-            else k_ks_inner_bulk<8><<<gb, 128, smem, st>>>(t, bt, cnt, key, L, k, alpha, sd);
+        if (ks_inner_bulk_ok(t, key, lmax, alpha)) {
+            KsKeys keys;
+            keys.mont[0] = key.mont;
+            keys.g[0] = 1;
+            ks_bulk<false>(t, bt, cnt, keys, 1, 0, L, k, alpha, lmax, st);
         } else if (key.compressed && t.n < 256) {  // lane pairs need full warps
             k_ks_inner_multi_generic<<<grid1, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
-        } else if (beta_max <= 4 && !key.compressed) k_ks_inner_multi<4, false><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
-        else if (beta_max <= 8 && !key.compressed) k_ks_inner_multi<8, false><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
-        else if (beta_max <= 4) k_ks_inner_multi<4, true><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
-        else if (beta_max <= 8) k_ks_inner_multi<8, true><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
+        } else if (beta <= 4 && !key.compressed) k_ks_inner_multi<4, false><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
+        else if (beta <= 8 && !key.compressed) k_ks_inner_multi<8, false><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
+        else if (beta <= 4) k_ks_inner_multi<4, true><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
+        else if (beta <= 8) k_ks_inner_multi<8, true><<<grid2, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
         else k_ks_inner_multi_generic<<<grid1, 128, 0, st>>>(t, bt, cnt, key, L, k, alpha);
         PFT_LAUNCH_CHECK("ks_inner_multi");
+    }
+}
+
+void ks_inner_hoisted(const DevTables& t, const KsDesc* descs, int B, const KeyRef* keyrefs, const u32* gs, int nk,
+                      size_t zstride, int L, int k, int alpha, cudaStream_t st) {
+    for (int a = 0; a < B; a += kMaxKs) {
+        const int cnt = B - a < kMaxKs ? B - a : kMaxKs;
+        double bytes;
+        int lmax;
+        const KsBatch bt = ks_batch(t, descs + a, cnt, L, k, alpha, &bytes, &lmax);
+        for (int z = 0; z < nk; z += kMaxKsKeys) {
+            const int nz = nk - z < kMaxKsKeys ? nk - z : kMaxKsKeys;
+            KsBatch bz = bt;
+            for (int i = 0; i < cnt; i++) bz.d[i].u += (size_t)z * zstride;
+            KsKeys keys;
+            for (int i = 0; i < nz; i++) {
+                keys.mont[i] = keyrefs[z + i].mont;
+                keys.g[i] = gs[z + i];
+            }
+            PFT_PROF("ks_inner", st, nz * (bytes + 2.0 * ((lmax + alpha - 1) / alpha) * (lmax + k) * t.n * 8.0));
+            ks_bulk<true>(t, bz, cnt, keys, nz, zstride, L, k, alpha, lmax, st);
+            PFT_LAUNCH_CHECK("ks_inner_hoisted");
+        }
     }
 }
 

@@ -366,10 +366,14 @@ void fwd_tile_diag(pft_ctx* c, pft_ft_tape& T, const pft_ct* const* w, int b0, i
     auto rk = [&](int b, int k) -> const pft_ct* { return doc_rot(T, b, k); };
     std::vector<int32_t> hs;
     for (int k = 1; k < n; k++) hs.push_back(k);
-    for (int b = b0; b < b1; b++) {
-        std::vector<pft_ct*> outs;
-        for (int k = 1; k < n; k++) outs.push_back(&T.r[(size_t)b * n + k]);
-        if (n > 1) op_rotate_hoisted(c, rk(b, 0), hs.data(), n - 1, outs.data());
+    if (n > 1) {
+        std::vector<const pft_ct*> rin;
+        std::vector<pft_ct*> routs;
+        for (int b = b0; b < b1; b++) {
+            rin.push_back(rk(b, 0));
+            for (int k = 1; k < n; k++) routs.push_back(&T.r[(size_t)b * n + k]);
+        }
+        op_rotate_hoisted(c, rin.data(), nb, hs.data(), n - 1, routs.data());
     }
     // Hb
     std::vector<pft_ct*> hx;
