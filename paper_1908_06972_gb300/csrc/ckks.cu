@@ -415,35 +415,42 @@ KeyRef keyref(pft_ctx* c, u32 key_id) {
     return r;
 }
 
-// conv <- NTT(conv), then out = (x + c - conv) s (+ acc; entries of acc with a null pointer, or
-// an empty acc: none), with per-limb constants {c, s, s'}: one fused pass where the transform
-// variant has it, else the transform and the elementwise epilogue.  gs (only where
-// ntt_always_fused): entry i's accumulator is read through X -> X^gs[i] if gs[i] > 1.
+// The operands of a fused ModDown pass over polynomials [lo, hi): entries of acc with a null pointer,
+// or an empty acc, have no accumulator; consts[i]: the i-th polynomial's constants (one entry: of all).
+static NttEpi epi_of(const std::vector<PolyRef>& x, const std::vector<PolyRef>& acc, const std::vector<PolyRef>& out,
+                     const std::vector<const u64*>& consts, const std::vector<u32>* gs, size_t lo, size_t hi) {
+    NttEpi e;
+    for (size_t i = lo; i < hi; i++) {
+        e.x[i - lo] = x[i].ptr;
+        e.acc[i - lo] = acc.empty() ? nullptr : acc[i].ptr;
+        e.out[i - lo] = out[i].ptr;
+        e.consts[i - lo] = consts[consts.size() == 1 ? 0 : i];
+        e.g[i - lo] = gs ? (*gs)[i] : 0;
+    }
+    return e;
+}
+
+// conv <- NTT(conv), then out = (x + c - conv) s (+ acc), with per-limb constants {c, s, s'}: one
+// fused pass where the transform variant has it, else the transform and the elementwise epilogue.
+// gs (only where ntt_always_fused): entry i's accumulator is read through X -> X^gs[i] if gs[i] > 1.
 static void ntt_fwd_sub_scale(pft_ctx* c, const std::vector<PolyRef>& conv, const std::vector<PolyRef>& x,
                               const std::vector<PolyRef>& acc, const std::vector<PolyRef>& out, const u64* consts,
                               const std::vector<u32>* gs = nullptr) {
-    std::vector<PolyRef> a = acc;
-    if (a.empty())
-        for (const PolyRef& r : x) a.push_back(ref(nullptr, r.nlimbs));
     bool fused = true;
     chunks(conv.size(), [&](size_t lo, size_t hi) {
-        NttEpi e;
-        e.x = mkset(x, lo, hi);
-        e.acc = mkset(a, lo, hi);
-        e.out = mkset(out, lo, hi);
-        e.consts = consts;
-        for (size_t i = lo; i < hi; i++) e.g[i - lo] = gs ? (*gs)[i] : 0;
-        if (fused) fused = ntt_forward_epilogue(c->tabs, mkset(conv, lo, hi), e, c->stream);
+        if (fused)
+            fused = ntt_forward_epilogue(c->tabs, mkset(conv, lo, hi), epi_of(x, acc, out, {consts}, gs, lo, hi),
+                                         c->stream);
     });
     if (fused) return;
     NEED(!gs, PFT_ERR_ARG, "internal: permuted accumulators without the fused pass");
     ntt_fwd(c, conv, conv);
     std::vector<PolyRef> xw, yw, aw, ow, xn, yn, on;
     for (size_t i = 0; i < conv.size(); i++) {
-        if (a[i].ptr) {
+        if (!acc.empty() && acc[i].ptr) {
             xw.push_back(x[i]);
             yw.push_back(conv[i]);
-            aw.push_back(a[i]);
+            aw.push_back(acc[i]);
             ow.push_back(out[i]);
         } else {
             xn.push_back(x[i]);
@@ -598,12 +605,6 @@ void keyswitch_batch(pft_ctx* c, u32 key_id, const std::vector<KsIO>& io) {
 }
 
 // ---- operations ---------------------------------------------------------------------------
-
-static std::map<int, std::vector<int>> by_level(const pft_ct* const* a, int B) {
-    std::map<int, std::vector<int>> g;
-    for (int i = 0; i < B; i++) g[a[i]->level].push_back(i);
-    return g;
-}
 
 void op_add_batch(pft_ctx* c, const pft_ct* const* a, const pft_ct* const* b, int B, pft_ct* const* out,
                          EwOp op) {
@@ -1013,6 +1014,42 @@ static void rotate_hoisted_one(pft_ctx* c, const pft_ct* a, const std::vector<u3
     }
 }
 
+// RESCALE of polynomials of any levels, in one launch per stage: in[i] at level l (evaluation form,
+// l limbs), last[i] one limb and rb[i] l - 1 limbs of working space, out[i] at level l - 1.
+static void rescale_polys(pft_ctx* c, const std::vector<PolyRef>& in, const std::vector<u64*>& last,
+                          const std::vector<u64*>& rb, const std::vector<PolyRef>& out) {
+    std::vector<PolyRef> lin, lout, rr, x;
+    std::vector<const u64*> consts;
+    for (size_t i = 0; i < in.size(); i++) {
+        const int l = in[i].nlimbs;
+        lin.push_back(ref(in[i].ptr + (size_t)(l - 1) * c->n, 1, l - 1));
+        lout.push_back(ref(last[i], 1, l - 1));
+        rr.push_back(ref(rb[i], l - 1));
+        x.push_back(ref(in[i].ptr, l - 1));
+        consts.push_back(c->rescale_consts[l - 1]);
+    }
+    ntt_inv(c, lin, lout);
+    if (ntt_always_fused(c->tabs)) {
+        chunks(rr.size(), [&](size_t lo, size_t hi) {
+            ntt_rescale_epilogue(c->tabs, mkset(lout, lo, hi), mkset(rr, lo, hi), epi_of(x, {}, out, consts, nullptr, lo, hi),
+                                 c->stream);
+        });
+        return;
+    }
+    chunks(rr.size(), [&](size_t lo, size_t hi) { rescale_bcast(c->tabs, mkset(lout, lo, hi), mkset(rr, lo, hi), c->stream); });
+    std::map<const u64*, std::vector<size_t>> by_consts;  // the elementwise epilogue takes one table per launch
+    for (size_t i = 0; i < rr.size(); i++) by_consts[consts[i]].push_back(i);
+    for (auto& kv : by_consts) {
+        std::vector<PolyRef> r2, x2, o2;
+        for (size_t i : kv.second) {
+            r2.push_back(rr[i]);
+            x2.push_back(x[i]);
+            o2.push_back(out[i]);
+        }
+        ntt_fwd_sub_scale(c, r2, x2, {}, o2, kv.first);
+    }
+}
+
 void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* out) {
     for (int i = 0; i < B; i++) {
         check_ct(c, a[i]);
@@ -1020,39 +1057,54 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
         NEED(a[i]->level >= 2, PFT_ERR_LEVEL_MISMATCH, "rescale needs at least two primes");
     }
     const size_t limb = c->n;
-    for (auto& kv : by_level(a, B)) {
-        const int l = kv.first;
-        const std::vector<int>& idx = kv.second;
-        const size_t G = idx.size();
-        Scratch Last(c, G * 2 * limb * 8), Rb(c, G * 2 * (l - 1) * limb * 8);
-        std::vector<PolyRef> lin, lout, rr, x, y, out_refs;
-        // fresh output buffers (the output is smaller than the input and may alias it)
-        std::vector<u64*> nb(G);
-        for (size_t i = 0; i < G; i++) nb[i] = (u64*)dalloc(c, 2 * (l - 1) * limb * 8);
-        for (size_t i = 0; i < G; i++) {
-            u64* A = a[idx[i]]->data;
+    // fresh output buffers (the output is smaller than the input and may alias it)
+    struct Fresh {
+        pft_ctx* c;
+        std::vector<u64*> p;
+        ~Fresh() {
+            for (u64* q : p) dfree(c, q);
+        }
+    } nb{c, {}};
+    std::vector<double> sc;
+    for (int i = 0; i < B; i++) {
+        nb.p.push_back((u64*)dalloc(c, 2 * (size_t)(a[i]->level - 1) * limb * 8));
+        sc.push_back(a[i]->scale / (double)c->primes[a[i]->level - 1]);
+    }
+    std::vector<int> lv;
+    for (int i = 0; i < B; i++) lv.push_back(a[i]->level);
+    int i0 = 0;
+    while (i0 < B) {  // all levels together, in tiles that bound the working space
+        int i1 = i0;
+        size_t words = 0;
+        while (i1 < B) {
+            const size_t w = 2 * (size_t)lv[i1] * limb;
+            if (i1 > i0 && (words + w) * 8 > kRescaleScratchBudget) break;
+            words += w;
+            i1++;
+        }
+        Scratch S(c, words * 8);
+        std::vector<PolyRef> in, o;
+        std::vector<u64*> last, rb;
+        u64* at = S.u();
+        for (int i = i0; i < i1; i++)
             for (int pol = 0; pol < 2; pol++) {
-                lin.push_back(ref(A + ((size_t)pol * l + l - 1) * limb, 1, l - 1));
-                lout.push_back(ref(Last.u() + (i * 2 + pol) * limb, 1, l - 1));
-                rr.push_back(ref(Rb.u() + (i * 2 + pol) * (l - 1) * limb, l - 1));
-                x.push_back(ref(A + (size_t)pol * l * limb, l - 1));
-                out_refs.push_back(ref(nb[i] + (size_t)pol * (l - 1) * limb, l - 1));
+                in.push_back(cpoly(a[i]->data, lv[i], c->n, pol));
+                o.push_back(cpoly(nb.p[i], lv[i] - 1, c->n, pol));
+                last.push_back(at);
+                rb.push_back(at + limb);
+                at += (size_t)lv[i] * limb;
             }
-        }
-        ntt_inv(c, lin, lout);
-        chunks(rr.size(), [&](size_t p, size_t q) { rescale_bcast(c->tabs, mkset(lout, p, q), mkset(rr, p, q), c->stream); });
-        ntt_fwd_sub_scale(c, rr, x, {}, out_refs, c->rescale_consts[l - 1]);
-        for (size_t i = 0; i < G; i++) {
-            pft_ct* o = out[idx[i]];
-            const double sc = a[idx[i]]->scale / (double)c->primes[l - 1];
-            dfree(c, o->data);  // stream-ordered: queued work on the old buffer completes first
-            o->data = nb[i];
-            o->cap = 2 * (size_t)(l - 1) * limb;
-            o->level = l - 1;
-            o->scale = sc;
-        }
-        // inputs aliased by an output of the same group were released above; make sure no
-        // later entry of this group still points at them (each handle appears once per group)
+        rescale_polys(c, in, last, rb, o);
+        i0 = i1;
+    }
+    for (int i = 0; i < B; i++) {
+        pft_ct* o = out[i];
+        dfree(c, o->data);  // stream-ordered: queued work on the old buffer completes first
+        o->data = nb.p[i];
+        nb.p[i] = nullptr;
+        o->cap = 2 * (size_t)(lv[i] - 1) * limb;
+        o->level = lv[i] - 1;
+        o->scale = sc[i];
     }
 }
 
@@ -2435,18 +2487,15 @@ int pft_rescale_noalloc(pft_ctx* c, const uint64_t* in, int level, uint64_t* out
         u64* last = c->noalloc_scratch;
         u64* rb = last + 2 * n;
         u64* src = (u64*)in;
-        std::vector<PolyRef> lin, lout, rr, x, o;
+        std::vector<PolyRef> x, o;
+        std::vector<u64*> lasts, rbs;
         for (int pol = 0; pol < 2; pol++) {
-            lin.push_back(ref(src + ((size_t)pol * l + l - 1) * n, 1, level - 1));
-            lout.push_back(ref(last + (size_t)pol * n, 1, level - 1));
-            rr.push_back(ref(rb + (size_t)pol * (l - 1) * n, level - 1));
-            x.push_back(ref(src + (size_t)pol * l * n, level - 1));
+            x.push_back(ref(src + (size_t)pol * l * n, level));
             o.push_back(ref(out + (size_t)pol * (l - 1) * n, level - 1));
+            lasts.push_back(last + (size_t)pol * n);
+            rbs.push_back(rb + (size_t)pol * (l - 1) * n);
         }
-        ntt_inv(c, lin, lout);
-        rescale_bcast(c->tabs, mkset(lout, 0, 2), mkset(rr, 0, 2), c->stream);
-        ntt_fwd(c, rr, rr);
-        subscale(c, x, &rr, nullptr, o, c->rescale_consts[level - 1]);
+        rescale_polys(c, x, lasts, rbs, o);
     });
 }
 

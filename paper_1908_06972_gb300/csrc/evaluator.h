@@ -286,6 +286,7 @@ struct RelinIO {
 void relin_batch(pft_ctx* c, const std::vector<RelinIO>& io);
 // Budget for the scratch of one batched key-switching call (inputs are tiled beyond it).
 constexpr size_t kKsScratchBudget = (size_t)24 << 30;
+constexpr size_t kRescaleScratchBudget = (size_t)8 << 30;  // the same of one rescale call
 // Scratch words of one key switch at level l.
 inline size_t ks_scratch_words(const pft_ctx* c, int l) {
     const int E = l + c->k, beta = (l + c->alpha - 1) / c->alpha;

@@ -324,7 +324,11 @@ __host__ __device__ constexpr int row_threads(int SA) { return rows_per_cta(SA) 
 // MT: resident threads per SM the registers are bounded for (768: 80 registers, 1024: 64).
 // UNSCALED (inverse): the last stage is a plain Gentleman-Sande butterfly (no N^-1) and the
 // output stays in [0, 4q): N times the inverse transform, for a consumer that scales anyway.
-template <bool INV, int SA, int MT, bool UNSCALED = false>
+// BCAST (forward): RESCALE's broadcast on the way in.  `in` holds one limb per polynomial, c_{l-1} in
+// coefficient form modulo the dropped prime p (the one after the output's limbs); limb k takes
+// (r - h) mod q_k with r = (c_{l-1} + h) mod p, h = floor(p/2).  A pass of its own for it (k_rescale_bcast)
+// took 17 % of a batch of rescales: it writes and the column pass reads back every limb.
+template <bool INV, int SA, int MT, bool UNSCALED = false, bool BCAST = false>
 __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
     k_ntt_cols(DevTables t, PolySet in, PolySet out, int flags) {
     constexpr int C = cols_per_cta(SA), LO = SA - 4;     // LO: bits of the second round
@@ -347,8 +351,23 @@ __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
     u64 x[16];
     if (!INV) {
         const bool lazy = q < kLazyBound;  // uniform over the CTA (one limb)
+        if constexpr (BCAST) {
+            const u64 p = __ldg(&t.primes[Ro.nlimbs].q), h = p >> 1;
+            const DPrime P = load_prime(t.primes, pi);
+            const u64 hq = reduce64(h, P);
+            const u64* last = in.p[poly].ptr + col;
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << LO) | w) << 8];
+            for (int e = 0; e < 16; e++) x[e] = last[(size_t)((e << LO) | w) << 8];
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+                u64 r = x[e] + h;
+                if (r >= p) r -= p;
+                x[e] = submod(reduce64(r, P), hq, q);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << LO) | w) << 8];
+        }
         if (lazy) ntt_round<false, LO, SA - 1, 4, true>(x, w, 0, tw, q, q2, NI, NI1);
         else ntt_round<false, LO, SA - 1>(x, w, 0, tw, q, q2, NI, NI1);
         if constexpr (SA > 4) {
@@ -523,8 +542,8 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
 }
 
 // Forward row stages fused with the ModDown epilogue: for the canonical transform value v,
-// out = (x + c - v) s mod q (+ acc when the polynomial has one), with per-limb constants
-// {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of the column pass.
+// out = (x + c - v) s mod q (+ acc when the polynomial has one), with the polynomial's per-limb
+// constants {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of the column pass.
 template <int SA, int MT>
 __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     k_ntt_rows_epi(DevTables t, PolySet in, NttEpi e, int flags) {
@@ -535,10 +554,11 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     if (limb >= Ri.nlimbs) return;
     const int pi = prime_of(Ri, limb);
     const size_t base = (size_t)limb << logn;
-    const u64* __restrict__ xs = e.x.p[poly].ptr + base;
-    const u64* __restrict__ as = e.acc.p[poly].ptr;  // null: no accumulator for this polynomial
+    const u64* __restrict__ xs = e.x[poly] + base;
+    const u64* __restrict__ as = e.acc[poly];        // null: no accumulator for this polynomial
     const u32 g = e.g[poly];                         // above 1: the accumulator is read through X -> X^g
-    u64* __restrict__ os = e.out.p[poly].ptr + base;
+    u64* __restrict__ os = e.out[poly] + base;
+    const u64* cs = e.consts[poly] + 3 * limb;
     if (flags & kPassPrefetch) {
         // ask L2 for this CTA's tile of the epilogue operands (one 128-byte line per thread and
         // operand: R rows x 256 words) so that their DRAM reads overlap the transform
@@ -549,7 +569,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     }
     fwd_rows<SA>(t, Ri.ptr + base, pi, sm);
     const u64 q = __ldg(&t.primes[pi].q);
-    const u64 c = __ldg(&e.consts[3 * limb]), s = __ldg(&e.consts[3 * limb + 1]), sp = __ldg(&e.consts[3 * limb + 2]);
+    const u64 c = __ldg(&cs[0]), s = __ldg(&cs[1]), sp = __ldg(&cs[2]);
     // each thread: two adjacent points (16-byte loads and stores) of eight rows or row parts; the
     // operands of four are loaded before any is used, so that more bytes are in flight (the
     // transform's registers are free by now).  An even point m and m + 1 share their 16-point
@@ -593,6 +613,7 @@ static void prepare_twopass(void) {
         const int co = 64;
         auto set = [&](auto k) { PFT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, co)); };
         set(k_ntt_cols<false, SA, MT>);
+        set(k_ntt_cols<false, SA, MT, false, true>);
         set(k_ntt_cols<true, SA, MT>);
         set(k_ntt_cols<true, SA, MT, true>);
         set(k_ntt_rows<false, SA, MT>);
@@ -626,8 +647,16 @@ struct TwoPass {
         k_ntt_rows<false, SA, MT><<<row_grid(out), row_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("ntt pass B");
     }
-    static void forward_epi(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
-        cols_fwd(t, io, io, st);
+    static void forward_epi(const DevTables& t, const PolySet& in, const PolySet& io, const NttEpi& e, bool bcast,
+                            cudaStream_t st) {
+        if (bcast) {
+            prepare_twopass<SA, MT>();
+            PFT_PROF("ntt.fwd.strided", st, work(t, io, SA));
+            k_ntt_cols<false, SA, MT, false, true><<<col_grid(io), col_threads(SA), 0, st>>>(t, in, io, 0);
+            PFT_LAUNCH_CHECK("rescale broadcast + ntt pass A");
+        } else {
+            cols_fwd(t, in, io, st);
+        }
         // named apart from the plain transform launches: it also moves the epilogue's operands
         PFT_PROF("epi.ntt_moddown", st, work(t, io, 8));
         k_ntt_rows_epi<SA, MT><<<row_grid(io), row_threads(SA), 0, st>>>(
@@ -1098,7 +1127,15 @@ bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e
     if (io.count == 0) return true;
     const int fam = ntt_family(t, set_limbs(io));
     if (fam > 1) return false;
-    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, io, e, st); });
+    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, io, io, e, false, st); });
+    return true;
+}
+bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e,
+                          cudaStream_t st) {
+    if (io.count == 0) return true;
+    const int fam = ntt_family(t, set_limbs(io));
+    if (fam > 1) return false;
+    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, last, io, e, true, st); });
     return true;
 }
 void ntt_inverse(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {

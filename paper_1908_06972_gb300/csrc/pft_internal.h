@@ -132,18 +132,24 @@ inline double set_limbs(const PolySet& s) {
 // Negacyclic transform of every limb of every polynomial of `out` (input from `in`,
 // which may be the same set).
 void ntt_forward(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
-// The ModDown epilogue applied by the last forward pass: out = (x + c - NTT(io)) s (+ acc; a null
-// acc pointer: none), per-limb constants {c, s, s'} at consts[3 limb].
-// acc may be read through X -> X^g per polynomial (g[i] > 1; then out must not overlap acc).
+// The ModDown epilogue applied by the last forward pass, per polynomial i of a launch: out = (x + c -
+// NTT(io)) s (+ acc; null: none), with per-limb constants {c, s, s'} at consts[i][3 limb].  acc may be
+// read through X -> X^g (g[i] > 1; then out must not overlap acc).
 struct NttEpi {
-    PolySet x, acc, out;
-    const u64* consts;
+    const u64* x[kMaxSet];
+    const u64* acc[kMaxSet];
+    u64* out[kMaxSet];
+    const u64* consts[kMaxSet];
     u32 g[kMaxSet];
 };
 // Forward transform of io (in place) fused with the epilogue; false (nothing launched) where
 // the ring or the transform variant has no fused kernel.
 bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st);
-// Whether launches of every size have that fused kernel.
+// RESCALE's forward part: io = the broadcast of `last` (one limb in coefficient form per polynomial,
+// the dropped prime being the one after io's limbs; see rescale_bcast), then the same; false
+// (nothing launched) where there is no fused kernel.
+bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e, cudaStream_t st);
+// Whether launches of every size have these fused kernels.
 bool ntt_always_fused(const DevTables& t);
 // N times the inverse transform (no N^-1 at the last stage, values in [0, 4q)) for consumers
 // that scale their input anyway; false (nothing launched) where the ring or the transform

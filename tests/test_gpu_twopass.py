@@ -67,3 +67,30 @@ def test_operations_bit_exact(gpu, logn, variant):
             p.assert_equal(r, o.rotate(want, step), "rotate %d" % step)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("logn,variant", [(11, 0), (12, 0), (13, 3), (13, 0), (14, 0), (15, 0), (15, 1), (16, 0), (16, 3)])
+def test_rescale_batch_mixed_levels(gpu, logn, variant):
+    """One call over ciphertexts of several levels (one in place), 60-bit and 40-bit dropped primes, and
+    the allocation-free form."""
+    import torch
+
+    p = Pair(gpu, logn, 4, 1, 4, mid_bits=40, rot_steps=(), relin=False)
+    try:
+        o, pf, ctx = p.orc, p.pft, p.ctx
+        pf.pft_set_transform_variant(ctx, variant)
+        levels = [4, 2, 3, 4, 2]
+        x = [o.encrypt_sk(o.encode(synth.slots(70 + i, 16), level=l), 80 + i) for i, l in enumerate(levels)]
+        x[0].c[:, -1, :3] = [0, o.q[3] - 1, o.q[3] // 2]  # the ends of the rounding
+        h = [p.ct(c) for c in x]
+        outs = [p.empty(), h[1]] + [p.empty() for _ in levels[2:]]
+        raw = torch.empty((2, 3, p.N), dtype=torch.int64, device="cuda")
+        pf.pft_rescale_noalloc(ctx, pf.pft_ct_data(h[0]), 4, raw.data_ptr())
+        pf.pft_rescale_batch(ctx, h, outs)
+        for i, (g, c) in enumerate(zip(outs, x)):
+            p.assert_equal(g, o.rescale(c), "ciphertext %d at level %d" % (i, levels[i]))
+        got = torch.empty_like(raw)
+        pf.pft_ct_copy_out(ctx, outs[0], got.data_ptr())
+        assert torch.equal(raw, got)
+    finally:
+        p.close()
