@@ -171,7 +171,8 @@ enum class EwOp { Add, Sub, Mul, Neg, Copy };
 void ew_binary(const DevTables& t, EwOp op, const PolySet& a, const PolySet& b, const PolySet& out, cudaStream_t st);
 // HMUL tensor: a, b refs point at ciphertexts [2][l][N]; d refs at [3][l][N] (nlimbs = l).
 void ew_tensor(const DevTables& t, const PolySet& a, const PolySet& b, const PolySet& d, cudaStream_t st);
-// O[p] = sum_{k<K} A[p K + k] * B[(shared ? 0 : p K) + k]; device pointer tables; l limbs each.
+// O[p] = sum_{k<K} A[p K + k] * B[(shared ? 0 : p K) + k]; device pointer tables; l limbs each.  Outputs come in
+// pairs (the two polynomials of a ciphertext) that multiply the same plaintexts.
 void ew_dot(const DevTables& t, const u64* const* A, const u64* const* B, u64* const* O, int n_out, int K,
             bool b_shared, int l, cudaStream_t st);
 // out = acc + ((x + c) - y) * s per limb, consts_dev[3 limb + {0,1,2}] = {c, s, s_shoup};

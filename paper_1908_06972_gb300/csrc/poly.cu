@@ -116,11 +116,48 @@ void ew_tensor(const DevTables& t, const PolySet& a, const PolySet& b, const Pol
     PFT_LAUNCH_CHECK("tensor");
 }
 
-// ---- dot products: out[p] = sum_k a[p*K + k] * b[(shared ? 0 : p*K) + k] --------------------
-// Pointer tables live in device memory (they can be long).  All polynomials carry
-// `l` limbs of the ciphertext chain.  128-bit accumulation, reduced every 8 terms.
-__global__ void k_dot(DevTables t, const u64* const* A, const u64* const* Bp, u64* const* O, int K, int b_shared,
-                      int l) {
+// ---- sums of products ---------------------------------------------------------------------------
+// Pointer tables live in device memory (they can be long) and go through shared memory a chunk of
+// kDotTerms terms at a time.  All polynomials carry `l` limbs of the ciphertext chain.  Products
+// are summed as 30-bit-split Karatsuba partial sums (three widening multiply-adds each), reduced
+// every 8 products (the middle sums' bound).  Bound: HBM.  Where the outputs share their plaintexts the grid's
+// fastest axis runs over the outputs, so that CTAs which read the same operand run together and it
+// comes from HBM once: with the outputs on the slowest axis the 48 plaintexts of two sums at level 12
+// (302 MB, above L2) were read four times, 349 us.  Outputs with plaintexts of their own keep the slowest
+// axis: each streams through its own buffers.
+constexpr int kDotTerms = 64;
+
+struct Split2 {  // two adjacent residues as 30-bit halves and their sums
+    u32 x0, x1, x01, y0, y1, y01;
+};
+__device__ __forceinline__ Split2 split2(ulonglong2 v) {
+    Split2 s;
+    split30(v.x, s.x0, s.x1);
+    split30(v.y, s.y0, s.y1);
+    s.x01 = s.x0 + s.x1;
+    s.y01 = s.y0 + s.y1;
+    return s;
+}
+struct Acc3K2 {
+    Acc3K x, y;
+};
+__device__ __forceinline__ void acc2_mac(Acc3K2& A, const Split2& a, const Split2& b) {
+    acc3k_mac(A.x, a.x0, a.x1, a.x01, b.x0, b.x1, b.x01);
+    acc3k_mac(A.y, a.y0, a.y1, a.y01, b.y0, b.y1, b.y01);
+}
+// r += the sums (canonical residues); the sums start again from zero
+__device__ __forceinline__ void acc2_flush(Acc3K2& A, ulonglong2& r, const DPrime& P) {
+    const U128 vx = acc3_value(acc3k_fold(A.x)), vy = acc3_value(acc3k_fold(A.y));
+    r.x = addmod(r.x, barrett_reduce(vx.hi, vx.lo, P), P.q);
+    r.y = addmod(r.y, barrett_reduce(vy.hi, vy.lo, P), P.q);
+    A.x = A.y = {0, 0, 0};
+}
+
+// ciphertext x plaintext: out[p] = sum_k a[p K + k] * b[(shared ? 0 : p K) + k], one polynomial per thread: for
+// sums of up to 8 terms and launches too small for the paired form below (64 columns of one term at
+// level 3: 90 us, 129 us in that form's loop; one sum of 64 at level 2: 52 against 59 us).
+__global__ void __launch_bounds__(kEwThreads) k_dot(DevTables t, const u64* const* A, const u64* const* Bp,
+                                                    u64* const* O, int K, int b_shared, int l) {
     const int p = blockIdx.z, limb = blockIdx.y;
     if (limb >= l) return;
     const int x2 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -146,73 +183,143 @@ __global__ void k_dot(DevTables t, const u64* const* A, const u64* const* Bp, u6
     *reinterpret_cast<ulonglong2*>(O[p] + off) = r;
 }
 
+// The same, both polynomials of output p per thread (they share the plaintext's loads and halves).
+// Five CTAs of 128 threads per SM, four terms' loads of 48 bytes in flight per thread: 235 us (6.5
+// TB/s) for two sums of 48 at level 12; two CTAs of 256 threads 294 us.
+constexpr int kDotThreads = 128;
+__global__ void __launch_bounds__(kDotThreads, 5) k_dot_pair(DevTables t, const u64* const* A, const u64* const* Bp,
+                                                             u64* const* O, int K, int b_shared, int l) {
+    __shared__ const u64* sp[3][kDotTerms];
+    const int p = b_shared ? blockIdx.x : blockIdx.z, limb = b_shared ? blockIdx.z : blockIdx.y;
+    const int x2 = (b_shared ? blockIdx.y : blockIdx.x) * blockDim.x + threadIdx.x;
+    const bool in = 2 * x2 < t.n;
+    const DPrime P = load_prime(t.primes, limb);
+    const size_t off = ((size_t)limb << t.logn) + 2 * (size_t)x2;
+    const u64* const* A0 = A + (size_t)2 * p * K;
+    const u64* const* B0 = Bp + (b_shared ? 0 : (size_t)2 * p * K);
+    ulonglong2 r0 = make_ulonglong2(0, 0), r1 = r0;
+    for (int k0 = 0; k0 < K; k0 += kDotTerms) {
+        const int kn = K - k0 < kDotTerms ? K - k0 : kDotTerms;
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * kn; i += blockDim.x) {
+            const int w = i / kn, k = i % kn;
+            sp[w][k] = w == 0 ? A0[k0 + k] : w == 1 ? A0[K + k0 + k] : B0[k0 + k];
+        }
+        __syncthreads();
+        if (!in) continue;
+        Acc3K2 s0 = {{0, 0, 0}, {0, 0, 0}}, s1 = s0;
+        for (int k = 0; k < kn; k += 8) {
+#pragma unroll
+            for (int h = 0; h < 8; h += 4) {  // four terms' loads are in flight before the first is used
+                ulonglong2 v[4][3];
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (k + h + i < kn) {
+#pragma unroll
+                        for (int w = 0; w < 3; w++)
+                            v[i][w] = *reinterpret_cast<const ulonglong2*>(sp[w][k + h + i] + off);
+                    }
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (k + h + i < kn) {
+                        const Split2 c = split2(v[i][2]);
+                        acc2_mac(s0, split2(v[i][0]), c);
+                        acc2_mac(s1, split2(v[i][1]), c);
+                    }
+            }
+            acc2_flush(s0, r0, P);
+            acc2_flush(s1, r1, P);
+        }
+    }
+    if (!in) return;
+    *reinterpret_cast<ulonglong2*>(O[2 * p] + off) = r0;
+    *reinterpret_cast<ulonglong2*>(O[2 * p + 1] + off) = r1;
+}
+
 void ew_dot(const DevTables& t, const u64* const* A, const u64* const* B, u64* const* O, int n_out, int K,
             bool b_shared, int l, cudaStream_t st) {
     if (n_out == 0) return;
-    dim3 g((unsigned)((t.n / 2 + kEwThreads - 1) / kEwThreads), (unsigned)l, (unsigned)n_out);
+    const int sh = b_shared ? 1 : 0;
+    const unsigned b1 = (unsigned)((t.n / 2 + kEwThreads - 1) / kEwThreads), b2 = (unsigned)((t.n / 2 + kDotThreads - 1) / kDotThreads);
+    const unsigned outs = (unsigned)(n_out / 2);
     PFT_PROF("dot", st, (double)n_out * l * t.n * 8.0 * (2 * K + 1));
-    k_dot<<<g, kEwThreads, 0, st>>>(t, A, B, O, K, b_shared ? 1 : 0, l);
+    if (K > 8 && (double)outs * b2 * l >= 5 * 152)
+        k_dot_pair<<<b_shared ? dim3(outs, b2, (unsigned)l) : dim3(b2, (unsigned)l, outs), kDotThreads, 0, st>>>(t, A, B, O, K,
+                                                                                                          sh, l);
+    else
+        k_dot<<<dim3(b1, (unsigned)l, (unsigned)n_out), kEwThreads, 0, st>>>(t, A, B, O, K, sh, l);
     PFT_LAUNCH_CHECK("dot");
 }
 
-// ---- sums of HMUL tensors: out[p] (+)= sum_k a[p*K+k] (x) b[p*K+k] ---------------------------
+// ciphertext x ciphertext: out[p] (+)= sum_k a[p*K+k] (x) b[p*K+k], with
 // (a0, a1) (x) (b0, b1) = (a0 b0, a0 b1 + a1 b0, a1 b1).  Tables: A[(p*K + k)*2 + pol] and
 // B likewise point at polynomial bases (limb r at r*N, so operands of a higher level are
-// read through their leading limbs); O[p*3 + i] at the three output polynomials.  128-bit
-// sums reduced every 4 terms (8 products in the middle term).
-__global__ void k_tensor_dot(DevTables t, const u64* const* A, const u64* const* B, u64* const* O, int K, int l,
-                             int accumulate) {
-    const int p = blockIdx.z, limb = blockIdx.y;
-    if (limb >= l) return;
-    const int x2 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (2 * x2 >= t.n) return;
+// read through their leading limbs); O[p*3 + i] at the three output polynomials.  Reduced every 4
+// terms (8 products in the middle sum).  Five CTAs of 128 threads per SM: 1.44 ms for the five sums of a
+// training step of 4 documents at level 16 (three: 1.56; one thread's 128-bit sums in CTAs of 256: 1.66).
+__global__ void __launch_bounds__(kDotThreads, 5) k_tensor_dot(DevTables t, const u64* const* A, const u64* const* B,
+                                                           u64* const* O, int K, int l, int accumulate) {
+    __shared__ const u64* sp[4][kDotTerms];
+    const int p = blockIdx.x, limb = blockIdx.z;
+    const int x2 = blockIdx.y * blockDim.x + threadIdx.x;
+    const bool in = 2 * x2 < t.n;
     const DPrime P = load_prime(t.primes, limb);
     const size_t off = ((size_t)limb << t.logn) + 2 * (size_t)x2;
-    U128 s0x = {0, 0}, s0y = {0, 0}, s1x = {0, 0}, s1y = {0, 0}, s2x = {0, 0}, s2y = {0, 0};
-    for (int k = 0; k < K; k++) {
-        const size_t e = ((size_t)p * K + k) * 2;
-        const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(A[e] + off);
-        const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(A[e + 1] + off);
-        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(B[e] + off);
-        const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(B[e + 1] + off);
-        mac_wide(s0x, a0.x, b0.x);
-        mac_wide(s0y, a0.y, b0.y);
-        mac_wide(s1x, a0.x, b1.x);
-        mac_wide(s1x, a1.x, b0.x);
-        mac_wide(s1y, a0.y, b1.y);
-        mac_wide(s1y, a1.y, b0.y);
-        mac_wide(s2x, a1.x, b1.x);
-        mac_wide(s2y, a1.y, b1.y);
-        if ((k & 3) == 3) {
-            s0x = {barrett_reduce(s0x.hi, s0x.lo, P), 0};
-            s0y = {barrett_reduce(s0y.hi, s0y.lo, P), 0};
-            s1x = {barrett_reduce(s1x.hi, s1x.lo, P), 0};
-            s1y = {barrett_reduce(s1y.hi, s1y.lo, P), 0};
-            s2x = {barrett_reduce(s2x.hi, s2x.lo, P), 0};
-            s2y = {barrett_reduce(s2y.hi, s2y.lo, P), 0};
-        }
-    }
-    const U128* S[3][2] = {{&s0x, &s0y}, {&s1x, &s1y}, {&s2x, &s2y}};
+    ulonglong2 r[3];
+#pragma unroll
     for (int i = 0; i < 3; i++) {
-        ulonglong2 r;
-        r.x = barrett_reduce(S[i][0]->hi, S[i][0]->lo, P);
-        r.y = barrett_reduce(S[i][1]->hi, S[i][1]->lo, P);
-        u64* dst = O[(size_t)p * 3 + i] + off;
-        if (accumulate) {
-            const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(dst);
-            r.x = addmod(r.x, o.x, P.q);
-            r.y = addmod(r.y, o.y, P.q);
-        }
-        *reinterpret_cast<ulonglong2*>(dst) = r;
+        r[i] = make_ulonglong2(0, 0);
+        if (accumulate && in) r[i] = *reinterpret_cast<const ulonglong2*>(O[(size_t)p * 3 + i] + off);
     }
+    for (int k0 = 0; k0 < K; k0 += kDotTerms) {
+        const int kn = K - k0 < kDotTerms ? K - k0 : kDotTerms;
+        __syncthreads();
+        for (int i = threadIdx.x; i < 4 * kn; i += blockDim.x) {
+            const int w = i & 3, k = i >> 2;
+            const size_t e = ((size_t)p * K + k0 + k) * 2 + (w & 1);
+            sp[w][k] = w < 2 ? A[e] : B[e];
+        }
+        __syncthreads();
+        if (!in) continue;
+        Acc3K2 s0 = {{0, 0, 0}, {0, 0, 0}}, s1 = s0, s2 = s0;
+        for (int k = 0; k < kn; k += 4) {
+#pragma unroll
+            for (int h = 0; h < 4; h += 2) {
+                ulonglong2 v[2][4];
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+                    if (k + h + i < kn) {
+#pragma unroll
+                        for (int w = 0; w < 4; w++)
+                            v[i][w] = *reinterpret_cast<const ulonglong2*>(sp[w][k + h + i] + off);
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+                    if (k + h + i < kn) {
+                        const Split2 a0 = split2(v[i][0]), a1 = split2(v[i][1]), b0 = split2(v[i][2]),
+                                     b1 = split2(v[i][3]);
+                        acc2_mac(s0, a0, b0);
+                        acc2_mac(s1, a0, b1);
+                        acc2_mac(s1, a1, b0);
+                        acc2_mac(s2, a1, b1);
+                    }
+            }
+            acc2_flush(s0, r[0], P);
+            acc2_flush(s1, r[1], P);
+            acc2_flush(s2, r[2], P);
+        }
+    }
+    if (!in) return;
+#pragma unroll
+    for (int i = 0; i < 3; i++) *reinterpret_cast<ulonglong2*>(O[(size_t)p * 3 + i] + off) = r[i];
 }
 
 void ew_tensor_dot(const DevTables& t, const u64* const* A, const u64* const* B, u64* const* O, int n_out, int K,
                    int l, bool accumulate, cudaStream_t st) {
     if (n_out == 0) return;
-    dim3 g((unsigned)((t.n / 2 + kEwThreads - 1) / kEwThreads), (unsigned)l, (unsigned)n_out);
+    dim3 g((unsigned)n_out, (unsigned)((t.n / 2 + kDotThreads - 1) / kDotThreads), (unsigned)l);
     PFT_PROF("tensor_dot", st, (double)n_out * l * t.n * 8.0 * (4 * K + (accumulate ? 6 : 3)));
-    k_tensor_dot<<<g, kEwThreads, 0, st>>>(t, A, B, O, K, l, accumulate ? 1 : 0);
+    k_tensor_dot<<<g, kDotThreads, 0, st>>>(t, A, B, O, K, l, accumulate ? 1 : 0);
     PFT_LAUNCH_CHECK("tensor_dot");
 }
 
