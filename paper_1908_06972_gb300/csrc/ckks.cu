@@ -785,9 +785,10 @@ static void op_rotate_batch(pft_ctx* c, const pft_ct* const* a, int B, int32_t s
 // One form for all keys and rings: the automorphism is applied where the digits and c0 are read
 // (k_ks_inner_bulk, k_ntt_rows_epi), every stage is one launch over a tile of inputs and steps.
 // Tiles: inputs whose extended digits fit kHoistExtBytes; steps such that the products of the tile
-// fit kHoistTileBytes (launches of some hundred limbs already fill the GPU; one input and step are
-// 10 MiB at level 3 and 64 MiB at level 30), halved while the allocator refuses.
-constexpr size_t kHoistExtBytes = (size_t)2 << 30, kHoistTileBytes = (size_t)512 << 20;
+// fit kHoistTileBytes (one input and step are 10 MiB at level 3 and 64 MiB at level 30), halved while
+// the allocator refuses.  Tiles that stay in L2 lose more to the launches' tails than they save: 32
+// inferences at level 3 took 57.1 ms with tiles of 128 MiB, 51.9 with 256 MiB, 47.9 with 1 GiB, 47.9 with 2.
+constexpr size_t kHoistExtBytes = (size_t)2 << 30, kHoistTileBytes = (size_t)1 << 30;
 
 static void hoisted_tile(pft_ctx* c, const pft_ct* const* in, int B, const std::vector<u32>& gs,
                          const std::vector<std::vector<pft_ct*>>& outs) {

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
-    const int logn = SA + 8;
+    const int logn = t.logn;  // SA + 8; as a compile-time constant the passes ran 1 to 3 % slower (addressing)
     const int pi = prime_of(Ro, limb);
     const int cc = threadIdx.x % C, w = threadIdx.x / C;
     const int col = blockIdx.x * C + cc;
@@ -491,7 +491,8 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
 template <bool INV, int SA, int MT>
 __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     k_ntt_rows(DevTables t, PolySet in, PolySet out, int flags) {
-    constexpr int R = rows_per_cta(SA), TOP = SA + 7, logn = SA + 8;
+    constexpr int R = rows_per_cta(SA), TOP = SA + 7;
+    const int logn = t.logn;
     __shared__ u64 sm[R * kRowStride];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ro = out.p[poly];
@@ -544,10 +545,11 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
 // Forward row stages fused with the ModDown epilogue: for the canonical transform value v,
 // out = (x + c - v) s mod q (+ acc when the polynomial has one), with the polynomial's per-limb
 // constants {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of the column pass.
-template <int SA, int MT>
+template <int SA, int MT, bool PERM>
 __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     k_ntt_rows_epi(DevTables t, PolySet in, NttEpi e, int flags) {
-    constexpr int R = rows_per_cta(SA), NT = R * 16, logn = SA + 8;
+    constexpr int R = rows_per_cta(SA), NT = R * 16;
+    const int logn = t.logn;
     __shared__ u64 sm[R * kRowStride];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ri = in.p[poly];
@@ -556,7 +558,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     const size_t base = (size_t)limb << logn;
     const u64* __restrict__ xs = e.x[poly] + base;
     const u64* __restrict__ as = e.acc[poly];        // null: no accumulator for this polynomial
-    const u32 g = e.g[poly];                         // above 1: the accumulator is read through X -> X^g
+    const u32 g = PERM ? e.g[poly] : 0;              // above 1: the accumulator is read through X -> X^g
     u64* __restrict__ os = e.out[poly] + base;
     const u64* cs = e.consts[poly] + 3 * limb;
     if (flags & kPassPrefetch) {
@@ -582,8 +584,8 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
             const int f = 2 * (threadIdx.x + NT * (4 * h + i));
             const size_t j = ((size_t)(blockIdx.x * R) << 8) + f;
             xv[i] = *reinterpret_cast<const ulonglong2*>(xs + j);
-            if (as && g <= 1) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
-            if (as && g > 1)  // a row of 256 points reads one row of 256 sources: L1 holds it
+            if (as && (!PERM || g <= 1)) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
+            if (PERM && as && g > 1)  // a row of 256 points reads one row of 256 sources: L1 holds it
                 av[i] = make_ulonglong2(as[base + automorph_src((u32)j, logn, g)],
                                         as[base + automorph_src((u32)j + 1, logn, g)]);
         }
@@ -609,7 +611,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
 // that fits them, the rest L1.
 template <int SA, int MT>
 static void prepare_twopass(void) {
-    if (MT == 1024 && first_on_device((const void*)&k_ntt_rows_epi<SA, MT>)) {
+    if (MT == 1024 && first_on_device((const void*)&k_ntt_rows_epi<SA, MT, false>)) {
         const int co = 64;
         auto set = [&](auto k) { PFT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, co)); };
         set(k_ntt_cols<false, SA, MT>);
@@ -618,7 +620,8 @@ static void prepare_twopass(void) {
         set(k_ntt_cols<true, SA, MT, true>);
         set(k_ntt_rows<false, SA, MT>);
         set(k_ntt_rows<true, SA, MT>);
-        set(k_ntt_rows_epi<SA, MT>);
+        set(k_ntt_rows_epi<SA, MT, false>);
+        set(k_ntt_rows_epi<SA, MT, true>);
     }
 }
 // flags of the second pass of a transform over the same data
@@ -659,8 +662,11 @@ struct TwoPass {
         }
         // named apart from the plain transform launches: it also moves the epilogue's operands
         PFT_PROF("epi.ntt_moddown", st, work(t, io, 8));
-        k_ntt_rows_epi<SA, MT><<<row_grid(io), row_threads(SA), 0, st>>>(
-            t, io, e, second_pass(t, (t.ntt_order & 4) ? kPassPrefetch : 0));
+        const int flags = second_pass(t, (t.ntt_order & 4) ? kPassPrefetch : 0);
+        bool perm = false;
+        for (int i = 0; i < io.count; i++) perm |= e.g[i] > 1;
+        if (perm) k_ntt_rows_epi<SA, MT, true><<<row_grid(io), row_threads(SA), 0, st>>>(t, io, e, flags);
+        else k_ntt_rows_epi<SA, MT, false><<<row_grid(io), row_threads(SA), 0, st>>>(t, io, e, flags);
         PFT_LAUNCH_CHECK("ntt pass B + ModDown epilogue");
     }
     static void inverse(const DevTables& t, const PolySet& in, const PolySet& out, bool unscaled, cudaStream_t st) {
