@@ -50,6 +50,89 @@ bool handle_live(const void* h) {
     return pft::handles().count(h) != 0;
 }
 
+// ---- memory ---------------------------------------------------------------------------------
+static void* raw_alloc(pft_ctx* c, size_t bytes) {
+    void* p = nullptr;
+    if (c->has_alloc) return c->alloc.alloc(bytes, (void*)c->stream, c->alloc.user);
+    if (cudaMallocAsync(&p, bytes, c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+static void raw_free(pft_ctx* c, void* p) {
+    if (c->has_alloc) c->alloc.free(p, (void*)c->stream, c->alloc.user);
+    else cudaFreeAsync(p, c->stream);
+}
+static bool capturing(pft_ctx* c) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &s) != cudaSuccess) {
+        cudaGetLastError();  // the legacy default stream beside a capture elsewhere
+        return true;
+    }
+    return s != cudaStreamCaptureStatusNone;
+}
+void release_blocks(pft_ctx* c) {
+    std::deque<BlockCache::Block> out;
+    {
+        std::lock_guard<std::mutex> g(c->blocks.mu);
+        out.swap(c->blocks.kept);
+        c->blocks.kept_bytes = 0;
+    }
+    for (auto& b : out) raw_free(c, b.p);
+}
+void* dalloc(pft_ctx* c, size_t bytes) {
+    if (bytes == 0) return nullptr;
+    BlockCache& B = c->blocks;
+    const bool small = bytes <= BlockCache::kMaxBlock && !capturing(c);
+    if (small) {
+        // the newest kept block that fits without wasting more than a quarter of it
+        std::lock_guard<std::mutex> g(B.mu);
+        for (auto it = B.kept.rbegin(); it != B.kept.rend(); ++it)
+            if (it->bytes >= bytes && it->bytes - bytes <= it->bytes / 4) {
+                const BlockCache::Block b = *it;
+                B.kept.erase(std::next(it).base());
+                B.kept_bytes -= b.bytes;
+                B.live[b.p] = {b.bytes, c->stream};
+                return b.p;
+            }
+    }
+    void* p = raw_alloc(c, bytes);
+    if (!p) {
+        release_blocks(c);
+        p = raw_alloc(c, bytes);
+    }
+    if (!p) fail(PFT_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
+    if (small) {
+        std::lock_guard<std::mutex> g(B.mu);
+        B.live[p] = {bytes, c->stream};
+    }
+    return p;
+}
+void dfree(pft_ctx* c, void* p) {
+    if (!p) return;
+    BlockCache& B = c->blocks;
+    std::vector<void*> out;
+    {
+        const bool keep = !capturing(c);
+        std::lock_guard<std::mutex> g(B.mu);
+        auto it = B.live.find(p);
+        if (it == B.live.end() || !keep || it->second.second != c->stream) {
+            out.push_back(p);
+        } else {
+            B.kept.push_back({p, it->second.first});
+            B.kept_bytes += it->second.first;
+            while (B.kept_bytes > BlockCache::kMaxCached) {
+                out.push_back(B.kept.front().p);
+                B.kept_bytes -= B.kept.front().bytes;
+                B.kept.pop_front();
+            }
+        }
+        if (it != B.live.end()) B.live.erase(it);
+    }
+    for (void* q : out) raw_free(c, q);
+}
+
 // ---- context construction ---------------------------------------------------------------
 static u64 shoup(u64 w, u64 q) { return (u64)(((unsigned __int128)w << 64) / q); }
 // basis-conversion constants are stored in Montgomery form c 2^64 mod t, split as
@@ -1758,6 +1841,7 @@ int pft_ctx_destroy(pft_ctx* c) {
     free_keys(c);
     dfree(c, c->s_ntt);
     dfree(c, c->pk);
+    release_blocks(c);
     cudaStreamSynchronize(c->stream);
     for (void* p : c->owned) cudaFree(p);
     delete c;
@@ -1766,6 +1850,7 @@ int pft_ctx_destroy(pft_ctx* c) {
 
 int pft_set_stream(pft_ctx* c, void* stream) {
     if (!c) return PFT_ERR_ARG;
+    if (c->stream != (cudaStream_t)stream) release_blocks(c);  // kept blocks belong to the old stream
     c->stream = (cudaStream_t)stream;
     return PFT_OK;
 }

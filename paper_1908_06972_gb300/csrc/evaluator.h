@@ -1,9 +1,12 @@
 // Handles of the evaluator and the host-side helpers shared by its translation units
 // (the operations in ckks.cu, the request server in serve.cu).
 #pragma once
+#include <deque>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "pft_internal.h"
@@ -14,6 +17,26 @@ using namespace pft;
     do {                      \
         if (!(cond)) fail(code, msg); \
     } while (0)
+
+// Freed device blocks that a context keeps for its next calls.  A call of a small ring allocates and
+// frees about ten short-lived blocks; through a caller's allocator (a callback into Python for
+// torch's) these cost more than its kernels.  Bounded: blocks up to kMaxBlock, kMaxCached bytes in all,
+// the oldest given back first; all are given back when the allocator refuses a request, when the
+// context's stream changes and when the context is destroyed.  Stream order makes reuse safe as it
+// does for the allocators: a block is kept only if it was allocated and freed on the stream that is
+// current, and never while that stream is being captured (a graph's memory must stay its own).
+// Callers may destroy handles from other threads, so the lists have a lock.
+struct BlockCache {
+    static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)128 << 20;
+    struct Block {
+        void* p;
+        size_t bytes;
+    };
+    std::mutex mu;
+    std::unordered_map<void*, std::pair<size_t, cudaStream_t>> live;  // blocks up to kMaxBlock in use
+    std::deque<Block> kept;                                           // oldest first
+    size_t kept_bytes = 0;
+};
 
 // ---- handles ---------------------------------------------------------------------------
 struct pft_ctx {
@@ -26,6 +49,7 @@ struct pft_ctx {
     pft_allocator alloc{};
     bool has_alloc = false;
     cudaStream_t stream = nullptr;
+    BlockCache blocks;
     std::string err;
     DevTables tabs{};
     std::vector<void*> owned;  // table buffers
@@ -92,23 +116,11 @@ struct pft_ft_model {
 };
 
 // ---- memory --------------------------------------------------------------------------
-inline void* dalloc(pft_ctx* c, size_t bytes) {
-    if (bytes == 0) return nullptr;
-    void* p = nullptr;
-    if (c->has_alloc) {
-        p = c->alloc.alloc(bytes, (void*)c->stream, c->alloc.user);
-    } else {
-        cudaError_t e = cudaMallocAsync(&p, bytes, c->stream);
-        if (e != cudaSuccess) p = nullptr;
-    }
-    if (!p) fail(PFT_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
-    return p;
-}
-inline void dfree(pft_ctx* c, void* p) {
-    if (!p) return;
-    if (c->has_alloc) c->alloc.free(p, (void*)c->stream, c->alloc.user);
-    else cudaFreeAsync(p, c->stream);
-}
+// Device memory on the context's stream: from the context's kept blocks, else from the allocator.
+void* dalloc(pft_ctx* c, size_t bytes);
+void dfree(pft_ctx* c, void* p);
+// Gives every kept block back to the allocator.
+void release_blocks(pft_ctx* c);
 struct Scratch {
     pft_ctx* c;
     void* p;
