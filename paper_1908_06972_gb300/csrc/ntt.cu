@@ -155,12 +155,15 @@ __device__ __forceinline__ int pass_limb(int flags) {
 // the k-th of these stages at lm[16 (2^k - 1 + j)], loaded under the L2 policy pol.
 // RT (the row round W0 = 4, thread = row r): the row's 15 twiddles of its first four stages
 // were copied to shared memory, the k-th stage's entry j at rt[2^k - 1 + j].
+// PRE: the round's twiddles were loaded into registers before (load_round), slot 2^(3-lb) - 1 + i for
+// the i-th group of register bit lb.
 template <bool INV, int W0, int TOP, int NB = 4, bool LAZY = false, bool UNSCALED = false, bool LM = false,
-          bool RT = false>
+          bool RT = false, bool PRE = false>
 __device__ __forceinline__ void ntt_round(u64 (&x)[16], int wpart, int r, const ulonglong2* __restrict__ tw, u64 q,
                                           u64 q2, ulonglong2 NI, ulonglong2 NI1,
                                           const ulonglong2* __restrict__ lm = nullptr,
-                                          const ulonglong2* rt = nullptr, u64 pol = 0) {
+                                          const ulonglong2* rt = nullptr, u64 pol = 0,
+                                          const ulonglong2* pre = nullptr) {
     static_assert(!LM || W0 == 0, "lane-major twiddles serve the row round of the last four stages");
     static_assert(!RT || W0 == 4, "staged row twiddles serve the first row round");
 #pragma unroll
@@ -173,7 +176,8 @@ __device__ __forceinline__ void ntt_round(u64 (&x)[16], int wpart, int r, const 
             if (e & (1 << lb)) continue;
             const int elem = (e << W0) | wpart;
             const int idx = (1 << s) + (r << (7 - p)) + (elem >> (p + 1));
-            const ulonglong2 W = LM   ? ldg_pol(&lm[16 * ((1 << (3 - p)) - 1 + (e >> (p + 1)))], pol)
+            const ulonglong2 W = PRE  ? pre[(1 << (3 - lb)) - 1 + (e >> (lb + 1))]
+                                 : LM ? ldg_pol(&lm[16 * ((1 << (3 - p)) - 1 + (e >> (p + 1)))], pol)
                                  : RT ? rt[(1 << (7 - p)) - 1 + (elem >> (p + 1))]
                                       : __ldg(&tw[idx]);
             if (!INV) {
@@ -191,6 +195,27 @@ __device__ __forceinline__ void ntt_round(u64 (&x)[16], int wpart, int r, const 
     }
 }
 
+
+// the same, issued where it stands (the compiler may move the plain form to the first use)
+__device__ __forceinline__ ulonglong2 ldg_now(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+// The twiddles of one round of ntt_round into registers: from the natural table, or from the lane-major copy (LM).
+template <int W0, int TOP, int NB = 4, bool LM = false>
+__device__ __forceinline__ void load_round(ulonglong2 (&W)[15], int wpart, int r, const ulonglong2* __restrict__ tw) {
+#pragma unroll
+    for (int lb = NB - 1; lb >= 0; lb--) {
+        const int p = W0 + lb, s = TOP - p;
+#pragma unroll
+        for (int i = 0; i < 8 >> lb; i++) {
+            const int slot = (1 << (3 - lb)) - 1 + i;
+            const int elem = (i << (lb + 1 + W0)) | wpart;
+            W[slot] = ldg_now(LM ? &tw[16 * slot] : &tw[(1 << s) + (r << (7 - p)) + (elem >> (p + 1))]);
+        }
+    }
+}
 
 constexpr int kN16Stride = 33;  // shared layout [256][33]: element (a, lane) at a * 33 + lane
 
@@ -321,7 +346,11 @@ __host__ __device__ constexpr int rows_per_cta(int SA) { return SA >= 7 ? 16 : S
 __host__ __device__ constexpr int col_threads(int SA) { return cols_per_cta(SA) << (SA - 4); }
 __host__ __device__ constexpr int row_threads(int SA) { return rows_per_cta(SA) * 16; }
 
-// MT: resident threads per SM the registers are bounded for (768: 80 registers, 1024: 64).
+// MT: resident threads per SM the registers are bounded for (768: 80 registers, 1024: 64), or 0 for
+// launches that fit the GPU at once (kPreThreadsPerSm): then one CTA's latency is the launch's time,
+// registers are plenty, and every twiddle is loaded at the start (the fused pass's operands with the data),
+// so that the stages wait for memory once: one HMUL + rescale at N = 2^13 100 -> 88 us.
+__host__ __device__ constexpr int min_ctas(int MT, int threads) { return MT == 0 ? 1 : MT / threads; }
 // UNSCALED (inverse): the last stage is a plain Gentleman-Sande butterfly (no N^-1) and the
 // output stays in [0, 4q): N times the inverse transform, for a consumer that scales anyway.
 // BCAST (forward): RESCALE's broadcast on the way in.  `in` holds one limb per polynomial, c_{l-1} in
@@ -329,9 +358,10 @@ __host__ __device__ constexpr int row_threads(int SA) { return rows_per_cta(SA) 
 // (r - h) mod q_k with r = (c_{l-1} + h) mod p, h = floor(p/2).  A pass of its own for it (k_rescale_bcast)
 // took 17 % of a batch of rescales: it writes and the column pass reads back every limb.
 template <bool INV, int SA, int MT, bool UNSCALED = false, bool BCAST = false>
-__global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
+__global__ void __launch_bounds__(col_threads(SA), min_ctas(MT, col_threads(SA)))
     k_ntt_cols(DevTables t, PolySet in, PolySet out, int flags) {
     constexpr int C = cols_per_cta(SA), LO = SA - 4;     // LO: bits of the second round
+    constexpr bool PRE = MT == 0;
     constexpr int ST = C == 16 ? 17 : C;
     __shared__ u64 sm[SA > 4 ? (1 << SA) * ST : 1];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
@@ -349,6 +379,12 @@ __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
     const ulonglong2 NI = INV ? __ldg(&t.ninv[pi]) : make_ulonglong2(0, 0);
     const ulonglong2 NI1 = INV ? __ldg(&t.inv1ninv[pi]) : make_ulonglong2(0, 0);
     u64 x[16];
+    ulonglong2 w1[15], w2[15];  // PRE: the twiddles of the rounds on bits LO.. and on the low bits
+    if (PRE) {
+        load_round<LO, SA - 1>(w1, w, 0, tw);
+        if (SA > 4) load_round<0, SA - 1, LO>(w2, w << 4, 0, tw);
+    }
+    pdl_wait();
     if (!INV) {
         const bool lazy = q < kLazyBound;  // uniform over the CTA (one limb)
         if constexpr (BCAST) {
@@ -368,16 +404,16 @@ __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
 #pragma unroll
             for (int e = 0; e < 16; e++) x[e] = src[(size_t)((e << LO) | w) << 8];
         }
-        if (lazy) ntt_round<false, LO, SA - 1, 4, true>(x, w, 0, tw, q, q2, NI, NI1);
-        else ntt_round<false, LO, SA - 1>(x, w, 0, tw, q, q2, NI, NI1);
+        if (lazy) ntt_round<false, LO, SA - 1, 4, true, false, false, false, PRE>(x, w, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
+        else ntt_round<false, LO, SA - 1, 4, false, false, false, false, PRE>(x, w, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
         if constexpr (SA > 4) {
 #pragma unroll
             for (int e = 0; e < 16; e++) sm[((e << LO) | w) * ST + cc] = x[e];
             __syncthreads();
 #pragma unroll
             for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + cc];
-            if (lazy) ntt_round<false, 0, SA - 1, LO, true>(x, w << 4, 0, tw, q, q2, NI, NI1);
-            else ntt_round<false, 0, SA - 1, LO>(x, w << 4, 0, tw, q, q2, NI, NI1);
+            if (lazy) ntt_round<false, 0, SA - 1, LO, true, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
+            else ntt_round<false, 0, SA - 1, LO, false, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
         }
 #pragma unroll
         for (int e = 0; e < 16; e++) dst[(size_t)((w << 4) | e) << 8] = x[e];
@@ -385,14 +421,14 @@ __global__ void __launch_bounds__(col_threads(SA), MT / col_threads(SA))
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = src[(size_t)((w << 4) | e) << 8];
         if constexpr (SA > 4) {
-            ntt_round<true, 0, SA - 1, LO>(x, w << 4, 0, tw, q, q2, NI, NI1);
+            ntt_round<true, 0, SA - 1, LO, false, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
 #pragma unroll
             for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + cc] = x[e];
             __syncthreads();
 #pragma unroll
             for (int e = 0; e < 16; e++) x[e] = sm[((e << LO) | w) * ST + cc];
         }
-        ntt_round<true, LO, SA - 1, 4, false, UNSCALED>(x, w, 0, tw, q, q2, NI, NI1);
+        ntt_round<true, LO, SA - 1, 4, false, UNSCALED, false, false, PRE>(x, w, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
 #pragma unroll
         for (int e = 0; e < 16; e++)
             dst[(size_t)((e << LO) | w) << 8] = (flags & kPassFinal) && !UNSCALED ? canon4(x[e], q, q2) : x[e];
@@ -439,7 +475,7 @@ __device__ __forceinline__ const ulonglong2* lm_base(const ulonglong2* rows, int
 // Forward stages SA..SA+7 of the rows of this CTA (limb `limb` of prime pi, rows read from
 // src): canonical results are left in sm, row c2 point m at c2 * kRowStride + m + (m >> 4),
 // after a barrier.
-template <int SA>
+template <int SA, bool PRE, bool WAIT>
 __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restrict__ src, int pi, u64* sm) {
     constexpr int R = rows_per_cta(SA), TOP = SA + 7;
     const int w = threadIdx.x & 15, cc = threadIdx.x >> 4;
@@ -450,23 +486,30 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
     const ulonglong2 NI = make_ulonglong2(0, 0);
     const ulonglong2* lm = lm_base<SA>(t.fwd_rows, pi, u, w);
     const u64 pol = tw_policy(t.ntt_order & 2);
-    __shared__ ulonglong2 rt[R * 15];  // twiddles of the first four row stages
+    __shared__ ulonglong2 rt[PRE ? 1 : R * 15];  // twiddles of the first four row stages
     u64* my = sm + cc * kRowStride;
     u64 x[16];
+    ulonglong2 w1[15], w2[15];
     const bool lazy = q < kLazyBound;  // uniform over the CTA (one limb)
-    stage_row_round1<SA>(tw, blockIdx.x * R, rt, pol);
+    if (PRE) {
+        load_round<4, TOP>(w1, w, u, tw);
+        load_round<0, TOP, 4, true>(w2, 0, 0, lm);
+    } else {
+        stage_row_round1<SA>(tw, blockIdx.x * R, rt, pol);
+    }
+    if (WAIT) pdl_wait();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = src[((size_t)u << 8) | (e << 4) | w];
-    __syncthreads();
-    if (lazy) ntt_round<false, 4, TOP, 4, true, false, false, true>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
-    else ntt_round<false, 4, TOP, 4, false, false, false, true>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15);
+    if (!PRE) __syncthreads();
+    if (lazy) ntt_round<false, 4, TOP, 4, true, false, false, !PRE, PRE>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15, 0, w1);
+    else ntt_round<false, 4, TOP, 4, false, false, false, !PRE, PRE>(x, w, u, tw, q, q2, NI, NI, nullptr, rt + cc * 15, 0, w1);
 #pragma unroll
     for (int e = 0; e < 16; e++) my[e * 17 + w] = x[e];  // point e*16 + w
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[w * 17 + e];  // point w*16 + e
     if (lazy) {
-        ntt_round<false, 0, TOP, 4, true, false, true>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
+        ntt_round<false, 0, TOP, 4, true, false, !PRE, false, PRE>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol, w2);
         const u32 ps = __ldg(&t.primes[pi].s);
         if (ps >= 24) {
             const u32 r = (u32)(__ldg(&t.primes[pi].mu) >> 32);
@@ -481,7 +524,7 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
             }
         }
     } else {
-        ntt_round<false, 0, TOP, 4, false, false, true>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol);
+        ntt_round<false, 0, TOP, 4, false, false, !PRE, false, PRE>(x, w << 4, u, tw, q, q2, NI, NI, lm, nullptr, pol, w2);
 #pragma unroll
         for (int e = 0; e < 16; e++) my[w * 17 + e] = canon8(x[e], q, q2);
     }
@@ -489,7 +532,7 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
 }
 
 template <bool INV, int SA, int MT>
-__global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
+__global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA)))
     k_ntt_rows(DevTables t, PolySet in, PolySet out, int flags) {
     constexpr int R = rows_per_cta(SA), TOP = SA + 7;
     const int logn = t.logn;
@@ -501,7 +544,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     const u64* src = in.p[poly].ptr + ((size_t)limb << logn);
     u64* dst = Ro.ptr + ((size_t)limb << logn);
     if (!INV) {
-        fwd_rows<SA>(t, src, pi, sm);
+        fwd_rows<SA, MT == 0, true>(t, src, pi, sm);
 #pragma unroll
         for (int k = 0; k < 16; k++) {
             const int f = threadIdx.x + R * 16 * k;
@@ -521,6 +564,13 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     const u64 pol = tw_policy(t.ntt_order & 2);
     u64* my = sm + cc * kRowStride;
     u64 x[16];
+    ulonglong2 w1[15], w2[15];
+    constexpr bool PRE = MT == 0;
+    if (PRE) {
+        load_round<0, TOP, 4, true>(w2, 0, 0, lm);
+        load_round<4, TOP>(w1, w, u, tw);
+    }
+    pdl_wait();
 #pragma unroll
     for (int k = 0; k < 16; k++) {
         const int f = threadIdx.x + R * 16 * k;
@@ -530,13 +580,13 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[w * 17 + e];  // point w*16 + e
-    ntt_round<true, 0, TOP, 4, false, false, true>(x, w << 4, u, tw, q, q2, NI, NI1, lm, nullptr, pol);
+    ntt_round<true, 0, TOP, 4, false, false, !PRE, false, PRE>(x, w << 4, u, tw, q, q2, NI, NI1, lm, nullptr, pol, w2);
 #pragma unroll
     for (int e = 0; e < 16; e++) my[w * 17 + e] = x[e];
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = my[e * 17 + w];  // point e*16 + w
-    ntt_round<true, 4, TOP>(x, w, u, tw, q, q2, NI, NI1);
+    ntt_round<true, 4, TOP, 4, false, false, false, false, PRE>(x, w, u, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
 #pragma unroll
     for (int e = 0; e < 16; e++)
         dst[((size_t)u << 8) | (e << 4) | w] = (flags & kPassFinal) ? canon4(x[e], q, q2) : x[e];
@@ -546,9 +596,10 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
 // out = (x + c - v) s mod q (+ acc when the polynomial has one), with the polynomial's per-limb
 // constants {c, s, s'} (Shoup) at consts[3 limb].  The rows of `in` hold the output of the column pass.
 template <int SA, int MT, bool PERM>
-__global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
+__global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA)))
     k_ntt_rows_epi(DevTables t, PolySet in, NttEpi e, int flags) {
     constexpr int R = rows_per_cta(SA), NT = R * 16;
+    constexpr bool PRE = MT == 0;
     const int logn = t.logn;
     __shared__ u64 sm[R * kRowStride];
     const int poly = pass_poly(flags), limb = pass_limb(flags);
@@ -561,6 +612,7 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
     const u32 g = PERM ? e.g[poly] : 0;              // above 1: the accumulator is read through X -> X^g
     u64* __restrict__ os = e.out[poly] + base;
     const u64* cs = e.consts[poly] + 3 * limb;
+    if (PRE || (flags & kPassPrefetch)) pdl_wait();
     if (flags & kPassPrefetch) {
         // ask L2 for this CTA's tile of the epilogue operands (one 128-byte line per thread and
         // operand: R rows x 256 words) so that their DRAM reads overlap the transform
@@ -569,25 +621,38 @@ __global__ void __launch_bounds__(row_threads(SA), MT / row_threads(SA))
         asm volatile("prefetch.global.L2 [%0];" ::"l"(xs + j));
         if (as) asm volatile("prefetch.global.L2 [%0];" ::"l"(as + base + j));
     }
-    fwd_rows<SA>(t, Ri.ptr + base, pi, sm);
+    // each thread: two adjacent points (16-byte loads and stores) of eight rows or row parts
+    auto load = [&](int i, ulonglong2& xv, ulonglong2& av) {
+        const size_t j = ((size_t)(blockIdx.x * R) << 8) + 2 * (threadIdx.x + NT * i);
+        xv = *reinterpret_cast<const ulonglong2*>(xs + j);
+        if (as && (!PERM || g <= 1)) av = *reinterpret_cast<const ulonglong2*>(as + base + j);
+        if (PERM && as && g > 1)  // a row of 256 points reads one row of 256 sources: L1 holds it
+            av = make_ulonglong2(as[base + automorph_src((u32)j, logn, g)],
+                                 as[base + automorph_src((u32)j + 1, logn, g)]);
+    };
+    ulonglong2 xp[PRE ? 8 : 1], ap[PRE ? 8 : 1];
+    if (PRE) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) load(i, xp[PRE ? i : 0], ap[PRE ? i : 0]);
+    }
+    if (flags & kPassPrefetch) fwd_rows<SA, PRE, false>(t, Ri.ptr + base, pi, sm);
+    else fwd_rows<SA, PRE, !PRE>(t, Ri.ptr + base, pi, sm);
     const u64 q = __ldg(&t.primes[pi].q);
     const u64 c = __ldg(&cs[0]), s = __ldg(&cs[1]), sp = __ldg(&cs[2]);
-    // each thread: two adjacent points (16-byte loads and stores) of eight rows or row parts; the
-    // operands of four are loaded before any is used, so that more bytes are in flight (the
-    // transform's registers are free by now).  An even point m and m + 1 share their 16-point
+    // (not PRE) the operands of four are loaded before any is used, so that more bytes are in flight
+    // (the transform's registers are free by now).  An even point m and m + 1 share their 16-point
     // group, so their transform values are adjacent in shared memory.
 #pragma unroll
     for (int h = 0; h < 2; h++) {
         ulonglong2 xv[4], av[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-            const int f = 2 * (threadIdx.x + NT * (4 * h + i));
-            const size_t j = ((size_t)(blockIdx.x * R) << 8) + f;
-            xv[i] = *reinterpret_cast<const ulonglong2*>(xs + j);
-            if (as && (!PERM || g <= 1)) av[i] = *reinterpret_cast<const ulonglong2*>(as + base + j);
-            if (PERM && as && g > 1)  // a row of 256 points reads one row of 256 sources: L1 holds it
-                av[i] = make_ulonglong2(as[base + automorph_src((u32)j, logn, g)],
-                                        as[base + automorph_src((u32)j + 1, logn, g)]);
+            if (PRE) {
+                xv[i] = xp[PRE ? 4 * h + i : 0];
+                av[i] = ap[PRE ? 4 * h + i : 0];
+            } else {
+                load(4 * h + i, xv[i], av[i]);
+            }
         }
 #pragma unroll
         for (int i = 0; i < 4; i++) {
@@ -641,13 +706,13 @@ struct TwoPass {
     static void cols_fwd(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
         prepare_twopass<SA, MT>();
         PFT_PROF("ntt.fwd.strided", st, work(t, out, SA));
-        k_ntt_cols<false, SA, MT><<<col_grid(out), col_threads(SA), 0, st>>>(t, in, out, 0);
+        launch_pdl(k_ntt_cols<false, SA, MT>, col_grid(out), col_threads(SA), 0, st, t, in, out, 0);
         PFT_LAUNCH_CHECK("ntt pass A");
     }
     static void forward(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
         cols_fwd(t, in, out, st);
         PFT_PROF("ntt.fwd.contig", st, work(t, out, 8));
-        k_ntt_rows<false, SA, MT><<<row_grid(out), row_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
+        launch_pdl(k_ntt_rows<false, SA, MT>, row_grid(out), row_threads(SA), 0, st, t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("ntt pass B");
     }
     static void forward_epi(const DevTables& t, const PolySet& in, const PolySet& io, const NttEpi& e, bool bcast,
@@ -655,7 +720,7 @@ struct TwoPass {
         if (bcast) {
             prepare_twopass<SA, MT>();
             PFT_PROF("ntt.fwd.strided", st, work(t, io, SA));
-            k_ntt_cols<false, SA, MT, false, true><<<col_grid(io), col_threads(SA), 0, st>>>(t, in, io, 0);
+            launch_pdl(k_ntt_cols<false, SA, MT, false, true>, col_grid(io), col_threads(SA), 0, st, t, in, io, 0);
             PFT_LAUNCH_CHECK("rescale broadcast + ntt pass A");
         } else {
             cols_fwd(t, in, io, st);
@@ -665,42 +730,45 @@ struct TwoPass {
         const int flags = second_pass(t, (t.ntt_order & 4) ? kPassPrefetch : 0);
         bool perm = false;
         for (int i = 0; i < io.count; i++) perm |= e.g[i] > 1;
-        if (perm) k_ntt_rows_epi<SA, MT, true><<<row_grid(io), row_threads(SA), 0, st>>>(t, io, e, flags);
-        else k_ntt_rows_epi<SA, MT, false><<<row_grid(io), row_threads(SA), 0, st>>>(t, io, e, flags);
+        if (perm) launch_pdl(k_ntt_rows_epi<SA, MT, true>, row_grid(io), row_threads(SA), 0, st, t, io, e, flags);
+        else launch_pdl(k_ntt_rows_epi<SA, MT, false>, row_grid(io), row_threads(SA), 0, st, t, io, e, flags);
         PFT_LAUNCH_CHECK("ntt pass B + ModDown epilogue");
     }
     static void inverse(const DevTables& t, const PolySet& in, const PolySet& out, bool unscaled, cudaStream_t st) {
         prepare_twopass<SA, MT>();
         {
             PFT_PROF("ntt.inv.contig", st, work(t, out, 8));
-            k_ntt_rows<true, SA, MT><<<row_grid(out), row_threads(SA), 0, st>>>(t, in, out, 0);
+            launch_pdl(k_ntt_rows<true, SA, MT>, row_grid(out), row_threads(SA), 0, st, t, in, out, 0);
         }
         PFT_LAUNCH_CHECK("intt pass B");
         PFT_PROF("ntt.inv.strided", st, work(t, out, SA));
         if (unscaled)
-            k_ntt_cols<true, SA, MT, true>
-                <<<col_grid(out), col_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
+            launch_pdl(k_ntt_cols<true, SA, MT, true>, col_grid(out), col_threads(SA), 0, st, t, out, out, second_pass(t, kPassFinal));
         else
-            k_ntt_cols<true, SA, MT><<<col_grid(out), col_threads(SA), 0, st>>>(t, out, out, second_pass(t, kPassFinal));
+            launch_pdl(k_ntt_cols<true, SA, MT>, col_grid(out), col_threads(SA), 0, st, t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("intt pass A");
     }
 };
-// f(TwoPass<..>) for the ring's shape; v: 0 = bounded for 768 resident threads per SM (3 CTAs of 256),
-// 1 = for 1024 (4 CTAs; N = 2^16 and 2^15)
+// A launch with at most this many threads per SM takes the form with everything loaded at the start (its 100
+// to 255 registers leave room for about that many; 256, 512 and 1024 measured within 2 % of each
+// other, none at all 10 % slower for small rings).
+static constexpr int kPreThreadsPerSm = 512;
+// f(TwoPass<..>) for the ring's shape and the launch's limbs; v: 0 = bounded for 768 resident threads per
+// SM (3 CTAs of 256), 1 = for 1024 (4 CTAs; N = 2^16 and 2^15)
+template <int SA, class F>
+static void with_twopass_sa(double limbs, int v, F f) {
+    if (limbs * (1 << SA) * 16 <= 152.0 * kPreThreadsPerSm) f(TwoPass<SA, 0>());
+    else if (SA >= 7 && v == 1) f(TwoPass<SA, SA >= 7 ? 1024 : 768>());
+    else f(TwoPass<SA, 768>());
+}
 template <class F>
-static void with_twopass(const DevTables& t, int v, F f) {
+static void with_twopass(const DevTables& t, int v, double limbs, F f) {
     switch (t.logn) {
-        case 12: f(TwoPass<4, 768>()); break;
-        case 13: f(TwoPass<5, 768>()); break;
-        case 14: f(TwoPass<6, 768>()); break;
-        case 15:
-            if (v == 1) f(TwoPass<7, 1024>());
-            else f(TwoPass<7, 768>());
-            break;
-        case 16:
-            if (v == 1) f(TwoPass<8, 1024>());
-            else f(TwoPass<8, 768>());
-            break;
+        case 12: with_twopass_sa<4>(limbs, v, f); break;
+        case 13: with_twopass_sa<5>(limbs, v, f); break;
+        case 14: with_twopass_sa<6>(limbs, v, f); break;
+        case 15: with_twopass_sa<7>(limbs, v, f); break;
+        case 16: with_twopass_sa<8>(limbs, v, f); break;
         default: fail(PFT_ERR_ARG, "internal: no two-pass transform for this ring degree");
     }
 }
@@ -983,7 +1051,7 @@ static void run(const DevTables& t, const PolySet& in, const PolySet& out, bool 
     if (out.count == 0) return;
     const int fam = ntt_family(t, set_limbs(out));
     if (fam <= 1) {
-        with_twopass(t, fam, [&](auto tp) {
+        with_twopass(t, fam, set_limbs(out), [&](auto tp) {
             if (inverse) tp.inverse(t, in, out, false, st);
             else tp.forward(t, in, out, st);
         });
@@ -1120,7 +1188,7 @@ bool ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& 
     if (out.count == 0) return true;
     const int fam = ntt_family(t, set_limbs(out));
     if (fam > 1) return false;
-    with_twopass(t, fam, [&](auto tp) { tp.inverse(t, in, out, true, st); });
+    with_twopass(t, fam, set_limbs(out), [&](auto tp) { tp.inverse(t, in, out, true, st); });
     return true;
 }
 
@@ -1133,7 +1201,7 @@ bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e
     if (io.count == 0) return true;
     const int fam = ntt_family(t, set_limbs(io));
     if (fam > 1) return false;
-    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, io, io, e, false, st); });
+    with_twopass(t, fam, set_limbs(io), [&](auto tp) { tp.forward_epi(t, io, io, e, false, st); });
     return true;
 }
 bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e,
@@ -1141,7 +1209,7 @@ bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet
     if (io.count == 0) return true;
     const int fam = ntt_family(t, set_limbs(io));
     if (fam > 1) return false;
-    with_twopass(t, fam, [&](auto tp) { tp.forward_epi(t, last, io, e, true, st); });
+    with_twopass(t, fam, set_limbs(io), [&](auto tp) { tp.forward_epi(t, last, io, e, true, st); });
     return true;
 }
 void ntt_inverse(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {

@@ -128,6 +128,24 @@ inline double set_limbs(const PolySet& s) {
     return t;
 }
 
+// Launch of a kernel that begins with pdl_wait (modarith.cuh): it may become resident before the kernel
+// ahead of it on the stream has finished, which hides its launch and its table loads.  Kernels and
+// copies launched in the ordinary way keep waiting for everything before them.
+template <class... P, class... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    check_cuda(cudaLaunchKernelEx(&cfg, kernel, args...), "kernel launch");
+}
+
 // ---- kernels (launchers) ------------------------------------------------------------
 // Negacyclic transform of every limb of every polynomial of `out` (input from `in`,
 // which may be the same set).

@@ -30,6 +30,7 @@ static dim3 ew_grid(int n, const PolySet& s) {
 // ---- HADD / sub / pointwise product / negate / copy --------------------------------------
 template <int OP>
 __global__ void k_ew_binary(DevTables t, PolySet a, PolySet b, PolySet out) {
+    pdl_wait();
     const int poly = blockIdx.z, limb = blockIdx.y;
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
@@ -66,11 +67,11 @@ void ew_binary(const DevTables& t, EwOp op, const PolySet& a, const PolySet& b, 
     PFT_PROF(op == EwOp::Mul ? "ew.mul" : (op == EwOp::Copy ? "ew.copy" : "ew.add"), st,
              set_limbs(out) * t.n * 8.0 * (op == EwOp::Copy || op == EwOp::Neg ? 2 : 3));
     switch (op) {
-        case EwOp::Add: k_ew_binary<0><<<g, kEwThreads, 0, st>>>(t, a, b, out); break;
-        case EwOp::Sub: k_ew_binary<1><<<g, kEwThreads, 0, st>>>(t, a, b, out); break;
-        case EwOp::Mul: k_ew_binary<2><<<g, kEwThreads, 0, st>>>(t, a, b, out); break;
-        case EwOp::Neg: k_ew_binary<3><<<g, kEwThreads, 0, st>>>(t, a, b, out); break;
-        case EwOp::Copy: k_ew_binary<4><<<g, kEwThreads, 0, st>>>(t, a, b, out); break;
+        case EwOp::Add: launch_pdl(k_ew_binary<0>, g, kEwThreads, 0, st, t, a, b, out); break;
+        case EwOp::Sub: launch_pdl(k_ew_binary<1>, g, kEwThreads, 0, st, t, a, b, out); break;
+        case EwOp::Mul: launch_pdl(k_ew_binary<2>, g, kEwThreads, 0, st, t, a, b, out); break;
+        case EwOp::Neg: launch_pdl(k_ew_binary<3>, g, kEwThreads, 0, st, t, a, b, out); break;
+        case EwOp::Copy: launch_pdl(k_ew_binary<4>, g, kEwThreads, 0, st, t, a, b, out); break;
     }
     PFT_LAUNCH_CHECK("ew_binary");
 }
@@ -78,6 +79,7 @@ void ew_binary(const DevTables& t, EwOp op, const PolySet& a, const PolySet& b, 
 // ---- HMUL tensor: d0 = a0 b0, d1 = a0 b1 + a1 b0, d2 = a1 b1 (evaluation domain) -----------
 // set a / b / d hold one ref per ciphertext: ptr to [2][l][N] (a, b) or [3][l][N] (d).
 __global__ void k_tensor(DevTables t, PolySet a, PolySet b, PolySet d) {
+    pdl_wait();
     const int c = blockIdx.z, limb = blockIdx.y;
     const int l = d.p[c].nlimbs;
     if (limb >= l) return;
@@ -112,7 +114,7 @@ __global__ void k_tensor(DevTables t, PolySet a, PolySet b, PolySet d) {
 void ew_tensor(const DevTables& t, const PolySet& a, const PolySet& b, const PolySet& d, cudaStream_t st) {
     if (d.count == 0) return;
     PFT_PROF("tensor", st, set_limbs(d) * t.n * 8.0 * 7);
-    k_tensor<<<ew_grid(t.n, d), kEwThreads, 0, st>>>(t, a, b, d);
+    launch_pdl(k_tensor, ew_grid(t.n, d), kEwThreads, 0, st, t, a, b, d);
     PFT_LAUNCH_CHECK("tensor");
 }
 
@@ -328,6 +330,7 @@ void ew_tensor_dot(const DevTables& t, const u64* const* A, const u64* const* B,
 // rescale (x = c + h, y = NTT(r), s = p^-1): consts[limb] = {add_to_x, s, s_shoup}.
 __global__ void k_sub_scale(DevTables t, PolySet x, PolySet y, PolySet acc, PolySet out, const u64* consts,
                             int has_y, int has_acc) {
+    pdl_wait();
     const int poly = blockIdx.z, limb = blockIdx.y;
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
@@ -357,7 +360,7 @@ void sub_scale(const DevTables& t, const PolySet& x, const PolySet* y, const Pol
                const u64* consts_dev, cudaStream_t st) {
     if (out.count == 0) return;
     PFT_PROF("sub_scale", st, set_limbs(out) * t.n * 8.0 * (2 + (y ? 1 : 0) + (acc ? 1 : 0)));
-    k_sub_scale<<<ew_grid(t.n, out), kEwThreads, 0, st>>>(t, x, y ? *y : out, acc ? *acc : out, out, consts_dev,
+    launch_pdl(k_sub_scale, ew_grid(t.n, out), kEwThreads, 0, st, t, x, y ? *y : out, acc ? *acc : out, out, consts_dev,
                                                          y ? 1 : 0, acc ? 1 : 0);
     PFT_LAUNCH_CHECK("sub_scale");
 }
@@ -371,6 +374,7 @@ void sub_scale(const DevTables& t, const PolySet& x, const PolySet* y, const Pol
 constexpr int kAutBlock = 256, kAutBlocks = 4;
 
 __global__ void __launch_bounds__(256) k_automorph_blocked(DevTables t, PolySet in, PolySet out, u64 g) {
+    pdl_wait();
     __shared__ u64 sm[kAutBlocks * kAutBlock];
     const int poly = blockIdx.z, limb = blockIdx.y;
     const PolyRef& Ro = out.p[poly];
@@ -408,7 +412,7 @@ void automorph(const DevTables& t, const PolySet& in, const PolySet& out, u64 g,
     PFT_PROF("automorph", st, set_limbs(out) * t.n * 16.0);
     if (t.n >= kAutBlocks * kAutBlock) {
         dim3 grid((unsigned)(t.n / (kAutBlocks * kAutBlock)), (unsigned)out.max_limbs, (unsigned)out.count);
-        k_automorph_blocked<<<grid, 256, 0, st>>>(t, in, out, g);
+        launch_pdl(k_automorph_blocked, grid, 256, 0, st, t, in, out, g);
     } else {
         dim3 grid((unsigned)((t.n + 255) / 256), (unsigned)out.max_limbs, (unsigned)out.count);
         k_automorph<<<grid, 256, 0, st>>>(t, in, out, g);
@@ -451,6 +455,7 @@ __global__ void __launch_bounds__(256) k_bconv(DevTables t, BconvBatch jobs) {
     const int x2 = blockIdx.x * blockDim.x + threadIdx.x;
     if (2 * x2 >= t.n) return;
     const int logn = t.logn;
+    pdl_wait();  // the constants above come from the context's tables
     u64 ya[NS], yb[NS];
 #pragma unroll
     for (int i = 0; i < NS; i++) {
@@ -675,14 +680,14 @@ void bconv(const DevTables& t, const BconvJob* jobs, int n_jobs, cudaStream_t st
             dim3 grid((unsigned)((t.n / 2 + 255) / 256), (unsigned)cnt);
             PFT_PROF("bconv", st, 0.0);
             switch (ns) {
-                case 1: k_bconv<1, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 2: k_bconv<2, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 3: k_bconv<3, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 4: k_bconv<4, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 5: k_bconv<5, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 6: k_bconv<6, 2><<<grid, 256, smem, st>>>(t, b); break;
-                case 7: k_bconv<7, 2><<<grid, 256, smem, st>>>(t, b); break;
-                default: k_bconv<8, 2><<<grid, 256, smem, st>>>(t, b); break;
+                case 1: launch_pdl(k_bconv<1, 2>, grid, 256, smem, st, t, b); break;
+                case 2: launch_pdl(k_bconv<2, 2>, grid, 256, smem, st, t, b); break;
+                case 3: launch_pdl(k_bconv<3, 2>, grid, 256, smem, st, t, b); break;
+                case 4: launch_pdl(k_bconv<4, 2>, grid, 256, smem, st, t, b); break;
+                case 5: launch_pdl(k_bconv<5, 2>, grid, 256, smem, st, t, b); break;
+                case 6: launch_pdl(k_bconv<6, 2>, grid, 256, smem, st, t, b); break;
+                case 7: launch_pdl(k_bconv<7, 2>, grid, 256, smem, st, t, b); break;
+                default: launch_pdl(k_bconv<8, 2>, grid, 256, smem, st, t, b); break;
             }
             PFT_LAUNCH_CHECK("bconv");
         }
@@ -955,6 +960,7 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
 #pragma unroll
         for (int c = 0; c < CPT; c++) xs[c] = automorph_src((u32)xo + c, logn, g) & (kKsChunk - 1);
     }
+    pdl_wait();
     u64 kb[BMAX][CPT], ka[BMAX][CPT];
 #pragma unroll
     for (int j = 0; j < BMAX; j++) {
@@ -1101,8 +1107,7 @@ static void launch_ks_bulk(const DevTables& t, const KsBatch& bt, int B, const K
                                       (int)((size_t)kKsStages * std::max(8, BMAX) * kKsChunk * 8)));
     // rows no input reaches (above the highest level) get no CTA
     const dim3 grid((unsigned)(t.n / kKsChunk), (unsigned)(lmax + k), (unsigned)nk);
-    k_ks_inner_bulk<BMAX, PERM>
-        <<<grid, kKsChunk / ks_cpt(BMAX), smem, st>>>(t, bt, B, keys, zstride, L, k, alpha, digits, per);
+    launch_pdl(k_ks_inner_bulk<BMAX, PERM>, grid, kKsChunk / ks_cpt(BMAX), smem, st, t, bt, B, keys, zstride, L, k, alpha, digits, per);
 }
 
 // Self-test of the bounded wait: an mbarrier that expects bytes no copy delivers (no copy is
@@ -1371,6 +1376,7 @@ void ks_inner_hoisted(const DevTables& t, const KsDesc* descs, int B, const KeyR
 // c'_k = (c_k - out_k) p^-1 = (c_k + h - r) / p coefficient by coefficient.
 // last: coefficient-form last limb of each polynomial; out: [l-1][N] per polynomial.
 __global__ void k_rescale_bcast(DevTables t, PolySet last, PolySet out) {
+    pdl_wait();
     const int poly = blockIdx.z, limb = blockIdx.y;
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
@@ -1388,7 +1394,7 @@ void rescale_bcast(const DevTables& t, const PolySet& last, const PolySet& out, 
     if (out.count == 0) return;
     dim3 grid((unsigned)((t.n + 255) / 256), (unsigned)out.max_limbs, (unsigned)out.count);
     PFT_PROF("rescale_bcast", st, set_limbs(out) * t.n * 8.0);
-    k_rescale_bcast<<<grid, 256, 0, st>>>(t, last, out);
+    launch_pdl(k_rescale_bcast, grid, 256, 0, st, t, last, out);
     PFT_LAUNCH_CHECK("rescale_bcast");
 }
 
