@@ -135,10 +135,10 @@ void dfree(pft_ctx* c, void* p) {
 
 // ---- context construction ---------------------------------------------------------------
 static u64 shoup(u64 w, u64 q) { return (u64)(((unsigned __int128)w << 64) / q); }
-// basis-conversion constants are stored in Montgomery form c 2^64 mod t, split as
+// basis-conversion constants are stored in Montgomery form c 2^60 mod t, split as
 // (c' mod 2^30) | (c' >> 30) << 32
 static u64 split30_host(u64 c) { return (c & 0x3fffffffull) | ((c >> 30) << 32); }
-static u64 mont_host(u64 c, u64 t) { return (u64)((((unsigned __int128)c) << 64) % t); }
+static u64 mont_host(u64 c, u64 t) { return (u64)((((unsigned __int128)c) << 60) % t); }
 static int bitlen(u64 x) { return 64 - __builtin_clzll(x); }
 
 static const int kSecureLogQP[17] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 27, 54, 109, 218, 438, 881, 1772};
@@ -199,6 +199,7 @@ static void build_tables(pft_ctx* c) {
         dp[i].q = q;
         dp[i].mu = (u64)((((unsigned __int128)1) << (64 + s)) / q);
         dp[i].r64 = (u64)((((unsigned __int128)1) << 64) % q);
+        dp[i].r60 = (1ull << 60) % q;
         u64 inv = 1;  // q^-1 mod 2^64 by Newton iteration (q odd)
         for (int it = 0; it < 6; it++) inv *= 2 - q * inv;
         dp[i].mneg = 0 - inv;
@@ -441,7 +442,7 @@ static u64* make_switch_key(pft_ctx* c, const u64* sp, u32 key_id) {
     return K;
 }
 
-// An uncompressed key's copy for the key inner product: every word k as (k 2^64 mod p) split
+// An uncompressed key's copy for the key inner product: every word k as (k 2^60 mod p) split
 // into 30-bit halves (the same 8 bytes; the inner product then sums 30-bit products without
 // carries and reduces once in Montgomery form).
 static void add_key(pft_ctx* c, u32 key_id, u64* K) {

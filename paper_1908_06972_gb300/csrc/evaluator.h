@@ -27,7 +27,7 @@ using namespace pft;
 // current, and never while that stream is being captured (a graph's memory must stay its own).
 // Callers may destroy handles from other threads, so the lists have a lock.
 struct BlockCache {
-    static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)128 << 20;
+    static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)1 << 30;
     struct Block {
         void* p;
         size_t bytes;

@@ -80,7 +80,7 @@ __device__ __forceinline__ u64 shoup_est(u64 y, u64 w, u64 wp, u64 nq) {
 // Cooley-Tukey (Harvey) with the estimated quotient, so WY lies in [0, 4q):
 // X, Y in [0, 8q) -> X + WY, X - WY in [0, 8q) (X corrected below 4q; primes below 2^61).
 // LAZY (primes below 2^57): no correction of X, values grow by less than 4q per stage: the
-// 16 stages of an N = 2^16 forward transform from [0, 2q) stay below 66q < 2^63.1.
+// 16 stages of an N = 2^16 forward transform from [0, 5q) (a basis conversion's output) stay below 69q < 2^63.2.
 template <bool LAZY = false>
 __device__ __forceinline__ void ct_bfly(u64& X, u64& Y, ulonglong2 W, u64 q, u64 q2) {
     const u64 q4 = 2 * q2;
@@ -435,12 +435,12 @@ __global__ void __launch_bounds__(col_threads(SA), min_ctas(MT, col_threads(SA))
     }
 }
 
-// Canonical residue of x < 66q (the output range of the uncorrected forward stages) for a prime
+// Canonical residue of x < 69q (the output range of the uncorrected forward stages) for a prime
 // of s + 1 >= 25 bits, with r = floor(2^(s+32) / q) (= mu >> 32) and sh = s - 24.  The quotient
-// is below 66, so one 32-bit high product estimates it: with xh = floor(x / 2^sh) < 2^32,
+// is below 69, so one 32-bit high product estimates it: with xh = floor(x / 2^sh) < 2^32,
 // est = floor(xh r / 2^56) is at most x/q and more than x/q - 2^-22, i.e. floor(x/q) or one
 // less; x - est q then lies in [0, 2q) and one conditional subtraction finishes.
-__device__ __forceinline__ u64 reduce_below66(u64 x, u64 q, u32 r, u32 sh) {
+__device__ __forceinline__ u64 reduce_below69(u64 x, u64 q, u32 r, u32 sh) {
     const u32 xh = (u32)(x >> sh);
     const u32 est = __umulhi(xh, r) >> 24;
     const u64 v = x - (u64)est * q;
@@ -475,7 +475,7 @@ __device__ __forceinline__ const ulonglong2* lm_base(const ulonglong2* rows, int
 // Forward stages SA..SA+7 of the rows of this CTA (limb `limb` of prime pi, rows read from
 // src): canonical results are left in sm, row c2 point m at c2 * kRowStride + m + (m >> 4),
 // after a barrier.
-template <int SA, bool PRE, bool WAIT>
+template <int SA, bool PRE>
 __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restrict__ src, int pi, u64* sm) {
     constexpr int R = rows_per_cta(SA), TOP = SA + 7;
     const int w = threadIdx.x & 15, cc = threadIdx.x >> 4;
@@ -497,7 +497,7 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
     } else {
         stage_row_round1<SA>(tw, blockIdx.x * R, rt, pol);
     }
-    if (WAIT) pdl_wait();
+    pdl_wait();
 #pragma unroll
     for (int e = 0; e < 16; e++) x[e] = src[((size_t)u << 8) | (e << 4) | w];
     if (!PRE) __syncthreads();
@@ -514,7 +514,7 @@ __device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restri
         if (ps >= 24) {
             const u32 r = (u32)(__ldg(&t.primes[pi].mu) >> 32);
 #pragma unroll
-            for (int e = 0; e < 16; e++) my[w * 17 + e] = reduce_below66(x[e], q, r, ps - 24);
+            for (int e = 0; e < 16; e++) my[w * 17 + e] = reduce_below69(x[e], q, r, ps - 24);
         } else {  // primes below 2^25: Shoup multiplication by 1 with 1' = floor(2^64 / q) = mu >> s
             const u64 one_p = __ldg(&t.primes[pi].mu) >> ps;
 #pragma unroll
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA))
     const u64* src = in.p[poly].ptr + ((size_t)limb << logn);
     u64* dst = Ro.ptr + ((size_t)limb << logn);
     if (!INV) {
-        fwd_rows<SA, MT == 0, true>(t, src, pi, sm);
+        fwd_rows<SA, MT == 0>(t, src, pi, sm);
 #pragma unroll
         for (int k = 0; k < 16; k++) {
             const int f = threadIdx.x + R * 16 * k;
@@ -635,8 +635,7 @@ __global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA))
 #pragma unroll
         for (int i = 0; i < 8; i++) load(i, xp[PRE ? i : 0], ap[PRE ? i : 0]);
     }
-    if (flags & kPassPrefetch) fwd_rows<SA, PRE, false>(t, Ri.ptr + base, pi, sm);
-    else fwd_rows<SA, PRE, !PRE>(t, Ri.ptr + base, pi, sm);
+    fwd_rows<SA, PRE>(t, Ri.ptr + base, pi, sm);
     const u64 q = __ldg(&t.primes[pi].q);
     const u64 c = __ldg(&cs[0]), s = __ldg(&cs[1]), sp = __ldg(&cs[2]);
     // (not PRE) the operands of four are loaded before any is used, so that more bytes are in flight

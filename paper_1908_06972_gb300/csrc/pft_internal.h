@@ -28,6 +28,7 @@ struct DPrime {
     u64 q;
     u64 mu;
     u64 r64;   // 2^64 mod q
+    u64 r60;   // 2^60 mod q
     u64 mneg;  // -q^-1 mod 2^64 (Montgomery reduction)
     u32 s;
     u32 pad;
@@ -241,7 +242,7 @@ constexpr u32 kDomKskAEval = 11;
 struct KeyRef {
     const u64* ptr;
     // uncompressed keys: the same words in Montgomery form split into 30-bit halves,
-    // (k 2^64 mod p) = k1 2^30 + k0 stored as k0 | k1 << 32 (the key inner product's operand)
+    // (k 2^60 mod p) = k1 2^30 + k0 stored as k0 | k1 << 32 (the key inner product's operand)
     const u64* mont;
     u32 id;
     int compressed;
@@ -292,7 +293,7 @@ void sample_small(const DevTables& t, const u64 seed[4], u32 dom, u32 obj, u32 s
 void reduce_signed(const DevTables& t, const i64* x_dev, const PolySet& out, cudaStream_t st);
 // out = in mod q per limb, for words of any 64-bit value (e.g. exact integer sums of residues)
 void reduce_words(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
-// out = (in 2^64 mod q) split into 30-bit halves, k0 | k1 << 32 (canonical residues in)
+// out = (in 2^60 mod q) split into 30-bit halves, k0 | k1 << 32 (canonical residues in)
 void mont_split(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
 
 // ---- host math (encode.cpp) -----------------------------------------------------------

@@ -423,33 +423,31 @@ void automorph(const DevTables& t, const PolySet& in, const PolySet& out, u64 g,
 // ---- fast basis conversion (ModUp of one digit, or ModDown from the special primes) ------
 // For each coefficient: y_i = x_i * qhat_i^-1 mod s_i (Shoup), then for every target row m
 // (rows [0, nrows) except [skip_lo, skip_hi), enumerated in order as targets 0..nt-1):
-//   out_m = sum_i y_i * (qhat_i mod t_m) mod t_m   (128-bit sum, one Montgomery reduction),
-// left in [0, 2 t_m): every output feeds a forward transform, whose butterflies take it.
+//   out_m = sum_i y_i * (qhat_i mod t_m) mod t_m   (30-bit-split sums, one Montgomery reduction),
+// left in [0, 5 t_m): every output feeds a forward transform, whose butterflies take it.
 // Target prime of row m: m < split ? m : base2 + m - split.  Table: [ns] {inv, inv_shoup},
-// then [nt][ns] qhat_i 2^64 mod t_m (Montgomery form, target-major, each split into 30-bit
+// then [nt][ns] qhat_i 2^60 mod t_m (Montgomery form, target-major, each split into 30-bit
 // halves: low word = c mod 2^30, high word = c >> 30).  NS (the number of source primes) is a
 // compile-time constant; each thread converts two adjacent coefficients for two targets at
 // a time (four independent accumulation chains).
 template <int NS, int TP>
 __global__ void __launch_bounds__(256) k_bconv(DevTables t, BconvBatch jobs) {
-    extern __shared__ u64 bsm[];
+    extern __shared__ __align__(16) u64 bsm[];
     const BconvJob J = jobs.j[blockIdx.y];
     const int gap = J.skip_hi - J.skip_lo;
     const int nt = J.nrows - gap;
     // the job's constants and, per target, its output row, prime and Montgomery constant,
     // staged once per CTA so that the accumulation loop reads only shared memory
     uint2* sT = reinterpret_cast<uint2*>(bsm);          // [nt][NS] (30-bit split)
-    u64* sQ = bsm + (size_t)nt * NS;                    // [nt] target prime
-    u64* sM = sQ + nt;                                  // [nt] -q^-1 mod 2^64
-    u32* sRow = reinterpret_cast<u32*>(sM + nt);        // [nt] output row
+    // [nt] target prime's halves, -q^-1 mod 2^30 and output row (16-byte aligned)
+    uint4* sP = reinterpret_cast<uint4*>(bsm + ((size_t)nt * NS + 1) / 2 * 2);
     const uint2* T = reinterpret_cast<const uint2*>(J.table + 2 * NS);
     for (int i = threadIdx.x; i < nt * NS; i += blockDim.x) sT[i] = __ldg(&T[i]);
     for (int i = threadIdx.x; i < nt; i += blockDim.x) {
         const int m = i < J.skip_lo ? i : i + gap;
         const int tp = m < J.split ? m : J.base2 + m - J.split;
-        sQ[i] = __ldg(&t.primes[tp].q);
-        sM[i] = __ldg(&t.primes[tp].mneg);
-        sRow[i] = (u32)m;
+        const Mont30 M = mont30(__ldg(&t.primes[tp].q), __ldg(&t.primes[tp].mneg));
+        sP[i] = make_uint4(M.p0, M.p1, M.np, (u32)m);
     }
     __syncthreads();
     const int x2 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -516,17 +514,22 @@ __global__ void __launch_bounds__(256) k_bconv(DevTables t, BconvBatch jobs) {
                 }
             }
         }
-        // constants are c 2^64 mod t, so a Montgomery reduction of the sum (< t 2^63) gives
-        // sum y_i c_i mod t
+        // constants are c 2^60 mod t, so a Montgomery reduction of the sum (< NS 2^60 t) gives
+        // sum y_i c_i mod t, below (NS + 1) t
 #pragma unroll
         for (int u = 0; u < TP; u++) {
             if (m0 + u < nt) {
-                const u64 q = sQ[m0 + u], mneg = sM[m0 + u];
-                const U128 va = acc3_value(a[u]), vb = acc3_value(b[u]);
+                const uint4 tp = sP[m0 + u];
+                const Mont30 M{tp.x, tp.y, tp.z};
                 ulonglong2 r;
-                r.x = mont_reduce_lazy(va.hi, va.lo, q, mneg);
-                r.y = mont_reduce_lazy(vb.hi, vb.lo, q, mneg);
-                *reinterpret_cast<ulonglong2*>(dst + ((size_t)sRow[m0 + u] << logn)) = r;
+                r.x = mont60<(NS > 4)>(a[u], M);
+                r.y = mont60<(NS > 4)>(b[u], M);
+                if (NS > 4) {
+                    const u64 t4 = (((u64)M.p1 << 30) | M.p0) << 2;
+                    if (r.x >= t4) r.x -= t4;
+                    if (r.y >= t4) r.y -= t4;
+                }
+                *reinterpret_cast<ulonglong2*>(dst + ((size_t)tp.w << logn)) = r;
             }
         }
     }
@@ -676,7 +679,7 @@ void bconv(const DevTables& t, const BconvJob* jobs, int n_jobs, cudaStream_t st
                 PFT_LAUNCH_CHECK("bconv (tensor cores)");
                 continue;
             }
-            const size_t smem = (size_t)ntmax * ns * 8 + (size_t)ntmax * 20;
+            const size_t smem = (size_t)(ntmax * ns + 1) / 2 * 16 + (size_t)ntmax * 16;
             dim3 grid((unsigned)((t.n / 2 + 255) / 256), (unsigned)cnt);
             PFT_PROF("bconv", st, 0.0);
             switch (ns) {
@@ -917,10 +920,18 @@ __device__ __forceinline__ void ks_mac(Acc3K& sb, Acc3K& sa, u64 v, u64 kb, u64 
     acc3k_mac(sb, x0, x1, x01, b0, b1, b0 + b1);
     acc3k_mac(sa, x0, x1, x01, a0, a1, a0 + a1);
 }
-// the canonical residue of the sum: (S00 + 2^30 S01 + 2^60 S11) 2^-64 mod p
-__device__ __forceinline__ u64 ks_value(const Acc3K& s, const DPrime& P) {
-    const U128 a = acc3_value(acc3k_fold(s));
-    return mont_reduce(a.hi, a.lo, P.q, P.mneg);
+// the canonical residue of a sum of up to TERMS products (8 of any prime, 12 of primes below 2^56):
+// (S00 + 2^30 S01 + 2^60 S11) 2^-60 mod p.  The reduction leaves it below 2p for narrow primes (below
+// 2^56), else below (TERMS + 1) p, which a few conditional subtractions finish.
+template <int TERMS>
+__device__ __forceinline__ u64 ks_value(const Acc3K& s, const DPrime& P, const Mont30& M, bool narrow) {
+    u64 r = mont60<(TERMS > 4)>(acc3k_fold(s), M);
+    if (TERMS > 1 && !narrow) {
+#pragma unroll
+        for (int k = TERMS > 4 ? 3 : TERMS > 2 ? 2 : 1; k > 0; k--)
+            if (r >= P.q << k) r -= P.q << k;
+    }
+    return r >= P.q ? r - P.q : r;
 }
 
 __host__ __device__ constexpr int ks_cpt(int bmax) { return bmax <= 8 ? 2 : 1; }  // coefficients per thread
@@ -948,7 +959,9 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
     const int xl = CPT * threadIdx.x;
     const size_t xo = chunk0 + xl;
     const DPrime P = load_prime(t.primes, row);
-    const u64* key = keys.mont[blockIdx.z];  // split Montgomery form: k0 | k1 << 32 with k 2^64 mod p = k1 2^30 + k0
+    const Mont30 M = mont30(P.q, P.mneg);
+    const bool narrow = P.s < 56;            // uniform over the CTA
+    const u64* key = keys.mont[blockIdx.z];  // split Montgomery form: k0 | k1 << 32 with k 2^60 mod p = k1 2^30 + k0
     const size_t uz = PERM ? (size_t)blockIdx.z * zstride : 0;
     size_t src0 = chunk0;
     int xs[CPT];  // this thread's coefficients in a staged row
@@ -1035,39 +1048,44 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
             const int l = D.l, E = l + k, beta = D.beta;
             const int m = row < L ? row : l + row - L;
             const u64* st = ring + ((size_t)s * per_stage + i) * stage_digits * kKsChunk;
-            // sums of at most 8 products of residues below 2^60 in 30-bit-split Karatsuba partial
-            // sums (three widening multiply-adds per product), then one Montgomery reduction: the
-            // key words carry the factor 2^64 (sum < 8 p^2 < p 2^63)
-            u64 r0[CPT], r1[CPT];
+            // 30-bit-split Karatsuba partial sums (three widening multiply-adds per product), then one
+            // Montgomery reduction: the key words carry the factor 2^60.  Up to 8 products of residues below
+            // 2^60 per sum (the middle sum's bound); with primes below 2^56 up to 12, so that more than 8
+            // digits need a second reduction only in the rows of larger primes
+            u64 r0[CPT] = {}, r1[CPT] = {};
+            Acc3K s0[CPT], s1[CPT];
 #pragma unroll
-            for (int h = 0; h < BMAX; h += 8) {
-                if (h > 0 && beta <= h) break;
-                Acc3K s0[CPT], s1[CPT];
+            for (int c = 0; c < CPT; c++) s0[c] = s1[c] = {0, 0, 0};
+            const bool halves = BMAX > 12 || (BMAX > 8 && !narrow);
 #pragma unroll
-                for (int c = 0; c < CPT; c++) s0[c] = s1[c] = {0, 0, 0};
+            for (int j = 0; j < BMAX; j++) {
+                if (BMAX > 8 && j == 8 && halves) {
 #pragma unroll
-                for (int j = h; j < (BMAX < h + 8 ? BMAX : h + 8); j++) {
-                    if (j < beta) {
-                        u64 v[CPT];
-                        if constexpr (CPT == 2 && !PERM) {
-                            const ulonglong2 vv =
-                                *reinterpret_cast<const ulonglong2*>(st + (size_t)j * kKsChunk + xl);
-                            v[0] = vv.x;
-                            v[1] = vv.y;
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < CPT; c++) v[c] = st[(size_t)j * kKsChunk + xs[c]];
-                        }
-#pragma unroll
-                        for (int c = 0; c < CPT; c++) ks_mac(s0[c], s1[c], v[c], kb[j][c], ka[j][c]);
+                    for (int c = 0; c < CPT; c++) {
+                        r0[c] = ks_value<8>(s0[c], P, M, narrow);
+                        r1[c] = ks_value<8>(s1[c], P, M, narrow);
+                        s0[c] = s1[c] = {0, 0, 0};
                     }
                 }
+                if (j < beta) {
+                    u64 v[CPT];
+                    if constexpr (CPT == 2 && !PERM) {
+                        const ulonglong2 vv = *reinterpret_cast<const ulonglong2*>(st + (size_t)j * kKsChunk + xl);
+                        v[0] = vv.x;
+                        v[1] = vv.y;
+                    } else {
 #pragma unroll
-                for (int c = 0; c < CPT; c++) {
-                    const u64 v0 = ks_value(s0[c], P), v1 = ks_value(s1[c], P);
-                    r0[c] = h ? addmod(r0[c], v0, P.q) : v0;
-                    r1[c] = h ? addmod(r1[c], v1, P.q) : v1;
+                        for (int c = 0; c < CPT; c++) v[c] = st[(size_t)j * kKsChunk + xs[c]];
+                    }
+#pragma unroll
+                    for (int c = 0; c < CPT; c++) ks_mac(s0[c], s1[c], v[c], kb[j][c], ka[j][c]);
                 }
+            }
+#pragma unroll
+            for (int c = 0; c < CPT; c++) {
+                const u64 v0 = ks_value<BMAX>(s0[c], P, M, narrow), v1 = ks_value<BMAX>(s1[c], P, M, narrow);
+                r0[c] = halves ? addmod(r0[c], v0, P.q) : v0;
+                r1[c] = halves ? addmod(r1[c], v1, P.q) : v1;
             }
             u64* o0 = D.u + uz + ((size_t)m << logn) + xo;
             u64* o1 = D.u + uz + (((size_t)E + m) << logn) + xo;
@@ -1317,6 +1335,7 @@ static void ks_bulk(const DevTables& t, const KsBatch& bt, int B, const KsKeys& 
     else if (digits <= 2) go(launch_ks_bulk<2, PERM>);
     else if (digits <= 4) go(launch_ks_bulk<4, PERM>);
     else if (digits <= 8) go(launch_ks_bulk<8, PERM>);
+    else if (digits <= 12) go(launch_ks_bulk<12, PERM>);
     else go(launch_ks_bulk<16, PERM>);
 }
 
@@ -1500,7 +1519,7 @@ __global__ void k_mont_split(DevTables t, PolySet in, PolySet out) {
     if (c >= t.n) return;
     const DPrime P = load_prime(t.primes, prime_of(Ro, limb));
     const size_t o = ((size_t)limb << t.logn) + c;
-    const u64 m = mulmod(in.p[poly].ptr[o], P.r64, P);  // k 2^64 mod p
+    const u64 m = mulmod(in.p[poly].ptr[o], P.r60, P);  // k 2^60 mod p
     Ro.ptr[o] = (m & 0x3fffffffull) | ((m >> 30) << 32);
 }
 
