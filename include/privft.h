@@ -352,8 +352,8 @@ int pft_rotate_batch(pft_ctx* ctx, const pft_ct* const* a, int B, int32_t step, 
 
 /* ---- autotuning -----------------------------------------------------------
  * A search over the ring's transform plans, per launch size.  A plan is one of the
- * specialised kernels (two-pass 8 + 8, at N = 2^15 7 + 8, with register rounds at 3 or 4 resident
- * CTAs per SM; N = 2^16 only: one launch on an 8-CTA cluster exchanging through distributed shared
+ * specialised kernels (two-pass 8 + 8, at N = 2^15 7 + 8, with register rounds, registers bounded
+ * for 640 or 1024 resident threads per SM; N = 2^16 only: one launch on an 8-CTA cluster exchanging through distributed shared
  * memory) or a sequence of generic shared-memory passes with a chosen number of stages and
  * sub-transforms per CTA (N = 2^16: 8+8 at two tile widths, 6+10, 10+6, 7+9, 9+7, 5+5+6; N = 2^15:
  * 8+7, 7+8, 9+6, 6+9, 5+5+5, then the two specialised ones; N <= 2^14 has a single plan).  For each launch-size bucket (total limbs of a
@@ -363,7 +363,7 @@ int pft_rotate_batch(pft_ctx* ctx, const pft_ct* const* a, int B, int32_t step, 
  * to `cap` plan times (microseconds) of the largest bucket, *chosen its choice (an index into
  * the plan list of pft_autotune_report).  Synchronous.  The environment variable PFT_NTT16
  * (twopass, twopass4, cluster, generic) overrides every choice at N = 2^16.  Before any search
- * a context (N >= 2^12) uses the two-pass kernels at 3 CTAs per SM, and at 4 CTAs per SM for launches of more
+ * a context (N >= 2^12) uses the two-pass kernels at 640 threads per SM, and at 1024 for launches of more
  * than 512 limbs at N = 2^16 (the search's choice for that bucket on a GB300). */
 #define PFT_NTT16_VARIANTS 4
 int pft_autotune(pft_ctx* ctx, double* us_out, int cap, int* chosen);
@@ -375,7 +375,7 @@ int pft_autotune_report(pft_ctx* ctx, char* buf, size_t cap, size_t* len);
 /* Use plan `plan` (index into the ring's plan list, in the order above) for every launch size;
  * -1: back to the plans a new context starts with. */
 int pft_set_transform_plan(pft_ctx* ctx, int plan);
-/* Pin the transform variant (0..PFT_NTT16_VARIANTS-1: two-pass 3 CTAs/SM, two-pass 4 CTAs/SM,
+/* Pin the transform variant (0..PFT_NTT16_VARIANTS-1: two-pass at 640 and at 1024 threads/SM,
  * cluster, generic) for every launch size, without timing.  N < 2^16 has no cluster form (variant 2
  * is variant 0 there), N <= 2^14 one two-pass form, and rings below 2^12 only the generic one. */
 int pft_set_transform_variant(pft_ctx* ctx, int variant);

@@ -336,17 +336,22 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
 // for launches of a few.  Against the generic kernels below (one CTA per limb to N = 2^14, staged
 // passes at 2^15; GB300): one HMUL + rescale at N = 2^13, level 3: 188 -> 100 us (its three inverse
 // launches took 58 us each on 1 to 3 SMs); 31 HMULs + rescales at N = 2^15, levels 12..18: 6.15 -> 3.70 ms.
-// Why these shapes: at N = 2^16 and 2^15 CTAs of 256 threads (16 columns, 32 columns; 16 rows); the
-// smaller rings meet launches of a few limbs, so their CTAs are small (64 or 128 threads) to
-// spread a limb over the SMs.
+// Why these shapes: CTAs of 128 threads (8 columns of 2^8 points, 16 of 2^7; 8 rows) meet their loads,
+// exchanges and stores at different times and overlap better than CTAs of 256: 480 limbs, forward and
+// inverse, 660 -> 622 us, and with five of them per SM at 96 registers instead of six at 80 606 us (four at 128:
+// 625).  Launches of more than 512 limbs keep 64 registers (1024 threads) and 16 columns in the forward
+// passes: 32 HMULs with 4 rotations 28.0 ms, 28.2 with five CTAs, 28.5 with 8 columns and 80 registers.
+// The smaller rings meet launches of a few limbs: smaller CTAs still spread a limb over the SMs.
 constexpr int kRowStride = 273;  // 256 + 16 padding + 1
 constexpr u64 kLazyBound = 1ull << 57;  // forward butterflies skip the correction below this prime
-__host__ __device__ constexpr int cols_per_cta(int SA) { return SA == 8 ? 16 : 32; }
-__host__ __device__ constexpr int rows_per_cta(int SA) { return SA >= 7 ? 16 : SA == 6 ? 8 : 4; }
-__host__ __device__ constexpr int col_threads(int SA) { return cols_per_cta(SA) << (SA - 4); }
+__host__ __device__ constexpr int cols_per_cta(int SA, bool INV, int MT) {
+    return SA == 8 ? (!INV && MT == 1024 ? 16 : 8) : SA == 7 ? 16 : 32;
+}
+__host__ __device__ constexpr int rows_per_cta(int SA) { return SA >= 6 ? 8 : 4; }
+__host__ __device__ constexpr int col_threads(int SA, bool INV, int MT) { return cols_per_cta(SA, INV, MT) << (SA - 4); }
 __host__ __device__ constexpr int row_threads(int SA) { return rows_per_cta(SA) * 16; }
 
-// MT: resident threads per SM the registers are bounded for (768: 80 registers, 1024: 64), or 0 for
+// MT: resident threads per SM the registers are bounded for (640: 96 registers, 1024: 64), or 0 for
 // launches that fit the GPU at once (kPreThreadsPerSm): then one CTA's latency is the launch's time,
 // registers are plenty, and every twiddle is loaded at the start (the fused pass's operands with the data),
 // so that the stages wait for memory once: one HMUL + rescale at N = 2^13 100 -> 88 us.
@@ -358,12 +363,14 @@ __host__ __device__ constexpr int min_ctas(int MT, int threads) { return MT == 0
 // (r - h) mod q_k with r = (c_{l-1} + h) mod p, h = floor(p/2).  A pass of its own for it (k_rescale_bcast)
 // took 17 % of a batch of rescales: it writes and the column pass reads back every limb.
 template <bool INV, int SA, int MT, bool UNSCALED = false, bool BCAST = false>
-__global__ void __launch_bounds__(col_threads(SA), min_ctas(MT, col_threads(SA)))
+__global__ void __launch_bounds__(col_threads(SA, INV, MT), min_ctas(MT, col_threads(SA, INV, MT)))
     k_ntt_cols(DevTables t, PolySet in, PolySet out, int flags) {
-    constexpr int C = cols_per_cta(SA), LO = SA - 4;     // LO: bits of the second round
+    constexpr int C = cols_per_cta(SA, INV, MT), LO = SA - 4;  // LO: bits of the second round
     constexpr bool PRE = MT == 0;
-    constexpr int ST = C == 16 ? 17 : C;
-    __shared__ u64 sm[SA > 4 ? (1 << SA) * ST : 1];
+    // row r of the exchange at r C words, every 16 rows C words apart (C < 32: without that the second
+    // round's reads, 16 rows apart within a warp, would meet in the same banks)
+    __shared__ u64 sm[SA > 4 ? (1 << SA) * C + (C < 32 ? (C << (SA - 4)) : 0) : 1];
+    auto at = [](int r, int c) { return r * C + (C < 32 ? (r >> 4) * C : 0) + c; };
     const int poly = pass_poly(flags), limb = pass_limb(flags);
     const PolyRef& Ro = out.p[poly];
     if (limb >= Ro.nlimbs) return;
@@ -408,10 +415,10 @@ __global__ void __launch_bounds__(col_threads(SA), min_ctas(MT, col_threads(SA))
         else ntt_round<false, LO, SA - 1, 4, false, false, false, false, PRE>(x, w, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
         if constexpr (SA > 4) {
 #pragma unroll
-            for (int e = 0; e < 16; e++) sm[((e << LO) | w) * ST + cc] = x[e];
+            for (int e = 0; e < 16; e++) sm[at((e << LO) | w, cc)] = x[e];
             __syncthreads();
 #pragma unroll
-            for (int e = 0; e < 16; e++) x[e] = sm[((w << 4) | e) * ST + cc];
+            for (int e = 0; e < 16; e++) x[e] = sm[at((w << 4) | e, cc)];
             if (lazy) ntt_round<false, 0, SA - 1, LO, true, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
             else ntt_round<false, 0, SA - 1, LO, false, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
         }
@@ -423,10 +430,10 @@ __global__ void __launch_bounds__(col_threads(SA), min_ctas(MT, col_threads(SA))
         if constexpr (SA > 4) {
             ntt_round<true, 0, SA - 1, LO, false, false, false, false, PRE>(x, w << 4, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w2);
 #pragma unroll
-            for (int e = 0; e < 16; e++) sm[((w << 4) | e) * ST + cc] = x[e];
+            for (int e = 0; e < 16; e++) sm[at((w << 4) | e, cc)] = x[e];
             __syncthreads();
 #pragma unroll
-            for (int e = 0; e < 16; e++) x[e] = sm[((e << LO) | w) * ST + cc];
+            for (int e = 0; e < 16; e++) x[e] = sm[at((e << LO) | w, cc)];
         }
         ntt_round<true, LO, SA - 1, 4, false, UNSCALED, false, false, PRE>(x, w, 0, tw, q, q2, NI, NI1, nullptr, nullptr, 0, w1);
 #pragma unroll
@@ -671,8 +678,7 @@ __global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA))
     }
 }
 
-// Shared-memory carveout of the kernels bounded for 1024 threads per SM (four CTAs of 35 KB): one
-// that fits them, the rest L1.
+// Shared-memory carveout of the kernels bounded for 1024 threads per SM: one that fits their CTAs, the rest L1.
 template <int SA, int MT>
 static void prepare_twopass(void) {
     if (MT == 1024 && first_on_device((const void*)&k_ntt_rows_epi<SA, MT, false>)) {
@@ -683,7 +689,6 @@ static void prepare_twopass(void) {
         set(k_ntt_cols<true, SA, MT>);
         set(k_ntt_cols<true, SA, MT, true>);
         set(k_ntt_rows<false, SA, MT>);
-        set(k_ntt_rows<true, SA, MT>);
         set(k_ntt_rows_epi<SA, MT, false>);
         set(k_ntt_rows_epi<SA, MT, true>);
     }
@@ -693,8 +698,8 @@ static int second_pass(const DevTables& t, int flags) { return flags | ((t.ntt_o
 
 template <int SA, int MT>
 struct TwoPass {
-    static dim3 col_grid(const PolySet& s) {
-        return dim3(256 / cols_per_cta(SA), (unsigned)s.max_limbs, (unsigned)s.count);
+    static dim3 col_grid(const PolySet& s, bool inv) {
+        return dim3(256 / cols_per_cta(SA, inv, MT), (unsigned)s.max_limbs, (unsigned)s.count);
     }
     static dim3 row_grid(const PolySet& s) {
         return dim3((1 << SA) / rows_per_cta(SA), (unsigned)s.max_limbs, (unsigned)s.count);
@@ -705,7 +710,7 @@ struct TwoPass {
     static void cols_fwd(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
         prepare_twopass<SA, MT>();
         PFT_PROF("ntt.fwd.strided", st, work(t, out, SA));
-        launch_pdl(k_ntt_cols<false, SA, MT>, col_grid(out), col_threads(SA), 0, st, t, in, out, 0);
+        launch_pdl(k_ntt_cols<false, SA, MT>, col_grid(out, false), col_threads(SA, false, MT), 0, st, t, in, out, 0);
         PFT_LAUNCH_CHECK("ntt pass A");
     }
     static void forward(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
@@ -719,7 +724,7 @@ struct TwoPass {
         if (bcast) {
             prepare_twopass<SA, MT>();
             PFT_PROF("ntt.fwd.strided", st, work(t, io, SA));
-            launch_pdl(k_ntt_cols<false, SA, MT, false, true>, col_grid(io), col_threads(SA), 0, st, t, in, io, 0);
+            launch_pdl(k_ntt_cols<false, SA, MT, false, true>, col_grid(io, false), col_threads(SA, false, MT), 0, st, t, in, io, 0);
             PFT_LAUNCH_CHECK("rescale broadcast + ntt pass A");
         } else {
             cols_fwd(t, in, io, st);
@@ -737,14 +742,14 @@ struct TwoPass {
         prepare_twopass<SA, MT>();
         {
             PFT_PROF("ntt.inv.contig", st, work(t, out, 8));
-            launch_pdl(k_ntt_rows<true, SA, MT>, row_grid(out), row_threads(SA), 0, st, t, in, out, 0);
+            launch_pdl(k_ntt_rows<true, SA, MT == 1024 ? 640 : MT>, row_grid(out), row_threads(SA), 0, st, t, in, out, 0);
         }
         PFT_LAUNCH_CHECK("intt pass B");
         PFT_PROF("ntt.inv.strided", st, work(t, out, SA));
         if (unscaled)
-            launch_pdl(k_ntt_cols<true, SA, MT, true>, col_grid(out), col_threads(SA), 0, st, t, out, out, second_pass(t, kPassFinal));
+            launch_pdl(k_ntt_cols<true, SA, MT, true>, col_grid(out, true), col_threads(SA, true, MT), 0, st, t, out, out, second_pass(t, kPassFinal));
         else
-            launch_pdl(k_ntt_cols<true, SA, MT>, col_grid(out), col_threads(SA), 0, st, t, out, out, second_pass(t, kPassFinal));
+            launch_pdl(k_ntt_cols<true, SA, MT>, col_grid(out, true), col_threads(SA, true, MT), 0, st, t, out, out, second_pass(t, kPassFinal));
         PFT_LAUNCH_CHECK("intt pass A");
     }
 };
@@ -752,13 +757,14 @@ struct TwoPass {
 // to 255 registers leave room for about that many; 256, 512 and 1024 measured within 2 % of each
 // other, none at all 10 % slower for small rings).
 static constexpr int kPreThreadsPerSm = 512;
-// f(TwoPass<..>) for the ring's shape and the launch's limbs; v: 0 = bounded for 768 resident threads per
-// SM (3 CTAs of 256), 1 = for 1024 (4 CTAs; N = 2^16 and 2^15)
+// f(TwoPass<..>) for the ring's shape and the launch's limbs; v: 0 = bounded for 640 resident threads per
+// SM, 1 = for 1024 (N = 2^16 and 2^15; its inverse row pass stays at 640: 1400 against 1480 us in the
+// workload above)
 template <int SA, class F>
 static void with_twopass_sa(double limbs, int v, F f) {
     if (limbs * (1 << SA) * 16 <= 152.0 * kPreThreadsPerSm) f(TwoPass<SA, 0>());
-    else if (SA >= 7 && v == 1) f(TwoPass<SA, SA >= 7 ? 1024 : 768>());
-    else f(TwoPass<SA, 768>());
+    else if (SA >= 7 && v == 1) f(TwoPass<SA, SA >= 7 ? 1024 : 640>());
+    else f(TwoPass<SA, 640>());
 }
 template <class F>
 static void with_twopass(const DevTables& t, int v, double limbs, F f) {
@@ -999,8 +1005,8 @@ int ntt_candidates(int logn, DevTables::Plan* out, const char** names, int cap) 
         DevTables::Plan p;
     };
     static const Cand c16[] = {
-        {"two-pass 8+8 (register rounds), 3 CTAs/SM", {0, 0, {0, 0, 0}, {0, 0, 0}}},
-        {"two-pass 8+8 (register rounds), 4 CTAs/SM", {1, 0, {0, 0, 0}, {0, 0, 0}}},
+        {"two-pass 8+8 (register rounds), 640 threads/SM", {0, 0, {0, 0, 0}, {0, 0, 0}}},
+        {"two-pass 8+8 (register rounds), 1024 threads/SM", {1, 0, {0, 0, 0}, {0, 0, 0}}},
         {"one launch, 8-CTA cluster (DSMEM exchange)", {2, 0, {0, 0, 0}, {0, 0, 0}}},
         {"staged 8+8, 16 sub-transforms/CTA", {3, 2, {8, 8, 0}, {16, 16, 0}}},
         {"staged 8+8, 8 sub-transforms/CTA", {3, 2, {8, 8, 0}, {8, 8, 0}}},
@@ -1016,8 +1022,8 @@ int ntt_candidates(int logn, DevTables::Plan* out, const char** names, int cap) 
         {"staged 9+6", {3, 2, {9, 6, 0}, {8, 64, 0}}},
         {"staged 6+9", {3, 2, {6, 9, 0}, {64, 8, 0}}},
         {"staged 5+5+5 (three passes)", {3, 3, {5, 5, 5}, {128, 128, 128}}},
-        {"two-pass 7+8 (register rounds), 3 CTAs/SM", {0, 0, {0, 0, 0}, {0, 0, 0}}},
-        {"two-pass 7+8 (register rounds), 4 CTAs/SM", {1, 0, {0, 0, 0}, {0, 0, 0}}},
+        {"two-pass 7+8 (register rounds), 640 threads/SM", {0, 0, {0, 0, 0}, {0, 0, 0}}},
+        {"two-pass 7+8 (register rounds), 1024 threads/SM", {1, 0, {0, 0, 0}, {0, 0, 0}}},
     };
     const Cand* c = logn == 16 ? c16 : logn == 15 ? c15 : nullptr;
     const int n = logn == 16 ? (int)(sizeof(c16) / sizeof(c16[0])) : logn == 15 ? (int)(sizeof(c15) / sizeof(c15[0])) : 0;

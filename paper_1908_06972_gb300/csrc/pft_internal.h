@@ -76,12 +76,12 @@ struct DevTables {
     // pass asks L2 for its epilogue operands at the start of each CTA: faster while the epilogue
     // read one 8-byte word per row, slower since it reads 16 bytes four rows ahead).  Default 3.
     int ntt_order;
-    int ntt_variant;       // transform of N >= 2^12: 0 two-pass (3 CTAs/SM), 1 two-pass (4 CTAs/SM),
+    int ntt_variant;       // transform of N >= 2^12: 0 two-pass (640 threads/SM), 1 two-pass (1024),
                            // 2 one-launch cluster (N = 2^16), 3 generic staged passes
     // Transform plan per launch size (bucket of the launch's total limbs: <= 64, <= 512,
     // larger), chosen by the autotuner; kind < 0: the fixed variant above.
     struct Plan {
-        int8_t kind;   // -1 none, 0 two-pass 3 CTAs/SM, 1 two-pass 4 CTAs/SM, 2 cluster, 3 generic
+        int8_t kind;   // -1 none, 0 two-pass 640 threads/SM, 1 two-pass 1024, 2 cluster, 3 generic
         int8_t npass;  // generic: passes, first (largest stride) first
         int8_t S[3];   // generic: stages per pass
         int16_t C[3];  // generic: sub-transforms per CTA of each pass
@@ -91,8 +91,8 @@ constexpr int kNttVariants = 4;
 constexpr int kNttBuckets = 3;
 inline int ntt_bucket(double limbs) { return limbs <= 64 ? 0 : limbs <= 512 ? 1 : 2; }
 // Plans before any search: the fixed variant, except that launches of more than 512 limbs at
-// N = 2^16 take the two-pass kernels at 4 CTAs per SM (the search's choice for that bucket on a
-// GB300: 324.5 against 313.8 mult+relin/s in the benchmark step).
+// N = 2^16 take the two-pass kernels at 1024 threads per SM (32 HMULs with 4 rotations: 28.0 ms, 28.2 at
+// 640).
 inline void default_plans(DevTables& t) {
     for (int b = 0; b < kNttBuckets; b++) t.plan[b].kind = -1;
     if (t.logn == 16) t.plan[2].kind = 1;
