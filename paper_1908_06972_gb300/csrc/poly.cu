@@ -4,6 +4,7 @@
 // limb-major [poly][limb][N] layout, moving two 64-bit words per thread with
 // 16-byte accesses.  Residues are canonical in [0, q) at every kernel boundary.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include <cstdlib>
@@ -429,9 +430,12 @@ void automorph(const DevTables& t, const PolySet& in, const PolySet& out, u64 g,
 // then [nt][ns] qhat_i 2^60 mod t_m (Montgomery form, target-major, each split into 30-bit
 // halves: low word = c mod 2^30, high word = c >> 30).  NS (the number of source primes) is a
 // compile-time constant; each thread converts two adjacent coefficients for two targets at
-// a time (four independent accumulation chains).
+// a time (four independent accumulation chains).  Bound: the integer multiply pipe (16 widening
+// multiplies per output of four sources; 68 % busy).  CTAs of 128 threads: 4.67 ms in 32 HMULs with 4
+// rotations; of 256: 4.80; four targets at a time: 5.24.
+constexpr int kBconvThreads = 128;
 template <int NS, int TP>
-__global__ void __launch_bounds__(256) k_bconv(DevTables t, BconvBatch jobs) {
+__global__ void __launch_bounds__(kBconvThreads) k_bconv(DevTables t, BconvBatch jobs) {
     extern __shared__ __align__(16) u64 bsm[];
     const BconvJob J = jobs.j[blockIdx.y];
     const int gap = J.skip_hi - J.skip_lo;
@@ -680,17 +684,17 @@ void bconv(const DevTables& t, const BconvJob* jobs, int n_jobs, cudaStream_t st
                 continue;
             }
             const size_t smem = (size_t)(ntmax * ns + 1) / 2 * 16 + (size_t)ntmax * 16;
-            dim3 grid((unsigned)((t.n / 2 + 255) / 256), (unsigned)cnt);
+            dim3 grid((unsigned)((t.n / 2 + kBconvThreads - 1) / kBconvThreads), (unsigned)cnt);
             PFT_PROF("bconv", st, 0.0);
             switch (ns) {
-                case 1: launch_pdl(k_bconv<1, 2>, grid, 256, smem, st, t, b); break;
-                case 2: launch_pdl(k_bconv<2, 2>, grid, 256, smem, st, t, b); break;
-                case 3: launch_pdl(k_bconv<3, 2>, grid, 256, smem, st, t, b); break;
-                case 4: launch_pdl(k_bconv<4, 2>, grid, 256, smem, st, t, b); break;
-                case 5: launch_pdl(k_bconv<5, 2>, grid, 256, smem, st, t, b); break;
-                case 6: launch_pdl(k_bconv<6, 2>, grid, 256, smem, st, t, b); break;
-                case 7: launch_pdl(k_bconv<7, 2>, grid, 256, smem, st, t, b); break;
-                default: launch_pdl(k_bconv<8, 2>, grid, 256, smem, st, t, b); break;
+                case 1: launch_pdl(k_bconv<1, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 2: launch_pdl(k_bconv<2, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 3: launch_pdl(k_bconv<3, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 4: launch_pdl(k_bconv<4, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 5: launch_pdl(k_bconv<5, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 6: launch_pdl(k_bconv<6, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                case 7: launch_pdl(k_bconv<7, 2>, grid, kBconvThreads, smem, st, t, b); break;
+                default: launch_pdl(k_bconv<8, 2>, grid, kBconvThreads, smem, st, t, b); break;
             }
             PFT_LAUNCH_CHECK("bconv");
         }
@@ -867,11 +871,12 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms.
 // The key slice is loaded before the ring is started: after it (copies in flight first) measured
 // slower for few inputs, 95 against 87 us for one at level 30.
-// PERM (hoisted rotations): grid z = several keys over the same inputs, key z with Galois element
+// PERM (hoisted rotations): several keys over the same inputs, key z (grid y) with Galois element
 // g[z]; the digit rows are read through X -> X^g.  A chunk of 256 destinations reads one aligned
 // block of 256 sources, so the copies stay whole blocks and only the reads from shared memory are
 // permuted: no permuted copy of the extended digits is made (it was beta (l + k) limbs written and
-// read per rotation).  With the batching of op_rotate_hoisted over inputs and steps, 32 rotation-light
+// read per rotation).  The keys of one row run together, so that the row's digits (18 MB for 8 inputs of 9
+// digits at N = 2^15) come from HBM once for all of them.  With the batching of op_rotate_hoisted over inputs and steps, 32 rotation-light
 // inferences at level 3: 132 -> 48 ms; 4 at N = 2^15, levels 12..18: 80 -> 22 ms.
 constexpr int kKsStages = 3;
 constexpr int kKsChunk = 256;                // coefficients per CTA (2 KiB per digit row)
@@ -935,6 +940,16 @@ __device__ __forceinline__ u64 ks_value(const Acc3K& s, const DPrime& P, const M
 }
 
 __host__ __device__ constexpr int ks_cpt(int bmax) { return bmax <= 8 ? 2 : 1; }  // coefficients per thread
+// f(integral_constant<beta>) for 1 <= beta <= NB
+template <int NB, class F>
+__device__ __forceinline__ void ks_digits(int beta, F f) {
+    if constexpr (NB == 1) {
+        f(std::integral_constant<int, 1>());
+    } else {
+        if (beta == NB) f(std::integral_constant<int, NB>());
+        else ks_digits<NB - 1>(beta, f);
+    }
+}
 struct KsKeys {
     const u64* mont[kMaxKsKeys];
     u32 g[kMaxKsKeys];
@@ -950,7 +965,8 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
     __shared__ __align__(8) u64 bars[kKsStages];
     // special rows first: every input uses them, so their CTAs are the longest and should not
     // form the last wave
-    const int row = (int)blockIdx.y < k ? L + (int)blockIdx.y : (int)blockIdx.y - k;
+    const int by = (int)blockIdx.z, z = (int)blockIdx.y;
+    const int row = by < k ? L + by : by - k;
     const int logn = t.logn;
     const int rows_total = L + k;
     const int need = bt.need[row];
@@ -961,14 +977,14 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
     const DPrime P = load_prime(t.primes, row);
     const Mont30 M = mont30(P.q, P.mneg);
     const bool narrow = P.s < 56;            // uniform over the CTA
-    const u64* key = keys.mont[blockIdx.z];  // split Montgomery form: k0 | k1 << 32 with k 2^60 mod p = k1 2^30 + k0
-    const size_t uz = PERM ? (size_t)blockIdx.z * zstride : 0;
+    const u64* key = keys.mont[z];  // split Montgomery form: k0 | k1 << 32 with k 2^60 mod p = k1 2^30 + k0
+    const size_t uz = PERM ? (size_t)z * zstride : 0;
     size_t src0 = chunk0;
     int xs[CPT];  // this thread's coefficients in a staged row
 #pragma unroll
     for (int c = 0; c < CPT; c++) xs[c] = xl + c;
     if (PERM) {
-        const u32 g = keys.g[blockIdx.z];
+        const u32 g = keys.g[z];
         src0 = automorph_src((u32)chunk0, logn, g) & ~(u32)(kKsChunk - 1);
 #pragma unroll
         for (int c = 0; c < CPT; c++) xs[c] = automorph_src((u32)xo + c, logn, g) & (kKsChunk - 1);
@@ -1052,22 +1068,25 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
             // Montgomery reduction: the key words carry the factor 2^60.  Up to 8 products of residues below
             // 2^60 per sum (the middle sum's bound); with primes below 2^56 up to 12, so that more than 8
             // digits need a second reduction only in the rows of larger primes
-            u64 r0[CPT] = {}, r1[CPT] = {};
-            Acc3K s0[CPT], s1[CPT];
-#pragma unroll
-            for (int c = 0; c < CPT; c++) s0[c] = s1[c] = {0, 0, 0};
+            u64 r0[CPT], r1[CPT];
             const bool halves = BMAX > 12 || (BMAX > 8 && !narrow);
+            // straight code for each number of digits: with a branch per digit the sums were moved around
+            // at every merge
+            ks_digits<BMAX>(beta, [&](auto count) {
+                constexpr int NB = decltype(count)::value;
+                Acc3K s0[CPT], s1[CPT];
 #pragma unroll
-            for (int j = 0; j < BMAX; j++) {
-                if (BMAX > 8 && j == 8 && halves) {
+                for (int c = 0; c < CPT; c++) s0[c] = s1[c] = {0, 0, 0};
 #pragma unroll
-                    for (int c = 0; c < CPT; c++) {
-                        r0[c] = ks_value<8>(s0[c], P, M, narrow);
-                        r1[c] = ks_value<8>(s1[c], P, M, narrow);
-                        s0[c] = s1[c] = {0, 0, 0};
+                for (int j = 0; j < NB; j++) {
+                    if (j == 8 && halves) {
+#pragma unroll
+                        for (int c = 0; c < CPT; c++) {
+                            r0[c] = ks_value<8>(s0[c], P, M, narrow);
+                            r1[c] = ks_value<8>(s1[c], P, M, narrow);
+                            s0[c] = s1[c] = {0, 0, 0};
+                        }
                     }
-                }
-                if (j < beta) {
                     u64 v[CPT];
                     if constexpr (CPT == 2 && !PERM) {
                         const ulonglong2 vv = *reinterpret_cast<const ulonglong2*>(st + (size_t)j * kKsChunk + xl);
@@ -1080,13 +1099,13 @@ __global__ void __launch_bounds__(kKsChunk / ks_cpt(BMAX))
 #pragma unroll
                     for (int c = 0; c < CPT; c++) ks_mac(s0[c], s1[c], v[c], kb[j][c], ka[j][c]);
                 }
-            }
 #pragma unroll
-            for (int c = 0; c < CPT; c++) {
-                const u64 v0 = ks_value<BMAX>(s0[c], P, M, narrow), v1 = ks_value<BMAX>(s1[c], P, M, narrow);
-                r0[c] = halves ? addmod(r0[c], v0, P.q) : v0;
-                r1[c] = halves ? addmod(r1[c], v1, P.q) : v1;
-            }
+                for (int c = 0; c < CPT; c++) {
+                    const u64 v0 = ks_value<NB>(s0[c], P, M, narrow), v1 = ks_value<NB>(s1[c], P, M, narrow);
+                    r0[c] = NB > 8 && halves ? addmod(r0[c], v0, P.q) : v0;
+                    r1[c] = NB > 8 && halves ? addmod(r1[c], v1, P.q) : v1;
+                }
+            });
             u64* o0 = D.u + uz + ((size_t)m << logn) + xo;
             u64* o1 = D.u + uz + (((size_t)E + m) << logn) + xo;
             if constexpr (CPT == 2) {
@@ -1124,7 +1143,7 @@ static void launch_ks_bulk(const DevTables& t, const KsBatch& bt, int B, const K
         PFT_CUDA(cudaFuncSetAttribute(k_ks_inner_bulk<BMAX, PERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)((size_t)kKsStages * std::max(8, BMAX) * kKsChunk * 8)));
     // rows no input reaches (above the highest level) get no CTA
-    const dim3 grid((unsigned)(t.n / kKsChunk), (unsigned)(lmax + k), (unsigned)nk);
+    const dim3 grid((unsigned)(t.n / kKsChunk), (unsigned)nk, (unsigned)(lmax + k));
     launch_pdl(k_ks_inner_bulk<BMAX, PERM>, grid, kKsChunk / ks_cpt(BMAX), smem, st, t, bt, B, keys, zstride, L, k, alpha, digits, per);
 }
 
@@ -1335,6 +1354,7 @@ static void ks_bulk(const DevTables& t, const KsBatch& bt, int B, const KsKeys& 
     else if (digits <= 2) go(launch_ks_bulk<2, PERM>);
     else if (digits <= 4) go(launch_ks_bulk<4, PERM>);
     else if (digits <= 8) go(launch_ks_bulk<8, PERM>);
+    else if (digits <= 10) go(launch_ks_bulk<10, PERM>);  // 64 registers against 116: 362, 457 us (31 inputs of 9)
     else if (digits <= 12) go(launch_ks_bulk<12, PERM>);
     else go(launch_ks_bulk<16, PERM>);
 }
