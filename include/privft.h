@@ -72,7 +72,9 @@ typedef struct pft_ft_model pft_ft_model; /* packed fastText weights (H, O) */
 
 /* Device allocator.  alloc(bytes, stream, user) returns device memory usable on
  * `stream` (NULL on failure); free(ptr, stream, user) releases it once the work
- * already queued on `stream` no longer needs it. */
+ * already queued on `stream` no longer needs it.  A context keeps freed blocks of up to
+ * 16 MiB (1 GiB at most) for its next calls on the same stream and frees them when an
+ * allocation fails, pft_set_stream changes the stream or the context is destroyed. */
 typedef struct {
     void* (*alloc)(size_t bytes, void* stream, void* user);
     void (*free)(void* ptr, void* stream, void* user);
@@ -353,10 +355,11 @@ int pft_rotate_batch(pft_ctx* ctx, const pft_ct* const* a, int B, int32_t step, 
 /* ---- autotuning -----------------------------------------------------------
  * A search over the ring's transform plans, per launch size.  A plan is one of the
  * specialised kernels (two-pass 8 + 8, at N = 2^15 7 + 8, with register rounds, registers bounded
- * for 640 or 1024 resident threads per SM; N = 2^16 only: one launch on an 8-CTA cluster exchanging through distributed shared
- * memory) or a sequence of generic shared-memory passes with a chosen number of stages and
- * sub-transforms per CTA (N = 2^16: 8+8 at two tile widths, 6+10, 10+6, 7+9, 9+7, 5+5+6; N = 2^15:
- * 8+7, 7+8, 9+6, 6+9, 5+5+5, then the two specialised ones; N <= 2^14 has a single plan).  For each launch-size bucket (total limbs of a
+ * for 640 or 1024 resident threads per SM; N = 2^16 only: one launch on an 8-CTA cluster
+ * exchanging through distributed shared memory) or a sequence of generic shared-memory passes
+ * with a chosen number of stages and sub-transforms per CTA (N = 2^16: 8+8 at two tile widths,
+ * 6+10, 10+6, 7+9, 9+7, 5+5+6; N = 2^15: 8+7, 7+8, 9+6, 6+9, 5+5+5, then the two specialised
+ * ones; N <= 2^14 has a single plan).  For each launch-size bucket (total limbs of a
  * launch: <= 64, <= 512, larger) every plan is timed on a forward + inverse transform of a
  * representative launch (32, 256, 1024 limbs; median of 3 CUDA-event timings on the context's
  * stream) and the fastest is kept for launches of that size.  us_out (may be NULL) receives up

@@ -335,7 +335,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
 // Bound: the integer multiply pipe for launches of many limbs, the latency of one thread's 16 points
 // for launches of a few.  Against the generic kernels below (one CTA per limb to N = 2^14, staged
 // passes at 2^15; GB300): one HMUL + rescale at N = 2^13, level 3: 188 -> 100 us (its three inverse
-// launches took 58 us each on 1 to 3 SMs); 31 HMULs + rescales at N = 2^15, levels 12..18: 6.15 -> 3.70 ms.
+// launches took 58 us each on 1 to 3 SMs), 52 with the later changes; 31 HMULs + rescales at N = 2^15,
+// levels 12..18: 6.15 -> 3.70 ms, 2.85 with the later ones.
 // Why these shapes: CTAs of 128 threads (8 columns of 2^8 points, 16 of 2^7; 8 rows) meet their loads,
 // exchanges and stores at different times and overlap better than CTAs of 256: 480 limbs, forward and
 // inverse, 660 -> 622 us, and with five of them per SM at 96 registers instead of six at 80 606 us (four at 128:

@@ -868,16 +868,18 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // Bound: HBM and the multiply pipe together from 3 digits on (187 us for 4 ciphertexts at level 30,
 // 5.3 TB/s), the latency of a stage below.  64 inputs of one digit (level 3): 265 us with one input
 // per stage, 194 us with four.  9 digits at N = 2^15 (31 inputs, levels 12..18) ran in the generic kernel
-// before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms.
+// before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms; the sum
+// itself 457 us in the form for 12 digits, 350 in the one for 10 with straight code per digit count.
 // The key slice is loaded before the ring is started: after it (copies in flight first) measured
 // slower for few inputs, 95 against 87 us for one at level 30.
 // PERM (hoisted rotations): several keys over the same inputs, key z (grid y) with Galois element
 // g[z]; the digit rows are read through X -> X^g.  A chunk of 256 destinations reads one aligned
 // block of 256 sources, so the copies stay whole blocks and only the reads from shared memory are
 // permuted: no permuted copy of the extended digits is made (it was beta (l + k) limbs written and
-// read per rotation).  The keys of one row run together, so that the row's digits (18 MB for 8 inputs of 9
-// digits at N = 2^15) come from HBM once for all of them.  With the batching of op_rotate_hoisted over inputs and steps, 32 rotation-light
-// inferences at level 3: 132 -> 48 ms; 4 at N = 2^15, levels 12..18: 80 -> 22 ms.
+// read per rotation).  The keys of one row run together, so that the row's digits (18 MB for 8 inputs
+// of 9 digits at N = 2^15) come from HBM once for all of them.  With the batching of op_rotate_hoisted
+// over inputs and steps, 32 rotation-light inferences at level 3: 132 -> 48 ms (40.7 with the later
+// changes); 4 at N = 2^15, levels 12..18: 80 -> 22 ms (18.2).
 constexpr int kKsStages = 3;
 constexpr int kKsChunk = 256;                // coefficients per CTA (2 KiB per digit row)
 constexpr long long kWaitPolls = 1ll << 22;  // polls of a bounded wait (seconds at most)
@@ -1354,7 +1356,7 @@ static void ks_bulk(const DevTables& t, const KsBatch& bt, int B, const KsKeys& 
     else if (digits <= 2) go(launch_ks_bulk<2, PERM>);
     else if (digits <= 4) go(launch_ks_bulk<4, PERM>);
     else if (digits <= 8) go(launch_ks_bulk<8, PERM>);
-    else if (digits <= 10) go(launch_ks_bulk<10, PERM>);  // 64 registers against 116: 362, 457 us (31 inputs of 9)
+    else if (digits <= 10) go(launch_ks_bulk<10, PERM>);  // 80 registers against 128
     else if (digits <= 12) go(launch_ks_bulk<12, PERM>);
     else go(launch_ks_bulk<16, PERM>);
 }
