@@ -865,9 +865,9 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // in place of the two CTA barriers per input measured slower: 201 against 196 us for 4
 // ciphertexts at level 30; so did one coefficient per thread in CTAs of 256 threads, 64
 // registers and twice the resident warps, for 8 digits: 221 us.)
-// Bound: HBM and the multiply pipe together from 3 digits on (187 us for 4 ciphertexts at level 30,
-// 5.3 TB/s), the latency of a stage below.  64 inputs of one digit (level 3): 265 us with one input
-// per stage, 194 us with four.  9 digits at N = 2^15 (31 inputs, levels 12..18) ran in the generic kernel
+// Bound: HBM and the multiply pipe together from 3 digits on (177 us for 4 ciphertexts at level 30,
+// 5.6 TB/s; 195 us with one 64-bit Montgomery reduction), the latency of a stage below.  64 inputs of one
+// digit (level 3): 265 us with one input per stage, 194 us with four, 161 with the two-step reduction.  9 digits at N = 2^15 (31 inputs, levels 12..18) ran in the generic kernel
 // before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms; the sum
 // itself 457 us in the form for 12 digits, 350 in the one for 10 with straight code per digit count.
 // The key slice is loaded before the ring is started: after it (copies in flight first) measured
