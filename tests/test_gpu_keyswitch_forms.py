@@ -29,7 +29,8 @@ def enc(p, i, level):
     return o.encrypt_sk(o.encode(synth.slots(50 + i, 32), level=level), 60 + i)
 
 
-@pytest.mark.parametrize("levels", [[18], [16], [17, 1, 3], [9, 1, 2, 8, 16, 5, 9], [2] * 7, [1] * 19, [8, 4, 4, 3]])
+@pytest.mark.parametrize("levels", [[18], [16], [17, 1, 3], [9, 1, 2, 8, 16, 5, 9], [2] * 7, [1] * 19, [8, 4, 4, 3],
+                                    [9, 9, 4], [10, 1, 9], [12, 8, 11, 9]])
 def test_digit_counts(p18, levels):
     p, o, pf = p18, p18.orc, p18.pft
     distinct = {l: (enc(p, 2 * l, l), enc(p, 2 * l + 1, l)) for l in set(levels)}
@@ -41,7 +42,7 @@ def test_digit_counts(p18, levels):
         p.assert_equal(h, want[l], "input %d at level %d" % (i, l))
 
 
-@pytest.mark.parametrize("level", [1, 2, 3, 8, 9, 16, 18])
+@pytest.mark.parametrize("level", [1, 2, 3, 8, 9, 10, 12, 16, 18])
 def test_hoisted_digit_counts(p18, level):
     p, o, pf = p18, p18.orc, p18.pft
     a = enc(p, 7, level)
