@@ -520,13 +520,12 @@ static NttEpi epi_of(const std::vector<PolyRef>& x, const std::vector<PolyRef>& 
 static void ntt_fwd_sub_scale(pft_ctx* c, const std::vector<PolyRef>& conv, const std::vector<PolyRef>& x,
                               const std::vector<PolyRef>& acc, const std::vector<PolyRef>& out, const u64* consts,
                               const std::vector<u32>* gs = nullptr) {
-    bool fused = true;
-    chunks(conv.size(), [&](size_t lo, size_t hi) {
-        if (fused)
-            fused = ntt_forward_epilogue(c->tabs, mkset(conv, lo, hi), epi_of(x, acc, out, {consts}, gs, lo, hi),
-                                         c->stream);
-    });
-    if (fused) return;
+    if (ntt_fused(c, conv)) {
+        chunks(conv.size(), [&](size_t lo, size_t hi) {
+            ntt_forward_epilogue(c->tabs, mkset(conv, lo, hi), epi_of(x, acc, out, {consts}, gs, lo, hi), c->stream);
+        });
+        return;
+    }
     NEED(!gs, PFT_ERR_ARG, "internal: permuted accumulators without the fused pass");
     ntt_fwd(c, conv, conv);
     std::vector<PolyRef> xw, yw, aw, ow, xn, yn, on;

@@ -194,15 +194,28 @@ inline void ntt_fwd(pft_ctx* c, const std::vector<PolyRef>& in, const std::vecto
 inline void ntt_inv(pft_ctx* c, const std::vector<PolyRef>& in, const std::vector<PolyRef>& out) {
     chunks(out.size(), [&](size_t a, size_t b) { ntt_inverse(c->tabs, mkset(in, a, b), mkset(out, a, b), c->stream); });
 }
+// Whether every launch of a batch over `polys` (chunks of kMaxSet, each with its own plan by size) has
+// the fused and unscaled kernels.  Asked before the first launch: a batch is processed in one form.
+inline bool ntt_fused(pft_ctx* c, const std::vector<PolyRef>& polys) {
+    bool all = true;
+    chunks(polys.size(), [&](size_t a, size_t b) {
+        double limbs = 0;
+        for (size_t i = a; i < b; i++) limbs += polys[i].nlimbs;
+        all = all && ntt_has_fused(c->tabs, limbs);
+    });
+    return all;
+}
 // N times the inverse transform where the transform variant has that kernel (true), else the
 // inverse transform itself (false)
 inline bool ntt_inv_unscaled(pft_ctx* c, const std::vector<PolyRef>& in, const std::vector<PolyRef>& out) {
-    bool unscaled = true;
+    if (!ntt_fused(c, out)) {
+        ntt_inv(c, in, out);
+        return false;
+    }
     chunks(out.size(), [&](size_t a, size_t b) {
-        if (unscaled) unscaled = ntt_inverse_unscaled(c->tabs, mkset(in, a, b), mkset(out, a, b), c->stream);
+        ntt_inverse_unscaled(c->tabs, mkset(in, a, b), mkset(out, a, b), c->stream);
     });
-    if (!unscaled) ntt_inv(c, in, out);
-    return unscaled;
+    return true;
 }
 inline void ew(pft_ctx* c, EwOp op, const std::vector<PolyRef>& a, const std::vector<PolyRef>& b,
                const std::vector<PolyRef>& out) {

@@ -1190,33 +1190,33 @@ void mul_rates(cudaStream_t st, double* lo, double* hi, double* wide) {
     PFT_CUDA(cudaFree(sink));
 }
 
-bool ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
-    if (out.count == 0) return true;
-    const int fam = ntt_family(t, set_limbs(out));
-    if (fam > 1) return false;
-    with_twopass(t, fam, set_limbs(out), [&](auto tp) { tp.inverse(t, in, out, true, st); });
-    return true;
+// the two-pass plan of a launch that needs its fused or unscaled kernels
+static int fused_family(const DevTables& t, double limbs) {
+    const int fam = ntt_family(t, limbs);
+    if (fam > 1) fail(PFT_ERR_ARG, "internal: no fused transform kernel in this launch's plan");
+    return fam;
 }
-
+bool ntt_has_fused(const DevTables& t, double limbs) { return ntt_family(t, limbs) <= 1; }
 bool ntt_always_fused(const DevTables& t) {
     for (double limbs : {1.0, 100.0, 1000.0})
-        if (ntt_family(t, limbs) > 1) return false;
+        if (!ntt_has_fused(t, limbs)) return false;
     return true;
 }
-bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
-    if (io.count == 0) return true;
-    const int fam = ntt_family(t, set_limbs(io));
-    if (fam > 1) return false;
-    with_twopass(t, fam, set_limbs(io), [&](auto tp) { tp.forward_epi(t, io, io, e, false, st); });
-    return true;
+void ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
+    if (out.count == 0) return;
+    const double limbs = set_limbs(out);
+    with_twopass(t, fused_family(t, limbs), limbs, [&](auto tp) { tp.inverse(t, in, out, true, st); });
 }
-bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e,
+void ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st) {
+    if (io.count == 0) return;
+    const double limbs = set_limbs(io);
+    with_twopass(t, fused_family(t, limbs), limbs, [&](auto tp) { tp.forward_epi(t, io, io, e, false, st); });
+}
+void ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e,
                           cudaStream_t st) {
-    if (io.count == 0) return true;
-    const int fam = ntt_family(t, set_limbs(io));
-    if (fam > 1) return false;
-    with_twopass(t, fam, set_limbs(io), [&](auto tp) { tp.forward_epi(t, last, io, e, true, st); });
-    return true;
+    if (io.count == 0) return;
+    const double limbs = set_limbs(io);
+    with_twopass(t, fused_family(t, limbs), limbs, [&](auto tp) { tp.forward_epi(t, last, io, e, true, st); });
 }
 void ntt_inverse(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st) {
     run(t, in, out, true, st);

@@ -161,19 +161,20 @@ struct NttEpi {
     const u64* consts[kMaxSet];
     u32 g[kMaxSet];
 };
-// Forward transform of io (in place) fused with the epilogue; false (nothing launched) where
-// the ring or the transform variant has no fused kernel.
-bool ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st);
-// RESCALE's forward part: io = the broadcast of `last` (one limb in coefficient form per polynomial,
-// the dropped prime being the one after io's limbs; see rescale_bcast), then the same; false
-// (nothing launched) where there is no fused kernel.
-bool ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e, cudaStream_t st);
-// Whether launches of every size have these fused kernels.
+// The fused and unscaled kernels below exist where a launch of that many limbs has a two-pass plan
+// (ntt_has_fused); the plan goes by a launch's size, so a batch of several launches asks for all of them
+// before the first.  Without one they fail and launch nothing.
+bool ntt_has_fused(const DevTables& t, double limbs);
+// The same for launches of every size.
 bool ntt_always_fused(const DevTables& t);
+// Forward transform of io (in place) fused with the epilogue.
+void ntt_forward_epilogue(const DevTables& t, const PolySet& io, const NttEpi& e, cudaStream_t st);
+// RESCALE's forward part: io = the broadcast of `last` (one limb in coefficient form per polynomial,
+// the dropped prime being the one after io's limbs; see rescale_bcast), then the same.
+void ntt_rescale_epilogue(const DevTables& t, const PolySet& last, const PolySet& io, const NttEpi& e, cudaStream_t st);
 // N times the inverse transform (no N^-1 at the last stage, values in [0, 4q)) for consumers
-// that scale their input anyway; false (nothing launched) where the ring or the transform
-// variant has no such kernel.
-bool ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
+// that scale their input anyway.
+void ntt_inverse_unscaled(const DevTables& t, const PolySet& in, const PolySet& out, cudaStream_t st);
 // Butterflies per second of the transform's (exact-path) butterfly arithmetic on register data
 // only: the arithmetic ceiling the transforms are measured against (synchronous).
 double bfly_ceiling(const DevTables& t, cudaStream_t st);
