@@ -868,11 +868,41 @@ static void op_rotate_batch(pft_ctx* c, const pft_ct* const* a, int B, int32_t s
 // One form for all keys and rings: the automorphism is applied where the digits and c0 are read
 // (k_ks_inner_bulk, k_ntt_rows_epi), every stage is one launch over a tile of inputs and steps.
 // Tiles: inputs whose extended digits fit kHoistExtBytes; steps such that the products of the tile
-// fit kHoistTileBytes (one input and step are 10 MiB at level 3 and 64 MiB at level 30), halved while
-// the allocator refuses.  Tiles that stay in L2 lose more to the launches' tails than they save: 32
+// fit kHoistTileBytes (one input and step are 10 MiB at level 3 and 64 MiB at level 30).  While the
+// allocator refuses, first the steps of a tile are halved, then its inputs, and one input that still does not
+// fit takes rotate_hoisted_one.  Tiles that stay in L2 lose more to the launches' tails than they save: 32
 // inferences at level 3 took 57.1 ms with tiles of 128 MiB, 51.9 with 256 MiB, 47.9 with 1 GiB, 47.9 with 2.
 constexpr size_t kHoistExtBytes = (size_t)2 << 30, kHoistTileBytes = (size_t)1 << 30;
 
+// Buffers for outputs that have none large enough, held apart until an operation has all its memory:
+// a refused allocation leaves every output as it was.
+struct FreshOutputs {
+    pft_ctx* c;
+    std::map<pft_ct*, u64*> p;
+    explicit FreshOutputs(pft_ctx* c_) : c(c_) {}
+    ~FreshOutputs() {
+        for (auto& kv : p) dfree(c, kv.second);
+    }
+    void add(pft_ct* o, int level) {
+        NEED(o && handle_live(o), PFT_ERR_ARG, "output is not a live ciphertext handle");
+        NEED(!o->ctx || o->ctx == c, PFT_ERR_ARG, "output handle from another context");
+        const size_t words = (size_t)2 * level * c->n;
+        if (o->cap < words && !p.count(o)) p[o] = (u64*)dalloc(c, words * 8);
+    }
+    void take(pft_ct* o, int level) {  // o gets its buffer (the old one is freed in stream order)
+        auto it = p.find(o);
+        if (it != p.end()) {
+            dfree(c, o->data);
+            o->data = it->second;
+            o->cap = (size_t)2 * level * c->n;
+            p.erase(it);
+        }
+        o->ctx = c;
+        o->level = level;
+    }
+};
+
+// PFT_ERR_OOM is thrown before any work is queued and any output is touched.
 static void hoisted_tile(pft_ctx* c, const pft_ct* const* in, int B, const std::vector<u32>& gs,
                          const std::vector<std::vector<pft_ct*>>& outs) {
     const int k = c->k, L = c->L, alpha = c->alpha, n = (int)gs.size();
@@ -890,29 +920,10 @@ static void hoisted_tile(pft_ctx* c, const pft_ct* const* in, int B, const std::
         tU += 2 * (size_t)E;
         tCv += 2 * (size_t)l;
     }
+    FreshOutputs fresh(c);
+    for (int b = 0; b < B; b++)
+        for (pft_ct* o : outs[b]) fresh.add(o, in[b]->level);
     Scratch Ext(c, tExt * limb * 8);
-    auto ext = [&](int b, int j) { return Ext.u() + (oExt[b] + (size_t)j * (in[b]->level + k)) * limb; };
-    std::vector<KsDesc> desc(B);
-    {
-        // ModUp of every c1, once
-        Scratch Dc(c, tDc * limb * 8);
-        std::vector<PolyRef> src, dst, rows;
-        for (int b = 0; b < B; b++) {
-            src.push_back(cpoly(in[b]->data, in[b]->level, c->n, 1));
-            dst.push_back(ref(Dc.u() + oDc[b] * limb, in[b]->level));
-        }
-        const bool unscaled = ntt_inv_unscaled(c, src, dst);  // N^-1 then in the conversion tables
-        std::vector<BconvJob> jobs;
-        for (int b = 0; b < B; b++) {
-            const int l = in[b]->level, beta = (l + alpha - 1) / alpha;
-            for (int j = 0; j < beta; j++) {
-                jobs.push_back(modup_job(c, l, j, dst[b].ptr, ext(b, j), unscaled));
-                modup_rows(c, l, j, ext(b, j), rows);
-            }
-        }
-        bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
-        ntt_fwd(c, rows, rows);
-    }
     int tile = (int)std::max<size_t>(1, std::min<size_t>(n, kHoistTileBytes / ((tU + tCv) * limb * 8)));
     std::unique_ptr<Scratch> U, Cv;
     for (;;) {
@@ -926,6 +937,32 @@ static void hoisted_tile(pft_ctx* c, const pft_ct* const* in, int B, const std::
             tile = (tile + 1) / 2;
         }
     }
+    for (int b = 0; b < B; b++)
+        for (pft_ct* o : outs[b]) {
+            fresh.take(o, in[b]->level);
+            o->scale = in[b]->scale;
+        }
+    auto ext = [&](int b, int j) { return Ext.u() + (oExt[b] + (size_t)j * (in[b]->level + k)) * limb; };
+    {
+        // ModUp of every c1, once; the coefficient form waits where ModDown's conversions go later
+        std::vector<PolyRef> src, dst, rows;
+        for (int b = 0; b < B; b++) {
+            src.push_back(cpoly(in[b]->data, in[b]->level, c->n, 1));
+            dst.push_back(ref(Cv->u() + oDc[b] * limb, in[b]->level));
+        }
+        const bool unscaled = ntt_inv_unscaled(c, src, dst);  // N^-1 then in the conversion tables
+        std::vector<BconvJob> jobs;
+        for (int b = 0; b < B; b++) {
+            const int l = in[b]->level, beta = (l + alpha - 1) / alpha;
+            for (int j = 0; j < beta; j++) {
+                jobs.push_back(modup_job(c, l, j, dst[b].ptr, ext(b, j), unscaled));
+                modup_rows(c, l, j, ext(b, j), rows);
+            }
+        }
+        bconv(c->tabs, jobs.data(), (int)jobs.size(), c->stream);
+        ntt_fwd(c, rows, rows);
+    }
+    std::vector<KsDesc> desc(B);
     for (int b = 0; b < B; b++) {
         desc[b].ext = ext(b, 0);
         desc[b].u = U->u() + oU[b] * limb;
@@ -976,14 +1013,14 @@ void op_rotate_hoisted(pft_ctx* c, const pft_ct* const* in, int B, const int32_t
                  "outputs must be distinct from the input");
     }
     std::vector<u32> gs;
-    std::vector<int> at;
+    std::vector<int> at, ident;
     bool streamed = ntt_always_fused(c->tabs);
     for (int s = 0; s < n; s++) {
         const u32 g = galois_of(c->n, steps[s]);
         NEED(g == 1 || c->keys.count(g), PFT_ERR_NO_KEY, "no rotation key for step " + std::to_string(steps[s]));
+        (g == 1 ? ident : at).push_back(s);
         if (g == 1) continue;
         gs.push_back(g);
-        at.push_back(s);
         streamed = streamed && ks_inner_bulk_ok(c->tabs, keyref(c, g), lmax, c->alpha);
     }
     // a handle that appears for several steps of one input ends with the last step's rotation: only
@@ -1000,42 +1037,41 @@ void op_rotate_hoisted(pft_ctx* c, const pft_ct* const* in, int B, const int32_t
         op_rotate_hoisted(c, in, 1, st.data(), (int)st.size(), o.data());
         return;
     }
-    const size_t limb = (size_t)c->n;
     std::vector<std::vector<pft_ct*>> act(B);
-    for (int b = 0; b < B; b++) {
-        const int l = in[b]->level;
-        for (int s = 0, i = 0; s < n; s++) {
-            pft_ct* o = outs[(size_t)b * n + s];
-            ensure_ct(c, o, l);
-            o->scale = in[b]->scale;
-            if (i < (int)at.size() && at[i] == s) {
-                act[b].push_back(o);
-                i++;
-            } else {  // identity rotation
-                PFT_CUDA(cudaMemcpyAsync(o->data, in[b]->data, 2 * l * limb * 8, cudaMemcpyDeviceToDevice, c->stream));
-            }
-        }
-    }
-    if (gs.empty()) return;
-    if (!streamed) {  // compressed keys, more than 16 digits, rings or plans without the fused pass
-        for (int b = 0; b < B; b++) rotate_hoisted_one(c, in[b], gs, act[b]);
-        return;
-    }
-    int b0 = 0;
+    for (int b = 0; b < B; b++)
+        for (int s : at) act[b].push_back(outs[(size_t)b * n + s]);
+    int b0 = gs.empty() ? B : 0, most = streamed ? B : 0;  // inputs per tile; none: step by step
     while (b0 < B) {
         int b1 = b0;
         size_t bytes = 0;
-        while (b1 < B) {
+        while (b1 < B && b1 - b0 < most) {
             const int l = in[b1]->level;
-            const size_t w = ((size_t)(l + c->alpha - 1) / c->alpha * (l + c->k) + l) * limb * 8;
+            const size_t w = ((size_t)(l + c->alpha - 1) / c->alpha * (l + c->k) + l) * c->n * 8;
             if (b1 > b0 && bytes + w > kHoistExtBytes) break;
             bytes += w;
             b1++;
         }
-        hoisted_tile(c, in + b0, b1 - b0, gs,
-                     std::vector<std::vector<pft_ct*>>(act.begin() + b0, act.begin() + b1));
-        b0 = b1;
+        if (b1 == b0) {  // compressed keys, more than 16 digits, rings or plans without the fused pass; no memory
+            rotate_hoisted_one(c, in[b0], gs, act[b0]);
+            b0++;
+            continue;
+        }
+        try {
+            hoisted_tile(c, in + b0, b1 - b0, gs, std::vector<std::vector<pft_ct*>>(act.begin() + b0, act.begin() + b1));
+            b0 = b1;
+        } catch (const Error& e) {
+            if (e.code != PFT_ERR_OOM) throw;
+            most = (b1 - b0) / 2;
+        }
     }
+    for (int b = 0; b < B; b++)
+        for (int s : ident) {
+            pft_ct* o = outs[(size_t)b * n + s];
+            const size_t words = 2 * (size_t)in[b]->level * c->n;
+            ensure_ct(c, o, in[b]->level);
+            o->scale = in[b]->scale;
+            PFT_CUDA(cudaMemcpyAsync(o->data, in[b]->data, words * 8, cudaMemcpyDeviceToDevice, c->stream));
+        }
 }
 
 // The same for one ciphertext, step by step, with permuted copies of the extended digits and of c0:
@@ -1067,6 +1103,8 @@ static void rotate_hoisted_one(pft_ctx* c, const pft_ct* a, const std::vector<u3
     }
     for (size_t i = 0; i < gs.size(); i++) {
         pft_ct* o = outs[i];
+        ensure_ct(c, o, l);
+        o->scale = a->scale;
         // automorphism of the extended digits and of c0
         std::vector<PolyRef> ein, eout;
         for (int j = 0; j < beta; j++) {
