@@ -1556,68 +1556,78 @@ static void ft_finish_columns(pft_ctx* c, const pft_ft_model* M, const std::vect
 
 // BEGIN, diagonal packing: Q = sum_i sum_k rot(v_i, k) D_{i,k} (chunk i of the vocabulary): the n - 1
 // hoisted rotations of every chunk of every document in one batched call, then one dot product
-// of chunks n terms per document.  Documents (any levels, ordered by level) go in groups that bound
-// the memory of the rotated copies.
-static void ft_begin_diag(pft_ctx* c, const pft_ft_model* M, const std::vector<FtDoc*>& docs) {
+// of chunks n terms per document.
+static void ft_begin_diag_group(pft_ctx* c, const pft_ft_model* M, const std::vector<FtDoc*>& group) {
     const int cols = M->n, nch = M->chunks;
     const size_t limb = c->n;
     std::vector<int32_t> hsteps;
     for (int k = 1; k < cols; k++) hsteps.push_back(k);
-    for (FtDoc* d : docs) ft_init_work(c, d, 1, d->v[0]->scale * M->H[0]->scale);
     const size_t rot_per_doc = (size_t)nch * (cols - 1);
+    std::vector<pft_ct> R(group.size() * rot_per_doc);
+    struct CleanR {
+        pft_ctx* c;
+        std::vector<pft_ct>* T;
+        ~CleanR() {
+            for (auto& x : *T) dfree(c, x.data);
+        }
+    } cleanR{c, &R};
+    std::vector<const pft_ct*> in;
+    std::vector<pft_ct*> outs;
+    for (FtDoc* d : group)
+        for (int i = 0; i < nch; i++) in.push_back(d->v[i]);
+    for (auto& x : R) {  // [document][chunk][k - 1]
+        x.ctx = c;
+        outs.push_back(&x);
+    }
+    op_rotate_hoisted(c, in.data(), (int)in.size(), hsteps.data(), cols - 1, outs.data());
+    size_t at = 0;
+    for (auto& kv : docs_by_level(group)) {  // ascending levels: the order of `group`
+        const int l = kv.first;
+        std::vector<const u64*> A, Bv;
+        std::vector<u64*> O;
+        for (int i = 0; i < nch; i++)
+            for (int k = 0; k < cols; k++) Bv.push_back(M->H[(size_t)i * cols + k]->data);
+        for (FtDoc* d : kv.second) {
+            const pft_ct* rot = &R[at * rot_per_doc];
+            at++;
+            for (int pol = 0; pol < 2; pol++) {
+                for (int i = 0; i < nch; i++) {
+                    A.push_back(d->v[i]->data + (size_t)pol * l * limb);
+                    for (int k = 1; k < cols; k++)
+                        A.push_back(rot[(size_t)i * (cols - 1) + k - 1].data + (size_t)pol * l * limb);
+                }
+                O.push_back(d->W[0].data + (size_t)pol * l * limb);
+            }
+        }
+        Scratch dA(c, A.size() * 8), dB(c, Bv.size() * 8), dO(c, O.size() * 8);
+        ew_dot(c->tabs, upload(c, dA, A), upload(c, dB, Bv), upload(c, dO, O), (int)O.size(), nch * cols, true, l,
+               c->stream);
+    }
+}
+
+// Documents (any levels, ordered by level) in groups that bound the memory of the rotated copies; a
+// group that the allocator has no room for is halved.
+static void ft_begin_diag(pft_ctx* c, const pft_ft_model* M, const std::vector<FtDoc*>& docs) {
+    for (FtDoc* d : docs) ft_init_work(c, d, 1, d->v[0]->scale * M->H[0]->scale);
+    const size_t rot_per_doc = (size_t)M->chunks * (M->n - 1);
     std::vector<FtDoc*> order(docs);
     std::stable_sort(order.begin(), order.end(), [](const FtDoc* x, const FtDoc* y) { return x->l < y->l; });
-    size_t b0 = 0;
+    size_t b0 = 0, most = order.size();
     while (b0 < order.size()) {
         size_t b1 = b0, bytes = 0;
-        while (b1 < order.size()) {
-            const size_t w = rot_per_doc * 2 * order[b1]->l * limb * 8;
+        while (b1 < order.size() && b1 - b0 < most) {
+            const size_t w = rot_per_doc * 2 * order[b1]->l * c->n * 8;
             if (b1 > b0 && bytes + w > ((size_t)16 << 30)) break;
             bytes += w;
             b1++;
         }
-        std::vector<pft_ct> R((b1 - b0) * rot_per_doc);
-        struct CleanR {
-            pft_ctx* c;
-            std::vector<pft_ct>* T;
-            ~CleanR() {
-                for (auto& x : *T) dfree(c, x.data);
-            }
-        } cleanR{c, &R};
-        std::vector<const pft_ct*> in;
-        std::vector<pft_ct*> outs;
-        for (size_t b = b0; b < b1; b++)
-            for (int i = 0; i < nch; i++) in.push_back(order[b]->v[i]);
-        for (auto& x : R) {  // [document][chunk][k - 1]
-            x.ctx = c;
-            outs.push_back(&x);
+        try {
+            ft_begin_diag_group(c, M, std::vector<FtDoc*>(order.begin() + b0, order.begin() + b1));
+            b0 = b1;
+        } catch (const Error& e) {
+            if (e.code != PFT_ERR_OOM || b1 - b0 == 1) throw;
+            most = (b1 - b0) / 2;
         }
-        op_rotate_hoisted(c, in.data(), (int)in.size(), hsteps.data(), cols - 1, outs.data());
-        const std::vector<FtDoc*> group(order.begin() + b0, order.begin() + b1);
-        size_t at = 0;
-        for (auto& kv : docs_by_level(group)) {  // ascending levels: the order of `group`
-            const int l = kv.first;
-            std::vector<const u64*> A, Bv;
-            std::vector<u64*> O;
-            for (int i = 0; i < nch; i++)
-                for (int k = 0; k < cols; k++) Bv.push_back(M->H[(size_t)i * cols + k]->data);
-            for (FtDoc* d : kv.second) {
-                const pft_ct* rot = &R[at * rot_per_doc];
-                at++;
-                for (int pol = 0; pol < 2; pol++) {
-                    for (int i = 0; i < nch; i++) {
-                        A.push_back(d->v[i]->data + (size_t)pol * l * limb);
-                        for (int k = 1; k < cols; k++)
-                            A.push_back(rot[(size_t)i * (cols - 1) + k - 1].data + (size_t)pol * l * limb);
-                    }
-                    O.push_back(d->W[0].data + (size_t)pol * l * limb);
-                }
-            }
-            Scratch dA(c, A.size() * 8), dB(c, Bv.size() * 8), dO(c, O.size() * 8);
-            ew_dot(c->tabs, upload(c, dA, A), upload(c, dB, Bv), upload(c, dO, O), (int)O.size(), nch * cols, true, l,
-                   c->stream);
-        }
-        b0 = b1;
     }
 }
 

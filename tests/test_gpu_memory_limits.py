@@ -75,7 +75,8 @@ def one_hoisted(l):
 # levels of the documents, and the limbs that inference takes one document (and one level) at a time: the
 # accumulators, the rotated copies of a level's documents and one document's working space.  The rotations after
 # that take (2 l) + (l + l E + 2 E + 2 l) limbs per document beside the accumulators
-@pytest.mark.parametrize("levels,limbs", [([6] * 6, 6 * 12 + 6 * 7 * 12 + one_hoisted(6))])
+@pytest.mark.parametrize("levels,limbs", [([6] * 6, 6 * 12 + 6 * 7 * 12 + one_hoisted(6)),
+                                          ([6, 4, 6, 4, 4, 6], 3 * (12 + 8) + 3 * 86 + 3 * 50)])
 def test_diagonal_inference(ring, levels, limbs):
     pf, ctx = ring.pf, ring.ctx
     H, O = synth.fasttext_weights(5, N // 2, COLS, CLASSES)
