@@ -1178,7 +1178,15 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
         NEED(out[i], PFT_ERR_ARG, "null output");
         NEED(a[i]->level >= 2, PFT_ERR_LEVEL_MISMATCH, "rescale needs at least two primes");
     }
-    const size_t limb = c->n;
+    std::vector<int> lv;
+    std::vector<double> sc;
+    std::vector<int> order;  // by level: a handle given for several inputs ends with the highest level's result
+    for (int i = 0; i < B; i++) {
+        lv.push_back(a[i]->level);
+        sc.push_back(a[i]->scale / (double)c->primes[a[i]->level - 1]);
+        order.push_back(i);
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return lv[x] < lv[y]; });
     // fresh output buffers (the output is smaller than the input and may alias it)
     struct Fresh {
         pft_ctx* c;
@@ -1186,47 +1194,74 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
         ~Fresh() {
             for (u64* q : p) dfree(c, q);
         }
-    } nb{c, {}};
-    std::vector<double> sc;
-    for (int i = 0; i < B; i++) {
-        nb.p.push_back((u64*)dalloc(c, 2 * (size_t)(a[i]->level - 1) * limb * 8));
-        sc.push_back(a[i]->scale / (double)c->primes[a[i]->level - 1]);
-    }
-    std::vector<int> lv;
-    for (int i = 0; i < B; i++) lv.push_back(a[i]->level);
-    int i0 = 0;
-    while (i0 < B) {  // all levels together, in tiles that bound the working space
-        int i1 = i0;
-        size_t words = 0;
-        while (i1 < B) {
-            const size_t w = 2 * (size_t)lv[i1] * limb;
-            if (i1 > i0 && (words + w) * 8 > kRescaleScratchBudget) break;
-            words += w;
-            i1++;
+    } nb{c, std::vector<u64*>(B, nullptr)};
+    // entries [e0, e1) of `order`; PFT_ERR_OOM is thrown before any work is queued
+    auto part = [&](int e0, int e1) {
+        size_t total = 0, most = 0;
+        for (int e = e0; e < e1; e++) {
+            const int i = order[e];
+            const size_t w = 2 * (size_t)lv[i] * c->n;
+            nb.p[i] = (u64*)dalloc(c, 2 * (size_t)(lv[i] - 1) * c->n * 8);
+            total += w;
+            most = std::max(most, w);
         }
-        Scratch S(c, words * 8);
-        std::vector<PolyRef> in, o;
-        std::vector<u64*> last, rb;
-        u64* at = S.u();
-        for (int i = i0; i < i1; i++)
-            for (int pol = 0; pol < 2; pol++) {
-                in.push_back(cpoly(a[i]->data, lv[i], c->n, pol));
-                o.push_back(cpoly(nb.p[i], lv[i] - 1, c->n, pol));
-                last.push_back(at);
-                rb.push_back(at + limb);
-                at += (size_t)lv[i] * limb;
+        size_t room = std::max(most, std::min(total, kRescaleScratchBudget / 8));
+        std::unique_ptr<Scratch> S;
+        while (!S) {
+            try {
+                S.reset(new Scratch(c, room * 8));
+            } catch (const Error& err) {
+                if (err.code != PFT_ERR_OOM || room == most) throw;
+                room = std::max(most, room / 2);
             }
-        rescale_polys(c, in, last, rb, o);
-        i0 = i1;
+        }
+        for (int e = e0; e < e1;) {  // all levels together, in tiles of the working space
+            std::vector<PolyRef> in, o;
+            std::vector<u64*> last, rb;
+            u64* at = S->u();
+            for (; e < e1 && at + 2 * (size_t)lv[order[e]] * c->n <= S->u() + room; e++)
+                for (int pol = 0; pol < 2; pol++) {
+                    const int i = order[e];
+                    in.push_back(cpoly(a[i]->data, lv[i], c->n, pol));
+                    o.push_back(cpoly(nb.p[i], lv[i] - 1, c->n, pol));
+                    last.push_back(at);
+                    rb.push_back(at + c->n);
+                    at += (size_t)lv[i] * c->n;
+                }
+            rescale_polys(c, in, last, rb, o);
+        }
+    };
+    auto install = [&](int e0, int e1) {
+        for (int e = e0; e < e1; e++) {
+            const int i = order[e];
+            pft_ct* o = out[i];
+            dfree(c, o->data);  // stream-ordered: queued work on the old buffer completes first
+            o->data = nb.p[i];
+            nb.p[i] = nullptr;
+            o->cap = 2 * (size_t)(lv[i] - 1) * c->n;
+            o->level = lv[i] - 1;
+            o->scale = sc[i];
+        }
+    };
+    try {
+        part(0, B);
+        install(0, B);
+        return;
+    } catch (const Error& err) {
+        if (err.code != PFT_ERR_OOM || B == 0 || lv[order[0]] == lv[order[B - 1]]) throw;
+        std::map<const pft_ct*, int> written;  // an output that a later level still reads: all or nothing
+        for (int e = 0; e < B; e++) written.emplace(out[order[e]], lv[order[e]]);  // the lowest such level
+        for (int i = 0; i < B; i++)
+            if (written.count(a[i]) && written[a[i]] < lv[i]) throw;
     }
-    for (int i = 0; i < B; i++) {
-        pft_ct* o = out[i];
-        dfree(c, o->data);  // stream-ordered: queued work on the old buffer completes first
-        o->data = nb.p[i];
-        nb.p[i] = nullptr;
-        o->cap = 2 * (size_t)(lv[i] - 1) * limb;
-        o->level = lv[i] - 1;
-        o->scale = sc[i];
+    for (u64*& q : nb.p) {
+        dfree(c, q);
+        q = nullptr;
+    }
+    for (int e0 = 0, e1 = 0; e0 < B; e0 = e1) {  // no room for the outputs of all levels: level by level
+        while (e1 < B && lv[order[e1]] == lv[order[e0]]) e1++;
+        part(e0, e1);
+        install(e0, e1);
     }
 }
 

@@ -110,3 +110,49 @@ def test_refused_hoisted_rotation_leaves_outputs(ring, spare):
         assert np.array_equal(g, w)
     pf.pft_rotate_hoisted(ctx, a, [1, 2, 3], outs)
     pf.pft_device_status(ctx)
+
+
+def test_rescale_of_mixed_levels(ring):
+    """Room for the outputs and the working space of the largest level alone; one call in place."""
+    pf, ctx = ring.pf, ring.ctx
+    levels = [6, 2, 5, 3, 4, 6, 2, 5, 3, 4]
+    a = [ring.ct(l, 40 + i) for i, l in enumerate(levels)]
+    outs = [ring.empty() for _ in levels]
+    pf.pft_rescale_batch(ctx, a, outs)
+    want = ring.words(outs)
+    ring.alloc.cap = ring.settle() + (2 * 10 + 2 * 12 + 4) * LIMB
+    pf.pft_rescale_batch(ctx, a, a)
+    ring.alloc.cap = None
+    for g, w, l in zip(ring.words(a), want, levels):
+        assert np.array_equal(g, w) and len(g[0]) == l - 1
+
+
+def test_rescale_working_space_shrinks(ring):
+    """All of one level: the outputs and one ciphertext's working space; then too little for the outputs."""
+    pf, ctx = ring.pf, ring.ctx
+    a = [ring.ct(5, 60 + i) for i in range(6)]
+    outs = [ring.empty() for _ in a]
+    pf.pft_rescale_batch(ctx, a, outs)
+    want = ring.words(outs)
+    base = ring.settle()
+    ring.alloc.cap = base + (6 * 8 + 10 + 4) * LIMB
+    pf.pft_rescale_batch(ctx, a, outs)
+    ring.alloc.cap = base + 5 * 8 * LIMB
+    with pytest.raises(pf.PftError) as e:
+        pf.pft_rescale_batch(ctx, a, a)
+    assert e.value.code == pf.PFT_ERR_OOM
+    ring.alloc.cap = None
+    assert [pf.pft_ct_level(h) for h in a] == [5] * 6
+    pf.pft_rescale_batch(ctx, a, a)
+    for g, h, w in zip(ring.words(a), ring.words(outs), want):
+        assert np.array_equal(g, w) and np.array_equal(h, w)
+
+
+def test_rescale_repeated_output(ring):
+    """A handle given for several inputs ends with the result of the highest level, then of the last of that level."""
+    pf, ctx = ring.pf, ring.ctx
+    a = [ring.ct(l, 80 + i) for i, l in enumerate([3, 5, 5, 4])]
+    want, out = ring.empty(), ring.empty()
+    pf.pft_rescale(ctx, a[2], want)
+    pf.pft_rescale_batch(ctx, a, [out] * 4)
+    assert np.array_equal(pf.pft_ct_export(ctx, out), pf.pft_ct_export(ctx, want))
