@@ -18,9 +18,12 @@ namespace pft {
 // Programmatic dependent launch.  A kernel started by launch_pdl becomes resident as the CTAs of the
 // kernel before it on the stream run out; pdl_wait returns when everything before this kernel has
 // completed and is visible.  Before pdl_wait a kernel reads only its parameters and the context's
-// constant tables.  (Letting the next kernel in earlier, with griddepcontrol.launch_dependents at the
-// start, measured slower: its waiting CTAs hold the slots.  One rotation at level 30: 481 us with
-// ordinary launches, 486 with the early trigger, 453 without.)
+// constant tables.  Operands are read after it, with plain loads through plain pointers: __ldg
+// (ld.global.nc) is for data that nothing writes during the kernel's whole life, which begins here
+// before the previous kernel's words are visible, and neither it nor a __restrict__ pointer's load
+// is ordered by the wait.  (Letting the next kernel in earlier, with griddepcontrol.launch_dependents
+// at the start, measured slower: its waiting CTAs hold the slots.  One rotation at level 30: 481 us
+// with ordinary launches, 486 with the early trigger, 453 without.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ u64 mulhi(u64 a, u64 b) { return __umul64hi(a, b); }

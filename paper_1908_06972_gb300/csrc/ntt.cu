@@ -484,7 +484,7 @@ __device__ __forceinline__ const ulonglong2* lm_base(const ulonglong2* rows, int
 // src): canonical results are left in sm, row c2 point m at c2 * kRowStride + m + (m >> 4),
 // after a barrier.
 template <int SA, bool PRE>
-__device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* __restrict__ src, int pi, u64* sm) {
+__device__ __forceinline__ void fwd_rows(const DevTables& t, const u64* src, int pi, u64* sm) {
     constexpr int R = rows_per_cta(SA), TOP = SA + 7;
     const int w = threadIdx.x & 15, cc = threadIdx.x >> 4;
     const int u = blockIdx.x * R + cc;
@@ -615,10 +615,10 @@ __global__ void __launch_bounds__(row_threads(SA), min_ctas(MT, row_threads(SA))
     if (limb >= Ri.nlimbs) return;
     const int pi = prime_of(Ri, limb);
     const size_t base = (size_t)limb << logn;
-    const u64* __restrict__ xs = e.x[poly] + base;
-    const u64* __restrict__ as = e.acc[poly];        // null: no accumulator for this polynomial
+    const u64* xs = e.x[poly] + base;
+    const u64* as = e.acc[poly];                     // null: no accumulator for this polynomial
     const u32 g = PERM ? e.g[poly] : 0;              // above 1: the accumulator is read through X -> X^g
-    u64* __restrict__ os = e.out[poly] + base;
+    u64* os = e.out[poly] + base;
     const u64* cs = e.consts[poly] + 3 * limb;
     if (PRE || (flags & kPassPrefetch)) pdl_wait();
     if (flags & kPassPrefetch) {

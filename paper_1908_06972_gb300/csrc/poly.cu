@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(256) k_automorph_blocked(DevTables t, PolySet 
 #pragma unroll
     for (int k = 0; k < kAutBlocks; k++) {
         const u32 ib = automorph_src(o0 + k * kAutBlock, logn, g) & ~(u32)(kAutBlock - 1);
-        sm[k * kAutBlock + threadIdx.x] = __ldg(src + ib + threadIdx.x);
+        sm[k * kAutBlock + threadIdx.x] = src[ib + threadIdx.x];
     }
     __syncthreads();
 #pragma unroll
@@ -1425,7 +1425,7 @@ __global__ void k_rescale_bcast(DevTables t, PolySet last, PolySet out) {
     if (x >= t.n) return;
     const int lp = Ro.nlimbs;  // index of the dropped prime
     const u64 p = __ldg(&t.primes[lp].q);
-    u64 r = __ldg(last.p[poly].ptr + x) + (p >> 1);
+    u64 r = last.p[poly].ptr[x] + (p >> 1);
     if (r >= p) r -= p;
     const DPrime P = load_prime(t.primes, limb);
     Ro.ptr[((size_t)limb << t.logn) + x] = submod(reduce64(r, P), reduce64(p >> 1, P), P.q);
