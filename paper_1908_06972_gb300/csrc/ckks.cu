@@ -73,29 +73,29 @@ static bool capturing(pft_ctx* c) {
     return s != cudaStreamCaptureStatusNone;
 }
 void release_blocks(pft_ctx* c) {
-    std::deque<BlockCache::Block> out;
+    std::map<u64, BlockCache::Block> out;
     {
         std::lock_guard<std::mutex> g(c->blocks.mu);
         out.swap(c->blocks.kept);
+        c->blocks.by_size.clear();
         c->blocks.kept_bytes = 0;
     }
-    for (auto& b : out) raw_free(c, b.p);
+    for (auto& b : out) raw_free(c, b.second.p);
 }
 void* dalloc(pft_ctx* c, size_t bytes) {
     if (bytes == 0) return nullptr;
     BlockCache& B = c->blocks;
     const bool small = bytes <= BlockCache::kMaxBlock && !capturing(c);
     if (small) {
-        // the newest kept block that fits without wasting more than a quarter of it
+        // the smallest kept block that fits, if no more than a quarter of it is wasted; the newest of its size
         std::lock_guard<std::mutex> g(B.mu);
-        for (auto it = B.kept.rbegin(); it != B.kept.rend(); ++it)
-            if (it->bytes >= bytes && it->bytes - bytes <= it->bytes / 4) {
-                const BlockCache::Block b = *it;
-                B.kept.erase(std::next(it).base());
-                B.kept_bytes -= b.bytes;
-                B.live[b.p] = {b.bytes, c->stream};
-                return b.p;
-            }
+        const auto fit = B.by_size.lower_bound({bytes, 0});
+        if (fit != B.by_size.end() && fit->first - bytes <= fit->first / 4) {
+            const auto newest = *std::prev(B.by_size.upper_bound({fit->first, ~0ull}));
+            void* p = B.kept.find(newest.second)->second.p;
+            B.live[p] = {newest.first, c->stream};
+            return B.take(newest.second);
+        }
     }
     void* p = raw_alloc(c, bytes);
     if (!p) {
@@ -105,32 +105,38 @@ void* dalloc(pft_ctx* c, size_t bytes) {
     if (!p) fail(PFT_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
     if (small) {
         std::lock_guard<std::mutex> g(B.mu);
-        B.live[p] = {bytes, c->stream};
+        try {
+            B.live[p] = {bytes, c->stream};
+        } catch (const std::bad_alloc&) {  // a block that is not listed goes straight back when it is freed
+        }
     }
     return p;
 }
 void dfree(pft_ctx* c, void* p) {
     if (!p) return;
     BlockCache& B = c->blocks;
-    std::vector<void*> out;
+    bool kept = !capturing(c);
     {
-        const bool keep = !capturing(c);
         std::lock_guard<std::mutex> g(B.mu);
-        auto it = B.live.find(p);
-        if (it == B.live.end() || !keep || it->second.second != c->stream) {
-            out.push_back(p);
-        } else {
-            B.kept.push_back({p, it->second.first});
-            B.kept_bytes += it->second.first;
-            while (B.kept_bytes > BlockCache::kMaxCached) {
-                out.push_back(B.kept.front().p);
-                B.kept_bytes -= B.kept.front().bytes;
-                B.kept.pop_front();
-            }
+        const auto it = B.live.find(p);
+        kept = kept && it != B.live.end() && it->second.second == c->stream;
+        try {
+            if (kept) B.keep(p, it->second.first);
+        } catch (const std::bad_alloc&) {
+            kept = false;
         }
         if (it != B.live.end()) B.live.erase(it);
     }
-    for (void* q : out) raw_free(c, q);
+    if (!kept) raw_free(c, p);
+    for (;;) {
+        void* old = nullptr;
+        {
+            std::lock_guard<std::mutex> g(B.mu);
+            if (B.over()) old = B.take(B.kept.begin()->first);
+        }
+        if (!old) return;
+        raw_free(c, old);
+    }
 }
 
 // ---- context construction ---------------------------------------------------------------

@@ -1,10 +1,10 @@
 // Handles of the evaluator and the host-side helpers shared by its translation units
 // (the operations in ckks.cu, the request server in serve.cu).
 #pragma once
-#include <deque>
 #include <map>
 #include <memory>
 #include <mutex>
+#include <set>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -25,17 +25,42 @@ using namespace pft;
 // context's stream changes and when the context is destroyed.  Stream order makes reuse safe as it
 // does for the allocators: a block is kept only if it was allocated and freed on the stream that is
 // current, and never while that stream is being captured (a graph's memory must stay its own).
-// Callers may destroy handles from other threads, so the lists have a lock.
+// Callers may destroy handles from other threads, so the lists have a lock.  The kept blocks are ordered by
+// size besides: a program that freed thousands of handles pays no walk over them on each allocation.
 struct BlockCache {
-    static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)1 << 30;
+    static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)1 << 30, kMaxBlocks = (size_t)1 << 16;
     struct Block {
         void* p;
         size_t bytes;
     };
     std::mutex mu;
     std::unordered_map<void*, std::pair<size_t, cudaStream_t>> live;  // blocks up to kMaxBlock in use
-    std::deque<Block> kept;                                           // oldest first
+    std::map<u64, Block> kept;                                        // by number: oldest first
+    std::set<std::pair<size_t, u64>> by_size;                         // (bytes, number) of the kept blocks
+    u64 next = 0;                                                     // number of the next kept block
     size_t kept_bytes = 0;
+
+    // with mu held
+    void keep(void* p, size_t bytes) {
+        const auto it = kept.emplace(next, Block{p, bytes}).first;
+        try {
+            by_size.emplace(bytes, next);
+        } catch (...) {
+            kept.erase(it);
+            throw;
+        }
+        next++;
+        kept_bytes += bytes;
+    }
+    void* take(u64 number) {
+        const auto it = kept.find(number);
+        void* p = it->second.p;
+        by_size.erase({it->second.bytes, number});
+        kept_bytes -= it->second.bytes;
+        kept.erase(it);
+        return p;
+    }
+    bool over() const { return kept_bytes > kMaxCached || kept.size() > kMaxBlocks; }
 };
 
 // ---- handles ---------------------------------------------------------------------------
