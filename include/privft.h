@@ -124,7 +124,9 @@ typedef struct {
  * device.  `alloc` may be NULL.  Errors: ARG, SECURITY, OOM, CUDA. */
 int pft_ctx_create(const pft_params* params, const pft_allocator* alloc, pft_ctx** out);
 int pft_ctx_destroy(pft_ctx* ctx);
-/* Set the cudaStream_t (passed as void*) on which all later work is queued. */
+/* Set the cudaStream_t (passed as void*) on which all later work is queued.  The stream that is left
+ * may have been destroyed already; what the context kept on it is freed (on a stream of the
+ * context's own, which an allocator's free is then given) once the work queued there is done. */
 int pft_set_stream(pft_ctx* ctx, void* stream);
 const char* pft_last_error(pft_ctx* ctx);
 /* Chain info: N, L, k, alpha; primes_out (may be NULL) receives [L + k] primes. */

@@ -60,10 +60,16 @@ static void* raw_alloc(pft_ctx* c, size_t bytes) {
     }
     return p;
 }
-static void raw_free(pft_ctx* c, void* p) {
-    if (c->has_alloc) c->alloc.free(p, (void*)c->stream, c->alloc.user);
-    else cudaFreeAsync(p, c->stream);
+static bool raw_free(pft_ctx* c, void* p, cudaStream_t st) {
+    if (c->has_alloc) {
+        c->alloc.free(p, (void*)st, c->alloc.user);
+        return true;
+    }
+    if (cudaFreeAsync(p, st) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
 }
+static bool default_stream(cudaStream_t st) { return st == nullptr || st == cudaStreamLegacy; }
 static bool capturing(pft_ctx* c) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &s) != cudaSuccess) {
@@ -72,15 +78,57 @@ static bool capturing(pft_ctx* c) {
     }
     return s != cudaStreamCaptureStatusNone;
 }
+// gives blocks back, freed on `st`
+static void give_back(pft_ctx* c, const std::map<u64, BlockCache::Block>& out, cudaStream_t st) {
+    for (auto& b : out)
+        if (!raw_free(c, b.second.p, st)) {
+            std::lock_guard<std::mutex> g(c->blocks.mu);
+            c->blocks.stuck.push_back(b.second.p);
+        }
+}
 void release_blocks(pft_ctx* c) {
     std::map<u64, BlockCache::Block> out;
     {
         std::lock_guard<std::mutex> g(c->blocks.mu);
-        out.swap(c->blocks.kept);
-        c->blocks.by_size.clear();
-        c->blocks.kept_bytes = 0;
+        out = c->blocks.take_all();
     }
-    for (auto& b : out) raw_free(c, b.second.p);
+    give_back(c, out, c->stream);
+}
+void mark_blocks(pft_ctx* c) {
+    BlockCache& B = c->blocks;
+    if (default_stream(c->stream)) return;
+    std::lock_guard<std::mutex> g(B.mu);
+    if (B.marked == B.next || capturing(c)) return;  // a captured event would not be one to wait for
+    if (!B.mark && cudaEventCreateWithFlags(&B.mark, cudaEventDisableTiming) != cudaSuccess) B.mark = nullptr;
+    if (B.mark && cudaEventRecord(B.mark, c->stream) == cudaSuccess) B.marked = B.next;
+    else cudaGetLastError();
+}
+void leave_stream(pft_ctx* c) {
+    if (default_stream(c->stream)) {
+        release_blocks(c);
+        return;
+    }
+    BlockCache& B = c->blocks;
+    std::map<u64, BlockCache::Block> out;
+    {
+        std::lock_guard<std::mutex> g(B.mu);
+        out = B.take_all();
+    }
+    if (out.empty()) return;
+    // calls that are unsafe beside a capture elsewhere in the process, and do no harm to it here
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool ok = B.side || cudaStreamCreateWithFlags(&B.side, cudaStreamNonBlocking) == cudaSuccess;
+    if (out.rbegin()->first < B.marked) ok = ok && cudaStreamWaitEvent(B.side, B.mark, 0) == cudaSuccess;
+    else ok = ok && cudaDeviceSynchronize() == cudaSuccess;  // kept outside any call since the mark
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (ok) {
+        give_back(c, out, B.side);
+    } else {
+        cudaGetLastError();
+        std::lock_guard<std::mutex> g(B.mu);
+        for (auto& b : out) B.stuck.push_back(b.second.p);
+    }
 }
 void* dalloc(pft_ctx* c, size_t bytes) {
     if (bytes == 0) return nullptr;
@@ -93,7 +141,7 @@ void* dalloc(pft_ctx* c, size_t bytes) {
         if (fit != B.by_size.end() && fit->first - bytes <= fit->first / 4) {
             const auto newest = *std::prev(B.by_size.upper_bound({fit->first, ~0ull}));
             void* p = B.kept.find(newest.second)->second.p;
-            B.live[p] = {newest.first, c->stream};
+            B.live[p] = {newest.first, B.id};
             return B.take(newest.second);
         }
     }
@@ -106,7 +154,7 @@ void* dalloc(pft_ctx* c, size_t bytes) {
     if (small) {
         std::lock_guard<std::mutex> g(B.mu);
         try {
-            B.live[p] = {bytes, c->stream};
+            B.live[p] = {bytes, B.id};
         } catch (const std::bad_alloc&) {  // a block that is not listed goes straight back when it is freed
         }
     }
@@ -119,7 +167,7 @@ void dfree(pft_ctx* c, void* p) {
     {
         std::lock_guard<std::mutex> g(B.mu);
         const auto it = B.live.find(p);
-        kept = kept && it != B.live.end() && it->second.second == c->stream;
+        kept = kept && it != B.live.end() && it->second.second == B.id;
         try {
             if (kept) B.keep(p, it->second.first);
         } catch (const std::bad_alloc&) {
@@ -127,7 +175,7 @@ void dfree(pft_ctx* c, void* p) {
         }
         if (it != B.live.end()) B.live.erase(it);
     }
-    if (!kept) raw_free(c, p);
+    if (!kept) raw_free(c, p, c->stream);
     for (;;) {
         void* old = nullptr;
         {
@@ -135,7 +183,7 @@ void dfree(pft_ctx* c, void* p) {
             if (B.over()) old = B.take(B.kept.begin()->first);
         }
         if (!old) return;
-        raw_free(c, old);
+        raw_free(c, old, c->stream);
     }
 }
 
@@ -1913,6 +1961,7 @@ int pft_ctx_create(const pft_params* prm, const pft_allocator* alloc, pft_ctx** 
             c->has_alloc = true;
         }
         PFT_CUDA(cudaGetDevice(&c->device));
+        PFT_CUDA(cudaStreamGetId(c->stream, &c->blocks.id));
         build_tables(c.get());
         c->noalloc_scratch = noalloc_scratch_lookup();
     });
@@ -1930,8 +1979,15 @@ int pft_ctx_destroy(pft_ctx* c) {
     free_keys(c);
     dfree(c, c->s_ntt);
     dfree(c, c->pk);
-    release_blocks(c);
+    leave_stream(c);
     cudaStreamSynchronize(c->stream);
+    if (c->blocks.side) cudaStreamSynchronize(c->blocks.side);
+    for (void* p : c->blocks.stuck) {
+        if (c->has_alloc) c->alloc.free(p, (void*)c->stream, c->alloc.user);
+        else cudaFree(p);
+    }
+    if (c->blocks.side) cudaStreamDestroy(c->blocks.side);
+    if (c->blocks.mark) cudaEventDestroy(c->blocks.mark);
     for (void* p : c->owned) cudaFree(p);
     delete c;
     return PFT_OK;
@@ -1939,8 +1995,13 @@ int pft_ctx_destroy(pft_ctx* c) {
 
 int pft_set_stream(pft_ctx* c, void* stream) {
     if (!c) return PFT_ERR_ARG;
-    if (c->stream != (cudaStream_t)stream) release_blocks(c);  // kept blocks belong to the old stream
+    unsigned long long id = 0;
+    if (cudaStreamGetId((cudaStream_t)stream, &id) != cudaSuccess) cudaGetLastError();
+    if (c->stream == (cudaStream_t)stream && c->blocks.id == id) return PFT_OK;
+    leave_stream(c);  // kept blocks belong to the old stream
+    std::lock_guard<std::mutex> g(c->blocks.mu);
     c->stream = (cudaStream_t)stream;
+    c->blocks.id = id;
     return PFT_OK;
 }
 
@@ -2056,6 +2117,7 @@ int pft_ct_destroy(pft_ct* ct) {
     if (!ct) return PFT_OK;
     if (!handle_live(ct)) return PFT_ERR_ARG;  // destroyed already, or never a handle
     dfree(ct->ctx, ct->data);
+    if (ct->ctx) mark_blocks(ct->ctx);
     delete ct;
     return PFT_OK;
 }
@@ -2063,6 +2125,7 @@ int pft_pt_destroy(pft_pt* pt) {
     if (!pt) return PFT_OK;
     if (!handle_live(pt)) return PFT_ERR_ARG;
     dfree(pt->ctx, pt->data);
+    if (pt->ctx) mark_blocks(pt->ctx);
     delete pt;
     return PFT_OK;
 }

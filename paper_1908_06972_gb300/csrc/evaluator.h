@@ -24,7 +24,12 @@ using namespace pft;
 // the oldest given back first; all are given back when the allocator refuses a request, when the
 // context's stream changes and when the context is destroyed.  Stream order makes reuse safe as it
 // does for the allocators: a block is kept only if it was allocated and freed on the stream that is
-// current, and never while that stream is being captured (a graph's memory must stay its own).
+// current, and never while that stream is being captured (a graph's memory must stay its own).  A stream
+// is told by its id, since a new one can have the handle of one that was destroyed.
+// A stream that is left may be gone already, so its handle is not used: every call that kept a block
+// records `mark` at its end (not on the default stream, which is always there: the record keeps the next
+// call's first kernel from starting early), and the blocks are freed on a stream of the context's own
+// that waits for the mark.
 // Callers may destroy handles from other threads, so the lists have a lock.  The kept blocks are ordered by
 // size besides: a program that freed thousands of handles pays no walk over them on each allocation.
 struct BlockCache {
@@ -34,11 +39,16 @@ struct BlockCache {
         size_t bytes;
     };
     std::mutex mu;
-    std::unordered_map<void*, std::pair<size_t, cudaStream_t>> live;  // blocks up to kMaxBlock in use
-    std::map<u64, Block> kept;                                        // by number: oldest first
-    std::set<std::pair<size_t, u64>> by_size;                         // (bytes, number) of the kept blocks
-    u64 next = 0;                                                     // number of the next kept block
+    std::unordered_map<void*, std::pair<size_t, unsigned long long>> live;  // blocks up to kMaxBlock in use: bytes, stream id
+    std::map<u64, Block> kept;                                              // by number: oldest first
+    std::set<std::pair<size_t, u64>> by_size;                               // (bytes, number) of the kept blocks
+    u64 next = 0;                                                           // number of the next kept block
     size_t kept_bytes = 0;
+    unsigned long long id = 0;     // of the current stream
+    cudaEvent_t mark = nullptr;    // follows the work of the blocks below number `marked`
+    u64 marked = 0;
+    cudaStream_t side = nullptr;   // where blocks of a stream that was left are freed
+    std::vector<void*> stuck;      // refused by their free (a stream under capture): freed with the context
 
     // with mu held
     void keep(void* p, size_t bytes) {
@@ -59,6 +69,13 @@ struct BlockCache {
         kept_bytes -= it->second.bytes;
         kept.erase(it);
         return p;
+    }
+    std::map<u64, Block> take_all() {
+        std::map<u64, Block> out;
+        out.swap(kept);
+        by_size.clear();
+        kept_bytes = 0;
+        return out;
     }
     bool over() const { return kept_bytes > kMaxCached || kept.size() > kMaxBlocks; }
 };
@@ -146,6 +163,10 @@ void* dalloc(pft_ctx* c, size_t bytes);
 void dfree(pft_ctx* c, void* p);
 // Gives every kept block back to the allocator.
 void release_blocks(pft_ctx* c);
+// The same without the current stream's handle, which may be gone.
+void leave_stream(pft_ctx* c);
+// The end of a call on c: the blocks it kept are followed by the context's mark.
+void mark_blocks(pft_ctx* c);
 struct Scratch {
     pft_ctx* c;
     void* p;
@@ -264,6 +285,12 @@ inline PolyRef cpoly(u64* data, int l, int n, int pol) { return ref(data + (size
 // ---- the C ABI guard ------------------------------------------------------------------
 template <class F>
 inline int guard(pft_ctx* c, F f) {
+    struct End {
+        pft_ctx* c;
+        ~End() {
+            if (c) mark_blocks(c);
+        }
+    } end{c};
     try {
         f();
         return PFT_OK;

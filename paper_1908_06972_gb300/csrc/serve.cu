@@ -265,6 +265,12 @@ static void step(pft_server* s) {
     admit(s);
     s->max_active = std::max<int>(s->max_active, (int)s->active.size());
     if (s->active.empty()) return;
+    struct End {
+        pft_server* s;
+        ~End() {
+            for (Ring& r : s->rings) mark_blocks(r.ctx);
+        }
+    } end{s};
     run_stages(s);
     const int cur = (int)(s->iterations & 1), prev = cur ^ 1;
     for (Ring& r : s->rings) {
@@ -334,6 +340,7 @@ int pft_server_destroy(pft_server* s) {
         cudaEventDestroy(r.t0);
         cudaEventDestroy(r.iter[0]);
         cudaEventDestroy(r.iter[1]);
+        mark_blocks(r.ctx);
     }
     delete s;
     return PFT_OK;

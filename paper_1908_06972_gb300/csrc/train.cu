@@ -673,7 +673,9 @@ int pft_ft_enc_model_levels(const pft_ft_enc_model* M, int* level_H, int* level_
 }
 
 int pft_ft_enc_model_destroy(pft_ft_enc_model* M) {
+    pft_ctx* c = M ? M->ctx : nullptr;
     delete M;
+    if (c) mark_blocks(c);
     return PFT_OK;
 }
 
@@ -742,7 +744,9 @@ int pft_fasttext_train_backward(pft_ctx* c, const pft_ft_tape* T, pft_ct* const*
 }
 
 int pft_ft_tape_destroy(pft_ft_tape* T) {
+    pft_ctx* c = T ? T->ctx : nullptr;
     delete T;
+    if (c) mark_blocks(c);
     return PFT_OK;
 }
 

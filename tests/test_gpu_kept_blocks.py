@@ -55,3 +55,88 @@ def test_many_kept_blocks_cost_nothing(gpu):
     for h in handles:
         pf.pft_ct_destroy(h)
     pf.pft_ctx_destroy(ctx)
+
+
+class Labelled:
+    """torch's caching allocator; records the stream that each free names."""
+
+    def __init__(self, pf):
+        self.live, self.freed_on = set(), []
+
+        def alloc(nbytes, stream, user):
+            p = torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+            self.live.add(p)
+            return p
+
+        def free(ptr, stream, user):
+            if ptr:
+                self.live.remove(ptr)
+                self.freed_on.append(int(stream or 0))
+                torch.cuda.caching_allocator_delete(ptr)
+
+        self.struct = pf.pft_allocator(pf.ALLOC_FN(alloc), pf.FREE_FN(free), None)
+
+
+def make(pf, alloc, stream, logn=12):
+    ctx = pf.pft_ctx_create(logn, 4, 1, 2, 60, 40, 60, 2.0 ** 40, SEED, flags=pf.PFT_ALLOW_INSECURE, allocator=alloc,
+                            stream=stream.cuda_stream)
+    pf.pft_keygen(ctx, [1], True)
+    return ctx
+
+
+def fresh(pf, ctx, level=4):
+    w = words(pf, ctx, level)
+    h = pf.pft_ct_create(ctx)
+    torch.cuda.synchronize()
+    pf.pft_ct_reduce_sum(ctx, w.data_ptr(), level, 2.0 ** 40, 1, h)
+    torch.cuda.synchronize()
+    return h
+
+
+@pytest.mark.parametrize("idle", [True, False])
+def test_a_stream_that_is_left_is_not_used_again(gpu, idle):
+    """The caller may have destroyed it: what was kept on it is freed elsewhere, after the work queued there."""
+    pf, alloc = gpu, Labelled(gpu)
+    left, other = torch.cuda.Stream(), torch.cuda.Stream()
+    ctx = make(pf, alloc.struct, left)
+    a, c, d = fresh(pf, ctx), pf.pft_ct_create(ctx), pf.pft_ct_create(ctx)
+    for _ in range(2):
+        pf.pft_mul_relin(ctx, a, a, c)
+    want = pf.pft_ct_export(ctx, c)
+    pf.pft_mul_relin(ctx, a, a, c)
+    pf.pft_ct_destroy(c)  # kept outside any call that does work
+    if idle:
+        torch.cuda.synchronize()
+    held, alloc.freed_on[:] = len(alloc.live), []
+    pf.pft_set_stream(ctx, other.cuda_stream)
+    assert len(alloc.live) < held, "the kept blocks are given back"
+    if not idle:
+        torch.cuda.synchronize()
+    pf.pft_mul_relin(ctx, a, a, d)
+    assert np.array_equal(pf.pft_ct_export(ctx, d), want)
+    pf.pft_ct_destroy(a)
+    pf.pft_ct_destroy(d)
+    pf.pft_ctx_destroy(ctx)
+    assert alloc.freed_on and left.cuda_stream not in alloc.freed_on
+    assert not alloc.live
+
+
+def test_streams_in_turn(gpu):
+    """Independent work on two streams through one context, nothing waited for between them."""
+    pf = gpu
+    s = [torch.cuda.Stream(), torch.cuda.Stream()]
+    ctx = make(pf, None, s[0], logn=14)
+    a = fresh(pf, ctx)
+    one = pf.pft_ct_create(ctx)
+    pf.pft_mul_relin(ctx, a, a, one)
+    want = pf.pft_ct_export(ctx, one)
+    outs = [pf.pft_ct_create(ctx) for _ in range(40)]
+    for i, h in enumerate(outs):
+        pf.pft_set_stream(ctx, s[i % 2].cuda_stream)
+        pf.pft_mul_relin(ctx, a, a, h)
+    torch.cuda.synchronize()
+    for h in outs:
+        assert np.array_equal(pf.pft_ct_export(ctx, h), want)
+    for h in outs + [a, one]:
+        pf.pft_ct_destroy(h)
+    pf.pft_ctx_destroy(ctx)
