@@ -146,7 +146,7 @@ void* dalloc(pft_ctx* c, size_t bytes) {
         }
     }
     void* p = raw_alloc(c, bytes);
-    if (!p) {
+    if (!p && !capturing(c)) {  // (the kept blocks are not the graph's: under capture they stay)
         release_blocks(c);
         p = raw_alloc(c, bytes);
     }

@@ -140,3 +140,36 @@ def test_streams_in_turn(gpu):
     for h in outs + [a, one]:
         pf.pft_ct_destroy(h)
     pf.pft_ctx_destroy(ctx)
+
+
+@pytest.mark.filterwarnings("ignore")
+def test_refusal_under_capture_keeps_the_blocks(gpu):
+    """Blocks that were kept before a capture are not freed into it: the call fails, and they serve the next one."""
+    from .test_gpu_faults import CappedAllocator
+
+    pf, alloc, st = gpu, CappedAllocator(gpu, torch), torch.cuda.Stream()
+    ctx = make(pf, alloc.struct, st)
+    a, c = fresh(pf, ctx), pf.pft_ct_create(ctx)
+    pf.pft_mul_relin(ctx, a, a, c)
+    want = pf.pft_ct_export(ctx, c)
+    pf.pft_mul_relin(ctx, a, a, c)
+    torch.cuda.synchronize()
+    held = set(alloc.live)
+    graph = torch.cuda.CUDAGraph()
+    alloc.cap = 0
+    with torch.cuda.stream(st):
+        graph.capture_begin(capture_error_mode="relaxed")
+        try:
+            with pytest.raises(pf.PftError) as e:
+                pf.pft_mul_relin(ctx, a, a, c)
+        finally:
+            graph.capture_end()
+    assert e.value.code == pf.PFT_ERR_OOM
+    assert set(alloc.live) == held
+    pf.pft_mul_relin(ctx, a, a, c)  # nothing new is needed
+    assert np.array_equal(pf.pft_ct_export(ctx, c), want)
+    alloc.cap = None
+    pf.pft_ct_destroy(a)
+    pf.pft_ct_destroy(c)
+    pf.pft_ctx_destroy(ctx)
+    assert alloc.in_use() == 0
