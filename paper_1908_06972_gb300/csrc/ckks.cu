@@ -135,14 +135,18 @@ void* dalloc(pft_ctx* c, size_t bytes) {
     BlockCache& B = c->blocks;
     const bool small = bytes <= BlockCache::kMaxBlock && !capturing(c);
     if (small) {
-        // the smallest kept block that fits, if no more than a quarter of it is wasted; the newest of its size
+        // the newest kept block that fits without wasting more than a quarter of it
         std::lock_guard<std::mutex> g(B.mu);
-        const auto fit = B.by_size.lower_bound({bytes, 0});
-        if (fit != B.by_size.end() && fit->first - bytes <= fit->first / 4) {
-            const auto newest = *std::prev(B.by_size.upper_bound({fit->first, ~0ull}));
-            void* p = B.kept.find(newest.second)->second.p;
-            B.live[p] = {newest.first, B.id};
-            return B.take(newest.second);
+        const std::pair<size_t, u64>* best = nullptr;
+        for (auto it = B.by_size.lower_bound({bytes, 0}); it != B.by_size.end() && it->first - bytes <= it->first / 4;) {
+            const auto end = B.by_size.upper_bound({it->first, ~0ull});  // of this size
+            const auto newest = std::prev(end);
+            if (!best || newest->second > best->second) best = &*newest;
+            it = end;
+        }
+        if (best) {
+            B.live[B.kept.find(best->second)->second.p] = {best->first, B.id};
+            return B.take(best->second);
         }
     }
     void* p = raw_alloc(c, bytes);
