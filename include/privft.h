@@ -73,8 +73,9 @@ typedef struct pft_ft_model pft_ft_model; /* packed fastText weights (H, O) */
 /* Device allocator.  alloc(bytes, stream, user) returns device memory usable on
  * `stream` (NULL on failure); free(ptr, stream, user) releases it once the work
  * already queued on `stream` no longer needs it.  A context keeps freed blocks of up to
- * 16 MiB (1 GiB at most) for its next calls on the same stream and frees them when an
- * allocation fails, pft_set_stream changes the stream or the context is destroyed. */
+ * 16 MiB (256 MiB at most) for its next calls on the same stream and frees them when an
+ * allocation fails (its own, or that of another context with the same device and allocator, from that
+ * context's thread), pft_set_stream changes the stream or the context is destroyed. */
 typedef struct {
     void* (*alloc)(size_t bytes, void* stream, void* user);
     void (*free)(void* ptr, void* stream, void* user);
@@ -489,7 +490,8 @@ int pft_fasttext_infer_batch(pft_ctx* ctx, const pft_ft_model* model, const pft_
  * products; one rotate-and-sum step; the output layer), requests at the same stage
  * of a ring forming one batched call.  It returns once the previous iteration has
  * finished on the device.  The key-switching work space of each call is allocated
- * per call besides the budget.  A result equals that of pft_fasttext_infer on the
+ * per call besides the budget, and so are the freed blocks that each ring's context keeps
+ * (pft_allocator; they are given back before a request for memory fails).  A result equals that of pft_fasttext_infer on the
  * same input, whatever else was in flight.  Destroy the server before its contexts
  * and models.  Calls on one server must not overlap;
  * after an error other than PFT_ERR_ARG / _LEVEL_MISMATCH / _OOM from

@@ -199,12 +199,16 @@ def _arr(handles):
 
 
 # ---- allocator backed by torch's caching allocator ---------------------------------------
-_KEEP = []
+_TORCH = {}
 
 
 def torch_allocator(device=0):
-    """A pft_allocator whose memory comes from torch's CUDA caching allocator."""
+    """The pft_allocator whose memory comes from torch's CUDA caching allocator (one per device: contexts that
+    share it can have each other's kept blocks when torch has no more)."""
     import torch
+
+    if device in _TORCH:
+        return _TORCH[device]
 
     def _alloc(nbytes, stream, user):
         try:
@@ -216,9 +220,7 @@ def torch_allocator(device=0):
         if ptr:
             torch.cuda.caching_allocator_delete(ptr)
 
-    a = pft_allocator(ALLOC_FN(_alloc), FREE_FN(_free), None)
-    _KEEP.append(a)
-    return a
+    return _TORCH.setdefault(device, pft_allocator(ALLOC_FN(_alloc), FREE_FN(_free), None))
 
 
 # ---- context --------------------------------------------------------------------------------

@@ -90,7 +90,7 @@ void release_blocks(pft_ctx* c) {
     std::map<u64, BlockCache::Block> out;
     {
         std::lock_guard<std::mutex> g(c->blocks.mu);
-        out = c->blocks.take_all();
+        out = c->blocks.take_below(c->blocks.next);
     }
     give_back(c, out, c->stream);
 }
@@ -103,31 +103,54 @@ void mark_blocks(pft_ctx* c) {
     if (B.mark && cudaEventRecord(B.mark, c->stream) == cudaSuccess) B.marked = B.next;
     else cudaGetLastError();
 }
-void leave_stream(pft_ctx* c) {
-    if (default_stream(c->stream)) {
-        release_blocks(c);
-        return;
-    }
+// Frees kept blocks without the stream they were kept on: those that a mark follows, or all of them.
+static void give_back_beside(pft_ctx* c, bool all) {
     BlockCache& B = c->blocks;
     std::map<u64, BlockCache::Block> out;
+    cudaStream_t st = nullptr;
+    bool ok = true;
     {
         std::lock_guard<std::mutex> g(B.mu);
-        out = B.take_all();
+        const bool def = default_stream(c->stream);
+        out = B.take_below(def || all ? B.next : B.marked);
+        if (out.empty()) return;
+        if (def) {
+            st = c->stream;
+        } else {
+            // calls that are unsafe beside a capture elsewhere in the process, and do no harm to it here
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            ok = B.side || cudaStreamCreateWithFlags(&B.side, cudaStreamNonBlocking) == cudaSuccess;
+            if (out.rbegin()->first < B.marked) ok = ok && cudaStreamWaitEvent(B.side, B.mark, 0) == cudaSuccess;
+            else ok = ok && cudaDeviceSynchronize() == cudaSuccess;  // kept outside any call since the mark
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            st = B.side;
+            if (!ok) {
+                cudaGetLastError();
+                for (auto& b : out) B.stuck.push_back(b.second.p);
+            }
+        }
     }
-    if (out.empty()) return;
-    // calls that are unsafe beside a capture elsewhere in the process, and do no harm to it here
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    bool ok = B.side || cudaStreamCreateWithFlags(&B.side, cudaStreamNonBlocking) == cudaSuccess;
-    if (out.rbegin()->first < B.marked) ok = ok && cudaStreamWaitEvent(B.side, B.mark, 0) == cudaSuccess;
-    else ok = ok && cudaDeviceSynchronize() == cudaSuccess;  // kept outside any call since the mark
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (ok) {
-        give_back(c, out, B.side);
-    } else {
-        cudaGetLastError();
-        std::lock_guard<std::mutex> g(B.mu);
-        for (auto& b : out) B.stuck.push_back(b.second.p);
+    if (ok) give_back(c, out, st);
+}
+void leave_stream(pft_ctx* c) { give_back_beside(c, true); }
+// The contexts that exist, and what those with c's device and allocator keep: memory that c's next request
+// could have.  Their threads may be in calls, so only blocks behind a mark go.
+static std::mutex& ctxs_mu() {
+    static std::mutex m;
+    return m;
+}
+static std::set<pft_ctx*>& ctxs() {
+    static std::set<pft_ctx*> s;
+    return s;
+}
+static void release_others(pft_ctx* c) {
+    std::lock_guard<std::mutex> g(ctxs_mu());
+    for (pft_ctx* o : ctxs()) {
+        const pft_allocator &x = c->alloc, &y = o->alloc;
+        const bool same = c->has_alloc == o->has_alloc &&
+                          (!c->has_alloc || (x.alloc == y.alloc && x.free == y.free && x.user == y.user));
+        if (o != c && o->device == c->device && same) give_back_beside(o, false);
     }
 }
 void* dalloc(pft_ctx* c, size_t bytes) {
@@ -153,6 +176,10 @@ void* dalloc(pft_ctx* c, size_t bytes) {
     if (!p && !capturing(c)) {  // (the kept blocks are not the graph's: under capture they stay)
         release_blocks(c);
         p = raw_alloc(c, bytes);
+        if (!p) {
+            release_others(c);
+            p = raw_alloc(c, bytes);
+        }
     }
     if (!p) fail(PFT_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
     if (small) {
@@ -1973,12 +2000,20 @@ int pft_ctx_create(const pft_params* prm, const pft_allocator* alloc, pft_ctx** 
         for (void* p : c->owned) cudaFree(p);
         return rc;
     }
+    {
+        std::lock_guard<std::mutex> g(ctxs_mu());
+        ctxs().insert(c.get());
+    }
     *out = c.release();
     return PFT_OK;
 }
 
 int pft_ctx_destroy(pft_ctx* c) {
     if (!c) return PFT_OK;
+    {
+        std::lock_guard<std::mutex> g(ctxs_mu());
+        ctxs().erase(c);
+    }
     cudaStreamSynchronize(c->stream);
     free_keys(c);
     dfree(c, c->s_ntt);

@@ -173,3 +173,60 @@ def test_refusal_under_capture_keeps_the_blocks(gpu):
     pf.pft_ct_destroy(c)
     pf.pft_ctx_destroy(ctx)
     assert alloc.in_use() == 0
+
+
+@pytest.mark.parametrize("own_streams", [False, True])
+def test_another_contexts_blocks_are_given_back(gpu, own_streams):
+    """Two contexts with one allocator: what one keeps does not refuse the other a request."""
+    from .test_gpu_faults import CappedAllocator
+
+    pf, alloc = gpu, CappedAllocator(gpu, torch)
+    st = [torch.cuda.Stream() if own_streams else torch.cuda.default_stream() for _ in range(2)]
+    one, two = [make(pf, alloc.struct, s) for s in st]
+    a, b = fresh(pf, one), fresh(pf, two)
+    c, d = pf.pft_ct_create(one), pf.pft_ct_create(two)
+    pf.pft_mul_relin(two, b, b, d)
+    want = pf.pft_ct_export(two, d)
+    pf.pft_ct_destroy(d)
+    torch.cuda.synchronize()
+    alloc.cap = 0
+    big = [pf.pft_ct_create(two) for _ in range(64)]
+    with pytest.raises(pf.PftError):  # the second context's kept blocks go back (and the first one's)
+        pf.pft_mul_relin_batch(two, [b] * 64, [b] * 64, big)
+    alloc.cap = None
+    pf.pft_mul_relin(one, a, a, c)
+    torch.cuda.synchronize()
+    alloc.cap = alloc.in_use() + 2 * 4 * 8 * 4096 + 4096  # the product; its working space is kept by the first
+    pf.pft_mul_relin(two, b, b, big[0])
+    assert np.array_equal(pf.pft_ct_export(two, big[0]), want)
+    alloc.cap = None
+    pf.pft_mul_relin(one, a, a, c)
+    for h in [a, b, c] + big:
+        pf.pft_ct_destroy(h)
+    pf.pft_ctx_destroy(one)
+    pf.pft_ctx_destroy(two)
+    assert alloc.in_use() == 0
+
+
+def test_torch_allocator_is_one(gpu):
+    assert gpu.torch_allocator() is gpu.torch_allocator()
+
+
+def test_what_a_context_keeps_is_small(gpu):
+    """Freed handles: at most 256 MiB stay with the context."""
+    from .test_gpu_faults import CappedAllocator
+
+    pf, alloc = gpu, CappedAllocator(gpu, torch)
+    ctx = make(pf, alloc.struct, torch.cuda.default_stream(), logn=16)
+    w = words(pf, ctx, 4)
+    torch.cuda.synchronize()
+    base = alloc.in_use()
+    hs = [pf.pft_ct_create(ctx) for _ in range(100)]  # 4 MiB each
+    for h in hs:
+        pf.pft_ct_reduce_sum(ctx, w.data_ptr(), 4, 2.0 ** 40, 1, h)
+    for h in hs:
+        pf.pft_ct_destroy(h)
+    torch.cuda.synchronize()
+    assert alloc.in_use() <= base + (256 << 20)
+    pf.pft_ctx_destroy(ctx)
+    assert alloc.in_use() == 0
