@@ -20,17 +20,18 @@ using namespace pft;
 
 // Freed device blocks that a context keeps for its next calls.  A call of a small ring allocates and
 // frees about ten short-lived blocks; through a caller's allocator (a callback into Python for
-// torch's) these cost more than its kernels.  Bounded: blocks up to kMaxBlock, kMaxCached bytes in all (1 GiB is
-// no faster: within 0.1 % in 32 rotation-light inferences and in every smaller call; 128 MiB 0.4 % slower there), the oldest given back first; all are given back when the allocator refuses a request (of this context, or
-// of another one with the same device and allocator), when the context's stream changes and when the
-// context is destroyed.  Stream order makes reuse safe as it
-// does for the allocators: a block is kept only if it was allocated and freed on the stream that is
-// current, and never while that stream is being captured (a graph's memory must stay its own).  A stream
-// is told by its id, since a new one can have the handle of one that was destroyed.
-// A stream that is left may be gone already, so its handle is not used: every call that kept a block
-// records `mark` at its end (not on the default stream, which is always there: the record keeps the next
-// call's first kernel from starting early), and the blocks are freed on a stream of the context's own
-// that waits for the mark.
+// torch's) these cost more than its kernels.  Bounded: blocks up to kMaxBlock, kMaxCached bytes in all,
+// the oldest given back first (1 GiB is no faster: within 0.1 % in 32 rotation-light inferences and in every
+// smaller call; 128 MiB 0.4 % slower there).  All are given back when the allocator refuses a request (of this
+// context, or of another one with the same device and allocator), when the context's stream changes and
+// when the context is destroyed.
+// Stream order makes reuse safe as it does for the allocators: a block is kept only if it was allocated
+// and freed on the stream that is current, and never while that stream is being captured (a graph's
+// memory must stay its own).  A stream is told by its id, since a new one can have the handle of one
+// that was destroyed.  A stream that is left may be gone already, so its handle is not used: every call
+// that kept a block on a stream of the caller's records `mark` at its end (no cost was measured: HMUL, RESCALE
+// and ROTATE at N = 2^13 are 89.3 us with and without), and the blocks are freed on a stream of the context's
+// own that waits for the mark.  The default stream is always there.
 // Callers may destroy handles from other threads, so the lists have a lock.  The kept blocks are ordered by
 // size besides: a program that freed thousands of handles pays no walk over them on each allocation.
 struct BlockCache {
