@@ -364,7 +364,7 @@ int pft_rotate_batch(pft_ctx* ctx, const pft_ct* const* a, int B, int32_t step, 
  * 6+10, 10+6, 7+9, 9+7, 5+5+6; N = 2^15: 8+7, 7+8, 9+6, 6+9, 5+5+5, then the two specialised
  * ones; N <= 2^14 has a single plan).  For each launch-size bucket (total limbs of a
  * launch: <= 64, <= 512, larger) every plan is timed on a forward + inverse transform of a
- * representative launch (32, 256, 1024 limbs; median of 3 CUDA-event timings on the context's
+ * representative launch (64, 256, 1024 limbs; median of 3 CUDA-event timings on the context's
  * stream) and the fastest is kept for launches of that size.  us_out (may be NULL) receives up
  * to `cap` plan times (microseconds) of the largest bucket, *chosen its choice (an index into
  * the plan list of pft_autotune_report).  Synchronous.  The environment variable PFT_NTT16

@@ -2605,7 +2605,7 @@ int pft_rotate_batch(pft_ctx* c, const pft_ct* const* a, int B, int32_t step, pf
 // The autotuner: for each launch-size bucket (by the launch's total limbs: <= 64, <= 512, larger)
 // it times every transform plan of the ring (ntt_candidates: the specialised kernels and generic
 // staged passes of several stage splits and tile widths) on a forward + inverse transform of a
-// representative launch (32, 256 and 1024 limbs of the chain's primes), median of 3, and keeps
+// representative launch (64, 256 and 1024 limbs of the chain's primes), median of 3, and keeps
 // the fastest plan for that bucket.
 int pft_autotune(pft_ctx* c, double* us_out, int cap, int* chosen) {
     return guard(c, [&] {
@@ -2618,7 +2618,10 @@ int pft_autotune(pft_ctx* c, double* us_out, int cap, int* chosen) {
         int best_last = 0;
         std::vector<double> us_last(std::max(nc, 1), 0.0);
         if (nc > 1) {
-            const int reps_limbs[kNttBuckets] = {32, 256, 1024};
+            // the first at its bucket's end: launches of up to 38 limbs at N = 2^15 and 19 at 2^16 run in one form
+            // whatever the two-pass plan (kPreThreadsPerSm), so that timing such a launch chooses by noise
+            // for the larger ones of the bucket
+            const int reps_limbs[kNttBuckets] = {64, 256, 1024};
             const int limbs = std::min(c->L + c->k, 32);
             cudaEvent_t e0, e1;
             PFT_CUDA(cudaEventCreate(&e0));
