@@ -79,18 +79,19 @@ static bool capturing(pft_ctx* c) {
     return s != cudaStreamCaptureStatusNone;
 }
 // gives blocks back, freed on `st`
-static void give_back(pft_ctx* c, const std::map<u64, BlockCache::Block>& out, cudaStream_t st) {
-    for (auto& b : out)
-        if (!raw_free(c, b.second.p, st)) {
-            std::lock_guard<std::mutex> g(c->blocks.mu);
-            c->blocks.stuck.push_back(b.second.p);
-        }
+static void give_back(pft_ctx* c, const BlockCache::Sizes& out, cudaStream_t st) {
+    for (auto& s : out)
+        for (size_t i = s.second.head; i < s.second.v.size(); i++)
+            if (!raw_free(c, s.second.v[i].p, st)) {
+                std::lock_guard<std::mutex> g(c->blocks.mu);
+                c->blocks.stuck.push_back(s.second.v[i].p);
+            }
 }
 void release_blocks(pft_ctx* c) {
-    std::map<u64, BlockCache::Block> out;
+    BlockCache::Sizes out;
     {
         std::lock_guard<std::mutex> g(c->blocks.mu);
-        out = c->blocks.take_below(c->blocks.next);
+        out = c->blocks.take_all();
     }
     give_back(c, out, c->stream);
 }
@@ -106,14 +107,18 @@ void mark_blocks(pft_ctx* c) {
 // Frees kept blocks without the stream they were kept on: those that a mark follows, or all of them.
 static void give_back_beside(pft_ctx* c, bool all) {
     BlockCache& B = c->blocks;
-    std::map<u64, BlockCache::Block> out;
+    BlockCache::Sizes out;
     cudaStream_t st = nullptr;
     bool ok = true;
     {
         std::lock_guard<std::mutex> g(B.mu);
         const bool def = default_stream(c->stream);
-        out = B.take_below(def || all ? B.next : B.marked);
-        if (out.empty()) return;
+        if (B.blocks == 0) return;
+        out = def || all ? B.take_all() : B.take_marked();
+        u64 end = 0;  // above the newest block's number
+        for (auto& s : out)
+            if (!s.second.empty()) end = std::max(end, s.second.v.back().number + 1);
+        if (end == 0) return;
         if (def) {
             st = c->stream;
         } else {
@@ -121,13 +126,14 @@ static void give_back_beside(pft_ctx* c, bool all) {
             cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
             cudaThreadExchangeStreamCaptureMode(&mode);
             ok = B.side || cudaStreamCreateWithFlags(&B.side, cudaStreamNonBlocking) == cudaSuccess;
-            if (out.rbegin()->first < B.marked) ok = ok && cudaStreamWaitEvent(B.side, B.mark, 0) == cudaSuccess;
+            if (end <= B.marked) ok = ok && cudaStreamWaitEvent(B.side, B.mark, 0) == cudaSuccess;
             else ok = ok && cudaDeviceSynchronize() == cudaSuccess;  // kept outside any call since the mark
             cudaThreadExchangeStreamCaptureMode(&mode);
             st = B.side;
             if (!ok) {
                 cudaGetLastError();
-                for (auto& b : out) B.stuck.push_back(b.second.p);
+                for (auto& s : out)
+                    for (size_t i = s.second.head; i < s.second.v.size(); i++) B.stuck.push_back(s.second.v[i].p);
             }
         }
     }
@@ -158,18 +164,11 @@ void* dalloc(pft_ctx* c, size_t bytes) {
     BlockCache& B = c->blocks;
     const bool small = bytes <= BlockCache::kMaxBlock && !capturing(c);
     if (small) {
-        // the newest kept block that fits without wasting more than a quarter of it
         std::lock_guard<std::mutex> g(B.mu);
-        const std::pair<size_t, u64>* best = nullptr;
-        for (auto it = B.by_size.lower_bound({bytes, 0}); it != B.by_size.end() && it->first - bytes <= it->first / 4;) {
-            const auto end = B.by_size.upper_bound({it->first, ~0ull});  // of this size
-            const auto newest = std::prev(end);
-            if (!best || newest->second > best->second) best = &*newest;
-            it = end;
-        }
-        if (best) {
-            B.live[B.kept.find(best->second)->second.p] = {best->first, B.id};
-            return B.take(best->second);
+        const auto it = B.fit(bytes);
+        if (it != B.kept.end()) {
+            B.live[it->second.v.back().p] = {it->first, B.id};
+            return B.pop(it, false);
         }
     }
     void* p = raw_alloc(c, bytes);
@@ -211,7 +210,7 @@ void dfree(pft_ctx* c, void* p) {
         void* old = nullptr;
         {
             std::lock_guard<std::mutex> g(B.mu);
-            if (B.over()) old = B.take(B.kept.begin()->first);
+            if (B.over()) old = B.oldest();
         }
         if (!old) return;
         raw_free(c, old, c->stream);
@@ -1995,14 +1994,12 @@ int pft_ctx_create(const pft_params* prm, const pft_allocator* alloc, pft_ctx** 
         PFT_CUDA(cudaStreamGetId(c->stream, &c->blocks.id));
         build_tables(c.get());
         c->noalloc_scratch = noalloc_scratch_lookup();
+        std::lock_guard<std::mutex> g(ctxs_mu());
+        ctxs().insert(c.get());
     });
     if (rc != PFT_OK) {
         for (void* p : c->owned) cudaFree(p);
         return rc;
-    }
-    {
-        std::lock_guard<std::mutex> g(ctxs_mu());
-        ctxs().insert(c.get());
     }
     *out = c.release();
     return PFT_OK;
@@ -2034,14 +2031,15 @@ int pft_ctx_destroy(pft_ctx* c) {
 
 int pft_set_stream(pft_ctx* c, void* stream) {
     if (!c) return PFT_ERR_ARG;
-    unsigned long long id = 0;
-    if (cudaStreamGetId((cudaStream_t)stream, &id) != cudaSuccess) cudaGetLastError();
-    if (c->stream == (cudaStream_t)stream && c->blocks.id == id) return PFT_OK;
-    leave_stream(c);  // kept blocks belong to the old stream
-    std::lock_guard<std::mutex> g(c->blocks.mu);
-    c->stream = (cudaStream_t)stream;
-    c->blocks.id = id;
-    return PFT_OK;
+    return guard(c, [&] {
+        unsigned long long id = 0;
+        if (cudaStreamGetId((cudaStream_t)stream, &id) != cudaSuccess) cudaGetLastError();
+        if (c->stream == (cudaStream_t)stream && c->blocks.id == id) return;
+        leave_stream(c);  // kept blocks belong to the old stream
+        std::lock_guard<std::mutex> g(c->blocks.mu);
+        c->stream = (cudaStream_t)stream;
+        c->blocks.id = id;
+    });
 }
 
 const char* pft_last_error(pft_ctx* c) { return c ? c->err.c_str() : "null context"; }

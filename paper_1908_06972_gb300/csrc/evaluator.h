@@ -4,7 +4,6 @@
 #include <map>
 #include <memory>
 #include <mutex>
-#include <set>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -36,16 +35,34 @@ using namespace pft;
 // size besides: a program that freed thousands of handles pays no walk over them on each allocation.
 struct BlockCache {
     static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)256 << 20, kMaxBlocks = (size_t)1 << 16;
+    static constexpr size_t kMaxSizes = 256;  // stacks, above which the empty ones go
     struct Block {
         void* p;
-        size_t bytes;
+        u64 number;
     };
+    struct Stack {  // kept blocks of one size, oldest first; it stays when it is empty, for the next one
+        std::vector<Block> v;
+        size_t head = 0;  // the first that is left
+        bool empty() const { return head == v.size(); }
+        void* pop(bool oldest) {
+            void* p = oldest ? v[head++].p : v.back().p;
+            if (!oldest) v.pop_back();
+            if (empty()) {
+                v.clear();
+                head = 0;
+            } else if (head > 64 && head > v.size() / 2) {
+                v.erase(v.begin(), v.begin() + head);
+                head = 0;
+            }
+            return p;
+        }
+    };
+    using Sizes = std::map<size_t, Stack>;
     std::mutex mu;
     std::unordered_map<void*, std::pair<size_t, unsigned long long>> live;  // blocks up to kMaxBlock in use: bytes, stream id
-    std::map<u64, Block> kept;                                              // by number: oldest first
-    std::set<std::pair<size_t, u64>> by_size;                               // (bytes, number) of the kept blocks
-    u64 next = 0;                                                           // number of the next kept block
-    size_t kept_bytes = 0;
+    Sizes kept;
+    u64 next = 0;                  // number of the next kept block
+    size_t blocks = 0, bytes = 0;  // of the kept ones
     unsigned long long id = 0;     // of the current stream
     cudaEvent_t mark = nullptr;    // follows the work of the blocks below number `marked`
     u64 marked = 0;
@@ -53,40 +70,52 @@ struct BlockCache {
     std::vector<void*> stuck;      // refused by their free (a stream under capture): freed with the context
 
     // with mu held
-    void keep(void* p, size_t bytes) {
-        const auto it = kept.emplace(next, Block{p, bytes}).first;
-        try {
-            by_size.emplace(bytes, next);
-        } catch (...) {
-            kept.erase(it);
-            throw;
-        }
+    void keep(void* p, size_t size) {
+        if (kept.size() >= kMaxSizes)
+            for (auto it = kept.begin(); it != kept.end();) it = it->second.empty() ? kept.erase(it) : std::next(it);
+        kept[size].v.push_back({p, next});
         next++;
-        kept_bytes += bytes;
+        blocks++;
+        bytes += size;
     }
-    void* take(u64 number) {
-        const auto it = kept.find(number);
-        void* p = it->second.p;
-        by_size.erase({it->second.bytes, number});
-        kept_bytes -= it->second.bytes;
-        kept.erase(it);
-        return p;
+    void* pop(Sizes::iterator it, bool oldest) {
+        blocks--;
+        bytes -= it->first;
+        return it->second.pop(oldest);
     }
-    std::map<u64, Block> take_below(u64 number) {
-        std::map<u64, Block> out;
-        if (number >= next) {
-            out.swap(kept);
-            by_size.clear();
-            kept_bytes = 0;
-        }
-        while (!kept.empty() && kept.begin()->first < number) {
-            const auto b = *kept.begin();
-            out.insert(b);
-            take(b.first);
-        }
+    // the newest block that fits without wasting more than a quarter of it
+    Sizes::iterator fit(size_t size) {
+        auto best = kept.end();
+        for (auto it = kept.lower_bound(size); it != kept.end() && it->first - size <= it->first / 4; ++it)
+            if (!it->second.empty() &&
+                (best == kept.end() || it->second.v.back().number > best->second.v.back().number))
+                best = it;
+        return best;
+    }
+    void* oldest() {
+        auto best = kept.end();
+        for (auto it = kept.begin(); it != kept.end(); ++it)
+            if (!it->second.empty() && (best == kept.end() || it->second.v[it->second.head].number <
+                                                                  best->second.v[best->second.head].number))
+                best = it;
+        return pop(best, true);
+    }
+    Sizes take_all() {
+        Sizes out;
+        out.swap(kept);
+        blocks = bytes = 0;
         return out;
     }
-    bool over() const { return kept_bytes > kMaxCached || kept.size() > kMaxBlocks; }
+    Sizes take_marked() {
+        Sizes out;
+        for (auto it = kept.begin(); it != kept.end(); ++it)
+            while (!it->second.empty() && it->second.v[it->second.head].number < marked) {
+                out[it->first].v.push_back(it->second.v[it->second.head]);
+                pop(it, true);
+            }
+        return out;
+    }
+    bool over() const { return bytes > kMaxCached || blocks > kMaxBlocks; }
 };
 
 // ---- handles ---------------------------------------------------------------------------
