@@ -10,6 +10,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <numeric>
 #include <set>
 #include <stdexcept>
 
@@ -1279,11 +1280,10 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
             for (u64* q : p) dfree(c, q);
         }
     } nb{c, std::vector<u64*>(B, nullptr)};
-    // entries [e0, e1) of `order`; PFT_ERR_OOM is thrown before any work is queued
-    auto part = [&](int e0, int e1) {
+    // PFT_ERR_OOM is thrown before any work is queued
+    auto part = [&](const std::vector<int>& ids) {
         size_t total = 0, most = 0;
-        for (int e = e0; e < e1; e++) {
-            const int i = order[e];
+        for (int i : ids) {
             const size_t w = 2 * (size_t)lv[i] * c->n;
             nb.p[i] = (u64*)dalloc(c, 2 * (size_t)(lv[i] - 1) * c->n * 8);
             total += w;
@@ -1299,13 +1299,13 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
                 room = std::max(most, room / 2);
             }
         }
-        for (int e = e0; e < e1;) {  // all levels together, in tiles of the working space
+        for (size_t e = 0; e < ids.size();) {  // all levels together, in tiles of the working space
             std::vector<PolyRef> in, o;
             std::vector<u64*> last, rb;
             u64* at = S->u();
-            for (; e < e1 && at + 2 * (size_t)lv[order[e]] * c->n <= S->u() + room; e++)
+            for (; e < ids.size() && at + 2 * (size_t)lv[ids[e]] * c->n <= S->u() + room; e++)
                 for (int pol = 0; pol < 2; pol++) {
-                    const int i = order[e];
+                    const int i = ids[e];
                     in.push_back(cpoly(a[i]->data, lv[i], c->n, pol));
                     o.push_back(cpoly(nb.p[i], lv[i] - 1, c->n, pol));
                     last.push_back(at);
@@ -1315,9 +1315,8 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
             rescale_polys(c, in, last, rb, o);
         }
     };
-    auto install = [&](int e0, int e1) {
-        for (int e = e0; e < e1; e++) {
-            const int i = order[e];
+    auto install = [&](const std::vector<int>& ids) {
+        for (int i : ids) {
             pft_ct* o = out[i];
             dfree(c, o->data);  // stream-ordered: queued work on the old buffer completes first
             o->data = nb.p[i];
@@ -1328,8 +1327,11 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
         }
     };
     try {
-        part(0, B);
-        install(0, B);
+        std::vector<int> all(B);
+        std::iota(all.begin(), all.end(), 0);
+        part(all);  // in the caller's order: by level the limbs that are left out (the launches are rectangular) come
+                    // together, 345 against 342 us for 13 at levels 2..30
+        install(order);
         return;
     } catch (const Error& err) {
         if (err.code != PFT_ERR_OOM || B == 0 || lv[order[0]] == lv[order[B - 1]]) throw;
@@ -1344,8 +1346,9 @@ void op_rescale_batch(pft_ctx* c, const pft_ct* const* a, int B, pft_ct* const* 
     }
     for (int e0 = 0, e1 = 0; e0 < B; e0 = e1) {  // no room for the outputs of all levels: level by level
         while (e1 < B && lv[order[e1]] == lv[order[e0]]) e1++;
-        part(e0, e1);
-        install(e0, e1);
+        const std::vector<int> level(order.begin() + e0, order.begin() + e1);
+        part(level);
+        install(level);
     }
 }
 
