@@ -1685,21 +1685,25 @@ static void ft_begin_diag_group(pft_ctx* c, const pft_ft_model* M, const std::ve
     std::vector<int32_t> hsteps;
     for (int k = 1; k < cols; k++) hsteps.push_back(k);
     const size_t rot_per_doc = (size_t)nch * (cols - 1);
+    // the rotated copies [document][chunk][k - 1], in one buffer: a thousand requests to a caller's allocator (32
+    // documents, level 3) are 1.5 ms
+    size_t words = 0;
+    for (FtDoc* d : group) words += rot_per_doc * 2 * d->l * limb;
+    Scratch buf(c, words * 8);
     std::vector<pft_ct> R(group.size() * rot_per_doc);
-    struct CleanR {
-        pft_ctx* c;
-        std::vector<pft_ct>* T;
-        ~CleanR() {
-            for (auto& x : *T) dfree(c, x.data);
-        }
-    } cleanR{c, &R};
     std::vector<const pft_ct*> in;
     std::vector<pft_ct*> outs;
-    for (FtDoc* d : group)
-        for (int i = 0; i < nch; i++) in.push_back(d->v[i]);
-    for (auto& x : R) {  // [document][chunk][k - 1]
-        x.ctx = c;
-        outs.push_back(&x);
+    u64* next = buf.u();
+    for (size_t b = 0; b < group.size(); b++) {
+        for (int i = 0; i < nch; i++) in.push_back(group[b]->v[i]);
+        for (size_t r = 0; r < rot_per_doc; r++) {
+            pft_ct& x = R[b * rot_per_doc + r];
+            x.ctx = c;
+            x.data = next;
+            x.cap = 2 * (size_t)group[b]->l * limb;
+            next += x.cap;
+            outs.push_back(&x);
+        }
     }
     op_rotate_hoisted(c, in.data(), (int)in.size(), hsteps.data(), cols - 1, outs.data());
     size_t at = 0;
