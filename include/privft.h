@@ -386,8 +386,8 @@ int pft_set_transform_plan(pft_ctx* ctx, int plan);
  * is variant 0 there), N <= 2^14 one two-pass form, and rings below 2^12 only the generic one. */
 int pft_set_transform_variant(pft_ctx* ctx, int variant);
 /* Environment switches (measured defaults otherwise), all kernel choices with identical results:
- *   PFT_NTT_ORDER  read at pft_ctx_create; bit 0: the second pass of an N = 2^16 two-pass
- *                  transform visits (polynomial, limb) in reverse, so it starts on the data the
+ *   PFT_NTT_ORDER  read at pft_ctx_create; bit 0: the second pass of a two-pass transform
+ *                  (N >= 2^12) visits (polynomial, limb) in reverse, so it starts on the data the
  *                  first pass wrote last (still in L2); bit 1: the row twiddles are read with an
  *                  L2 evict-last policy; bit 2: the pass that applies ModDown's epilogue asks L2
  *                  for the epilogue's operands at the start of each block (measured slower with

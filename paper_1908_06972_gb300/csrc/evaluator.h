@@ -20,8 +20,8 @@ using namespace pft;
 // Freed device blocks that a context keeps for its next calls.  A call of a small ring allocates and
 // frees about ten short-lived blocks; through a caller's allocator (a callback into Python for
 // torch's) these cost more than its kernels.  Bounded: blocks up to kMaxBlock, kMaxCached bytes in all,
-// the oldest given back first (1 GiB is no faster: within 0.1 % in 32 rotation-light inferences and in every
-// smaller call; 128 MiB 0.4 % slower there).  All are given back when the allocator refuses a request (of this
+// the oldest given back first (128 MiB, 256 MiB and 1 GiB measured the same, within 0.1 % in every call
+// of a millisecond or more).  All are given back when the allocator refuses a request (of this
 // context, or of another one with the same device and allocator), when the context's stream changes and
 // when the context is destroyed.
 // Stream order makes reuse safe as it does for the allocators: a block is kept only if it was allocated

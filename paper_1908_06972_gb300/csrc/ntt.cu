@@ -334,14 +334,13 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, MINB)
 // (inverse) through shared memory to keep the global side coalesced.
 // Bound: the integer multiply pipe for launches of many limbs, the latency of one thread's 16 points
 // for launches of a few.  Against the generic kernels below (one CTA per limb to N = 2^14, staged
-// passes at 2^15; GB300): one HMUL + rescale at N = 2^13, level 3: 188 -> 100 us (its three inverse
-// launches took 58 us each on 1 to 3 SMs), 52 with the later changes; 31 HMULs + rescales at N = 2^15,
-// levels 12..18: 6.15 -> 3.70 ms, 2.85 with the later ones.
+// passes at 2^15; GB300): one HMUL + rescale at N = 2^13, level 3: 188 -> 100 us (three inverse launches
+// of 58 us each on 1 to 3 SMs went); 31 HMULs + rescales at N = 2^15, levels 12..18: 6.15 -> 3.70 ms.
 // Why these shapes: CTAs of 128 threads (8 columns of 2^8 points, 16 of 2^7; 8 rows) meet their loads,
 // exchanges and stores at different times and overlap better than CTAs of 256: 480 limbs, forward and
 // inverse, 660 -> 622 us, and with five of them per SM at 96 registers instead of six at 80 606 us (four at 128:
 // 625).  Launches of more than 512 limbs keep 64 registers (1024 threads) and 16 columns in the forward
-// passes: 32 HMULs with 4 rotations 28.0 ms, 28.2 with five CTAs, 28.5 with 8 columns and 80 registers.
+// passes: 32 HMULs with 4 rotations, levels 5..30, 28.0 ms, 28.2 with five CTAs, 28.5 with 8 columns and 80 registers.
 // The smaller rings meet launches of a few limbs: smaller CTAs still spread a limb over the SMs.
 constexpr int kRowStride = 273;  // 256 + 16 padding + 1
 constexpr u64 kLazyBound = 1ull << 57;  // forward butterflies skip the correction below this prime
@@ -754,9 +753,10 @@ struct TwoPass {
         PFT_LAUNCH_CHECK("intt pass A");
     }
 };
-// A launch with at most this many threads per SM takes the form with everything loaded at the start (its 100
-// to 255 registers leave room for about that many; 256, 512 and 1024 measured within 2 % of each
-// other, none at all 10 % slower for small rings).
+// A launch with at most this many threads on each of the GPU's 152 SMs takes the form with everything loaded
+// at the start.  The line is a measured one (256, 512 and 1024 within 2 % of each other, none at all 10 %
+// slower for small rings): at 100 to 255 registers an SM holds 256 to 640 threads of it, so that at the
+// line's end its widest kernels run in two rounds.
 static constexpr int kPreThreadsPerSm = 512;
 // f(TwoPass<..>) for the ring's shape and the launch's limbs; v: 0 = bounded for 640 resident threads per
 // SM, 1 = for 1024 (N = 2^16 and 2^15; its inverse row pass stays at 640: 1400 against 1480 us in the

@@ -867,9 +867,9 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // registers and twice the resident warps, for 8 digits: 221 us.)
 // Bound: HBM and the multiply pipe together from 3 digits on (177 us for 4 ciphertexts at level 30,
 // 5.6 TB/s; 195 us with one 64-bit Montgomery reduction), the latency of a stage below.  64 inputs of one
-// digit (level 3): 265 us with one input per stage, 194 us with four, 161 with the two-step reduction.  9 digits at N = 2^15 (31 inputs, levels 12..18) ran in the generic kernel
-// before, which reads the key again for every input: that HMUL + rescale batch 3.70 -> 3.56 ms; the sum
-// itself 457 us in the form for 12 digits, 350 in the one for 10 with straight code per digit count.
+// digit (level 3): 161 us; with one input per stage instead of four the same took 265 instead of 194 before
+// the two-step reduction.  9 digits at N = 2^15 (31 inputs, levels 12..18): 350 us in the form for 10, 457 in
+// the one for 12; the generic kernel reads the key again for every input.
 // The key slice is loaded before the ring is started: after it (copies in flight first) measured
 // slower for few inputs, 95 against 87 us for one at level 30.
 // PERM (hoisted rotations): several keys over the same inputs, key z (grid y) with Galois element
@@ -878,8 +878,8 @@ __global__ void __launch_bounds__(128) k_ks_inner_multi(DevTables t, KsBatch bt,
 // permuted: no permuted copy of the extended digits is made (it was beta (l + k) limbs written and
 // read per rotation).  The keys of one row run together, so that the row's digits (18 MB for 8 inputs
 // of 9 digits at N = 2^15) come from HBM once for all of them.  With the batching of op_rotate_hoisted
-// over inputs and steps, 32 rotation-light inferences at level 3: 132 -> 48 ms (40.7 with the later
-// changes); 4 at N = 2^15, levels 12..18: 80 -> 22 ms (18.2).
+// over inputs and steps, 32 rotation-light inferences at level 3: 132 -> 48 ms; 4 at N = 2^15, levels
+// 12..18: 80 -> 22 ms.
 constexpr int kKsStages = 3;
 constexpr int kKsChunk = 256;                // coefficients per CTA (2 KiB per digit row)
 constexpr long long kWaitPolls = 1ll << 22;  // polls of a bounded wait (seconds at most)
