@@ -35,7 +35,7 @@ using namespace pft;
 // size besides: a program that freed thousands of handles pays no walk over them on each allocation.
 struct BlockCache {
     static constexpr size_t kMaxBlock = (size_t)16 << 20, kMaxCached = (size_t)256 << 20, kMaxBlocks = (size_t)1 << 16;
-    static constexpr size_t kMaxSizes = 256;  // stacks, above which the empty ones go
+    static constexpr size_t kMaxSizes = 1024;  // different sizes: bounds the walks below
     struct Block {
         void* p;
         u64 number;
@@ -71,7 +71,7 @@ struct BlockCache {
 
     // with mu held
     void keep(void* p, size_t size) {
-        if (kept.size() >= kMaxSizes)
+        if (kept.size() >= kMaxSizes)  // the empty stacks go
             for (auto it = kept.begin(); it != kept.end();) it = it->second.empty() ? kept.erase(it) : std::next(it);
         kept[size].v.push_back({p, next});
         next++;
@@ -98,7 +98,9 @@ struct BlockCache {
             if (!it->second.empty() && (best == kept.end() || it->second.v[it->second.head].number <
                                                                   best->second.v[best->second.head].number))
                 best = it;
-        return pop(best, true);
+        void* p = pop(best, true);
+        if (best->second.empty()) kept.erase(best);
+        return p;
     }
     Sizes take_all() {
         Sizes out;
@@ -115,7 +117,7 @@ struct BlockCache {
             }
         return out;
     }
-    bool over() const { return bytes > kMaxCached || blocks > kMaxBlocks; }
+    bool over() const { return bytes > kMaxCached || blocks > kMaxBlocks || kept.size() > kMaxSizes; }
 };
 
 // ---- handles ---------------------------------------------------------------------------

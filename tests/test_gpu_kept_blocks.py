@@ -230,3 +230,30 @@ def test_what_a_context_keeps_is_small(gpu):
     assert alloc.in_use() <= base + (256 << 20)
     pf.pft_ctx_destroy(ctx)
     assert alloc.in_use() == 0
+
+
+def test_many_sizes(gpu):
+    """More different sizes than a context keeps blocks of (one handle's words each): results, and everything given back."""
+    from .test_gpu_faults import CappedAllocator
+
+    pf, alloc, n = gpu, CappedAllocator(gpu, torch), 1300
+    ctx = pf.pft_ctx_create(4, 1, 1, 1, 60, 40, 60, 2.0 ** 40, SEED, flags=pf.PFT_ALLOW_INSECURE, allocator=alloc.struct)
+    q = pf.pft_ctx_info(ctx)["primes"][0]
+    w = torch.arange(n * 16, dtype=torch.int64, device="cuda")
+    a = [pf.pft_ct_create(ctx) for _ in range(n)]
+    v = torch.cat([w, w]).contiguous()
+    for h in a:
+        pf.pft_ct_reduce_sum(ctx, v.data_ptr(), 1, 2.0 ** 40, 1, h)
+    pt = pf.pft_pt_import(ctx, np.eye(1, 16, dtype=np.uint64), 1.0)  # the constant 1
+    out = pf.pft_ct_create(ctx)
+    for k in list(range(1, n + 1)) * 2:  # pointer tables of k and 2 k words
+        pf.pft_dot_plain_batch(ctx, a[:k], [pt] * k, k, [out], pts_shared=True)
+    got = torch.empty((2, 1, 16), dtype=torch.int64, device="cuda")
+    pf.pft_ct_copy_out(ctx, out, got.data_ptr())
+    want = v[:32].cpu().numpy().astype(object) * n % q
+    assert np.array_equal(got.cpu().numpy().reshape(-1).astype(object), want)
+    for h in a + [out]:
+        pf.pft_ct_destroy(h)
+    pf.pft_pt_destroy(pt)
+    pf.pft_ctx_destroy(ctx)
+    assert alloc.in_use() == 0
